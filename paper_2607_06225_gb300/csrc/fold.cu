@@ -1,7 +1,12 @@
 // fold.cu -- Nussinov RNA folding (Table 1) with X-drop transferred to it
-// (Sec. 9.5): the kernel and the filtr_fold_batch entry point.
+// (Sec. 9.5): the filtr_fold_batch entry point, and the plain kernel.
 //
-// One CTA per sequence.  The triangle 0 <= i <= j < n is swept along the span
+// Folds run in k_fold_tiled (k_fold_tiled.cuh).  Its 16-bit matrix takes about
+// the bytes of the plain kernel's 32-bit triangle plus a few per row, so a
+// sequence whose triangle only just fits the workspace runs in the plain
+// kernel below instead.
+//
+// Plain kernel: one CTA per sequence.  The triangle 0 <= i <= j < n is swept along the span
 // k = j - i: the cells of one span depend only on shorter spans, so the CTA's
 // threads take a span's positions i in parallel and a barrier separates spans.
 // The table lives in global memory span-major (row k holds F(i, i+k) for
@@ -23,6 +28,19 @@
 namespace filtr {
 namespace {
 
+__device__ __forceinline__ bool rna_pair(int a, int b) {
+  const int s = a + b;  // A=0 C=1 G=2 U=3: A-U and C-G sum to 3, G-U to 5
+  return s == 3 || (s == 5 && a != b);
+}
+
+}  // namespace
+}  // namespace filtr
+
+#include "k_fold_tiled.cuh"
+
+namespace filtr {
+namespace {
+
 constexpr int FOLD_THREADS = 256;
 
 struct FoldArgs {
@@ -35,13 +53,7 @@ struct FoldArgs {
   filtr_fold_result *out;
   int32_t *partner;            // nullptr without traceback
   int min_loop, use_xdrop, xdrop, warmup;
-  int max_group;               // largest thread group per cell (1 or 32)
 };
-
-__device__ __forceinline__ bool rna_pair(int a, int b) {
-  const int s = a + b;  // A=0 C=1 G=2 U=3: A-U and C-G sum to 3, G-U to 5
-  return s == 3 || (s == 5 && a != b);
-}
 
 // first word of span k's row in a table of n positions
 __device__ __forceinline__ int64_t row_off(int k, int n) {
@@ -75,49 +87,24 @@ __global__ void __launch_bounds__(FOLD_THREADS) k_fold(const FoldArgs a) {
     const int32_t *r2 = k >= 2 ? D + row_off(k - 2, n) : nullptr;
     int32_t *rk = D + row_off(k, n);
     int tmax = INT_MIN, tlo = INT_MAX, thi = INT_MIN;
-    // a group of G threads per cell (G = 1..32, a power of two, as many as the
-    // span's domain leaves room for): the group splits the cell's split terms
-    // and reduces them with shuffles, so the long, narrow spans near the top of
-    // the triangle keep the CTA busy.  The group's lanes read different rows, so
-    // this pays only while the resident tables stay in L2 (short sequences)
-    int G = 1;
-    while (G < a.max_group && 2 * G * (dh - dl + 1) <= FOLD_THREADS) G *= 2;
-    const int per_pass = FOLD_THREADS / G, sub = tid & (G - 1), slot = tid / G;
-    for (int i0 = 0; i0 <= n - 1 - k; i0 += per_pass) {  // uniform trip count
-      const int i = i0 + slot;
-      const bool in_dom = i >= dl && i <= dh;
+    for (int i = tid; i <= n - 1 - k; i += FOLD_THREADS) {
       int f = NEG;
-      if (in_dom) {
+      if (i >= dl && i <= dh) {
         const int j = i + k;
-        if (sub == 0) {
-          f = max(r1[i + 1], r1[i]);  // i unpaired, j unpaired
-          if (rna_pair(sx[i], sx[j]) && k - 1 >= a.min_loop) {
-            const int inner = k >= 2 ? r2[i + 1] : 0;  // an empty interval is 0
-            f = max(f, inner + 1);
-          }
+        f = max(r1[i + 1], r1[i]);  // i unpaired, j unpaired
+        if (rna_pair(sx[i], sx[j]) && k - 1 >= a.min_loop) {
+          const int inner = k >= 2 ? r2[i + 1] : 0;  // an empty interval is 0
+          f = max(f, inner + 1);
         }
         // F(i, i+t) + F(i+t+1, j): o1 -> F(i, i+t) in row t, o2 -> F(i+t+1, j)
         // in row k-1-t, both stepped by whole rows (row t holds n - t cells)
-        if (G == 1) {
-          int o1 = i, o2 = roff[k - 1] + i + 1;
+        int o1 = i, o2 = roff[k - 1] + i + 1;
 #pragma unroll 4
-          for (int t = 0; t < k; ++t) {
-            f = max(f, D[o1] + D[o2]);
-            o1 += n - t;
-            o2 -= n - k + 1 + t;
-          }
-        } else if (sub < k) {  // t = sub, sub + G, ...: row_off(a + G) - row_off(a) = G n - G a - G(G-1)/2
-          const int gg = G * (G - 1) / 2;
-          int o1 = roff[sub] + i, o2 = roff[k - 1 - sub] + i + sub + 1;
-          for (int t = sub; t < k; t += G) {
-            f = max(f, D[o1] + D[o2]);
-            o1 += G * n - G * t - gg;
-            o2 -= G * n - G * (k - 1 - t - G) - gg - G;
-          }
+        for (int t = 0; t < k; ++t) {
+          f = max(f, D[o1] + D[o2]);
+          o1 += n - t;
+          o2 -= n - k + 1 + t;
         }
-      }
-      for (int o = G >> 1; o; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
-      if (in_dom) {
         const bool alive = f > NEG_HALF && (!a.use_xdrop || k <= a.warmup || f >= best - a.xdrop);
         if (!alive) f = NEG;
         if (alive) {
@@ -126,7 +113,7 @@ __global__ void __launch_bounds__(FOLD_THREADS) k_fold(const FoldArgs a) {
           thi = max(thi, i);
         }
       }
-      if (sub == 0 && i <= n - 1 - k) rk[i] = f;
+      rk[i] = f;
     }
     tmax = __reduce_max_sync(0xffffffffu, tmax);
     tlo = __reduce_min_sync(0xffffffffu, tlo);
@@ -230,6 +217,48 @@ __global__ void __launch_bounds__(FOLD_THREADS) k_fold(const FoldArgs a) {
   }
 }
 
+// Launch classes of the tiled kernel, by length: the instance's span tables are
+// laid out for the longest sequence of its class (90 bytes per base), so a class
+// fixes how many blocks share an SM.  Up to 320 bases four warps per fold (more
+// folds per SM hide the barrier after each span), above that eight, and sixteen
+// over 512 bases when the launch leaves SMs idle.  Three staging buffers, but two
+// for the 512-base class, where the third would cost the third block of the SM
+// (1024 folds of 500 bases: 4.59 against 4.74 ms).  Over 1200 bases the span
+// tables no longer fit shared memory beside the staging and live in the
+// sequence's area.
+// Measured against the plain kernel, whole calls: 1024 folds of 300 bases 8.92 ->
+// 1.35 ms, 1024 of 500 bases with X = 2 34.0 -> 4.6 ms.  What bounds it now: the
+// bulk phase waits for its chunks and barriers (one block alone on an SM takes
+// 0.94 ms for 500 bases, three share it in 1.46 ms).
+constexpr int FOLD_PLAIN = 5;  // not a tiled class: the plain kernel
+inline int fold_class(int n) { return n <= 160 ? 0 : n <= 320 ? 1 : n <= 512 ? 2 : n <= 1200 ? 3 : 4; }
+inline uint64_t fold_area_bytes(int n) {
+  return fold_q_bytes(n) + (fold_class(n) == 4 ? fold_span_bytes(FILTR_FOLD_MAX_LEN) : 0);
+}
+
+template <int NW, int ST, int MAXN, bool GS, int MINB>
+cudaError_t fold_launch(const FoldTiledArgs &a, uint32_t count, cudaStream_t st) {
+  constexpr size_t smem = fold_smem_bytes(NW, ST, MAXN, GS);
+  static_assert(smem * MINB <= 224 * 1024, "shared memory of the blocks of one SM");
+  auto k = k_fold_tiled<NW, ST, MAXN, GS, MINB>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k<<<count, NW * 32, smem, st>>>(a);
+  return cudaGetLastError();
+}
+cudaError_t launch_fold_tiled(const FoldTiledArgs &a, uint32_t count, int cls, int sms, cudaStream_t st) {
+  const bool few = count <= (uint32_t)sms;
+  switch (cls) {
+    case 0: return fold_launch<4, 3, 160, false, 6>(a, count, st);
+    case 1: return fold_launch<4, 3, 320, false, 4>(a, count, st);
+    case 2: return fold_launch<8, 2, 512, false, 3>(a, count, st);
+    case 3: return few ? fold_launch<16, 3, 1200, false, 1>(a, count, st)
+                       : fold_launch<8, 3, 1200, false, 1>(a, count, st);
+    default: return few ? fold_launch<16, 3, FILTR_FOLD_MAX_LEN, true, 1>(a, count, st)
+                        : fold_launch<8, 3, FILTR_FOLD_MAX_LEN, true, 3>(a, count, st);
+  }
+}
+
 struct Carve {
   char *base;
   size_t cap, used = 0;
@@ -290,47 +319,60 @@ static filtr_status fold_impl(Ctx *ctx, const filtr_fold_params *prm, uint32_t n
     set_error("%u codes are 4 or more (RNA codes A=0 C=1 G=2 U=3)", *h_bad);
     return FILTR_ERR_INVALID;
   }
-  std::vector<uint64_t> words(n);
-  std::vector<uint32_t> h_len_copy(h_len, h_len + n);  // h_stage is reused below
-  for (uint32_t p = 0; p < n; ++p) {
-    if (h_len[p] > FILTR_FOLD_MAX_LEN) {
-      set_error("sequence %u has %u bases; the limit is %u", p, h_len[p], FILTR_FOLD_MAX_LEN);
+  std::vector<uint32_t> lens(h_len, h_len + n);  // h_stage is reused below
+  for (uint32_t p = 0; p < n; ++p)
+    if (lens[p] > FILTR_FOLD_MAX_LEN) {
+      set_error("sequence %u has %u bases; the limit is %u", p, lens[p], FILTR_FOLD_MAX_LEN);
       return FILTR_ERR_UNSUPPORTED;
     }
-    words[p] = (uint64_t)h_len[p] * (h_len[p] + 1) / 2;
-  }
   // workspace: order, table offsets, then the tables in waves
   Carve c{ctx->ws, ctx->ws_bytes};
   uint32_t *d_order = c.take<uint32_t>(n);
   uint64_t *d_toff = c.take<uint64_t>(n);
   const size_t tbase = (c.used + 255) / 256 * 256;
-  const uint64_t twords = ctx->ws_bytes > tbase ? (ctx->ws_bytes - tbase) / 4 : 0;
+  const uint64_t troom = ctx->ws_bytes > tbase ? (ctx->ws_bytes - tbase) / 16 : 0;  // 16-byte units
   if (!ctx->ensure_host((size_t)n * 12 + 256)) {
     set_error("pinned host allocation failed");
     return FILTR_ERR_NOMEM;
   }
   uint64_t *h_toff = reinterpret_cast<uint64_t *>(ctx->h_stage);
   uint32_t *h_ord = reinterpret_cast<uint32_t *>(h_toff + n);
-  std::vector<std::pair<uint32_t, uint32_t>> waves;
-  uint64_t used = 0;
-  uint32_t begin = 0;
+  // launches of like lengths, longest first: a launch's shared memory is sized
+  // by its class
+  struct Launch {
+    uint32_t begin, end;
+    int cls;
+    bool new_wave;
+  };
+  std::vector<uint32_t> ord(n);
+  std::vector<int> cls(n);
   for (uint32_t p = 0; p < n; ++p) {
-    const uint64_t w = (words[p] + 3) / 4 * 4;
-    if (w > twords) {
-      set_error("sequence %u needs %llu table words; the workspace holds %llu", p,
-                (unsigned long long)w, (unsigned long long)twords);
+    ord[p] = p;
+    const uint64_t units = fold_area_bytes((int)lens[p]) / 16;
+    const uint64_t plain = ((uint64_t)lens[p] * (lens[p] + 1) / 2 + 3) / 4;
+    if (units > troom && plain > troom) {
+      set_error("sequence %u needs %llu table bytes; the workspace holds %llu", p,
+                (unsigned long long)plain * 16, (unsigned long long)troom * 16);
       return FILTR_ERR_NOMEM;
     }
-    if (used + w > twords) {
-      waves.push_back({begin, p});
-      begin = p;
-      used = 0;
-    }
-    h_toff[p] = used;
-    h_ord[p] = p;
+    cls[p] = units > troom ? FOLD_PLAIN : fold_class((int)lens[p]);
+  }
+  std::stable_sort(ord.begin(), ord.end(), [&](uint32_t x, uint32_t y) { return lens[x] > lens[y]; });
+  std::vector<Launch> runs;
+  uint64_t used = 0;
+  for (uint32_t t = 0; t < n; ++t) {
+    const uint32_t p = ord[t];
+    const uint64_t w = cls[p] == FOLD_PLAIN ? ((uint64_t)lens[p] * (lens[p] + 1) / 2 + 3) / 4
+                                   : fold_area_bytes((int)lens[p]) / 16;
+    const bool wave = used + w > troom;
+    if (wave) used = 0;
+    if (runs.empty() || wave || runs.back().cls != cls[p])
+      runs.push_back({t, t, cls[p], wave});
+    runs.back().end = t + 1;
+    h_toff[p] = cls[p] == FOLD_PLAIN ? used * 4 : used;  // the plain kernel counts words
+    h_ord[t] = p;
     used += w;
   }
-  waves.push_back({begin, n});
   ce = cudaMemcpyAsync(d_toff, h_toff, (size_t)n * 8, cudaMemcpyHostToDevice, st);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_order, h_ord, (size_t)n * 4, cudaMemcpyHostToDevice, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "uploading the table layout");
@@ -346,24 +388,36 @@ static filtr_status fold_impl(Ctx *ctx, const filtr_fold_params *prm, uint32_t n
   a.use_xdrop = prm->use_xdrop ? 1 : 0;
   a.xdrop = prm->xdrop;
   a.warmup = prm->warmup;
-  // thread groups per cell for short sequences only: measured on 1024-2048
-  // structured RNAs, grouping took 76 bases 1.14 -> 0.62 ms, 120 bases 2.67 ->
-  // 1.54 ms and 300 bases 13.6 -> 11.7 ms, but 500 bases 61 -> 77 ms, whose
-  // tables (0.5 MB each) no longer stay in L2 once the group's loads scatter
-  uint32_t max_len = 0;
-  for (uint32_t p = 0; p < n; ++p) max_len = std::max(max_len, h_len_copy[p]);
-  a.max_group = max_len <= 320 ? 32 : 1;
+  FoldTiledArgs ta{};
+  ta.seq = seq;
+  ta.off = off;
+  ta.len = len;
+  ta.area_off = d_toff;
+  ta.area = ctx->ws + tbase;
+  ta.out = out;
+  ta.partner = a.partner;
+  ta.min_loop = a.min_loop;
+  ta.use_xdrop = a.use_xdrop;
+  ta.xdrop = a.xdrop;
+  ta.warmup = a.warmup;
   ctx->span_begin(Ctx::PH_FORWARD, st);
-  for (const auto &w : waves) {
-    a.order = d_order + w.first;
-    k_fold<<<w.second - w.first, FOLD_THREADS, 0, st>>>(a);
+  uint32_t n_waves = 1;
+  for (const Launch &w : runs) {
+    n_waves += w.new_wave ? 1 : 0;
+    if (w.cls == FOLD_PLAIN) {
+      a.order = d_order + w.begin;
+      k_fold<<<w.end - w.begin, FOLD_THREADS, 0, st>>>(a);
+      ce = cudaGetLastError();
+    } else {
+      ta.order = d_order + w.begin;
+      ce = launch_fold_tiled(ta, w.end - w.begin, w.cls, ctx->sms, st);
+    }
     ++launches;
-    ce = cudaGetLastError();
     if (ce != cudaSuccess) break;
   }
   ctx->span_end(st);
   if (ce != cudaSuccess) return cuda_fail(ce, "fold kernel");
-  ctx->last_waves = (int)waves.size();
+  ctx->last_waves = (int)n_waves;
   ctx->last_launches = launches;
   ctx->last_cells_estimate = 0;
   ctx->last_cells_packed = 0;

@@ -110,3 +110,52 @@ def test_table_waves(F):
     assert np.array_equal(res["score"].astype(np.int64), ores["score"])
     assert np.array_equal(res["cells"].astype(np.int64), ores["cells"])
     assert np.array_equal(part, opart[: len(seq)])
+
+
+@pytest.mark.parametrize("xdrop", [None, 1, 6])
+def test_tile_edges(F, ctx, xdrop):
+    """Lengths around the tiled kernel's edges: groups of 21 spans from length 2,
+    blocks of 16 positions, rows of 8 halfwords, and the launch classes (160, 320,
+    512 and 1200 bases), with one or many sequences of a class in the launch."""
+    rng = np.random.default_rng(75)
+    lens = np.array([1, 2, 3, 15, 16, 17, 21, 22, 23, 24, 31, 32, 33, 43, 44, 45, 64, 65, 66, 85, 86, 87,
+                     127, 128, 129, 159, 160, 161, 255, 256, 320, 321, 512, 513, 1199, 1200, 1201, 1237],
+                    np.uint32)
+    off = np.zeros(len(lens), np.uint64)
+    off[1:] = np.cumsum(lens[:-1].astype(np.uint64))
+    seq = rng.integers(0, 4, size=int(lens.sum())).astype(np.uint8)
+    kw = {} if xdrop is None else dict(xdrop=xdrop, warmup=20)
+    check(F, ctx, seq, off, lens, str(kw), **kw)
+
+
+def test_many_long(F, ctx):
+    """More sequences of 650 bases than SMs: the eight-warp form of that class."""
+    seq, off, lens = synth.rna_structured(160, 650, seed=76)
+    res, part, rc = F.fold_batch(ctx, F.make_fold_params(xdrop=4), seq, off, lens)
+    assert rc == 0, F.last_error()
+    k = 3
+    ores, opart = oracle.fold_batch(seq[: 650 * k], off[:k], lens[:k], xdrop=4)
+    assert np.array_equal(res["score"][:k].astype(np.int64), ores["score"])
+    assert np.array_equal(res["cells"][:k].astype(np.int64), ores["cells"])
+    assert np.array_equal(part[: 650 * k], opart[: 650 * k])
+    one, ppart, rc = F.fold_batch(ctx, F.make_fold_params(xdrop=4), seq[650 * 100: 650 * 160],
+                                  off[:60], lens[:60])  # 60 sequences: sixteen warps
+    assert rc == 0 and np.array_equal(one["score"], res["score"][100:])
+    assert np.array_equal(ppart, part[650 * 100:])
+
+
+def test_plain_kernel(F):
+    """A workspace that holds the 32-bit triangle of 700 bases but not the tiled
+    kernel's matrix: the plain kernel folds the sequence."""
+    n = 700
+    seq, off, lens = synth.rna_structured(1, n, seed=77)
+    triangle, matrix = n * (n + 1) // 2 * 4, (n + 1) * ((n + 8) // 8 * 8) * 2
+    room = 512 + (triangle + matrix) // 2
+    assert triangle + 512 < room < matrix
+    for X in (None, 3):
+        small = F.Context(0, room)
+        try:
+            kw = {} if X is None else dict(xdrop=X)
+            check(F, small, seq, off, lens, f"plain X={X}", **kw)
+        finally:
+            small.close()

@@ -49,6 +49,11 @@ filtr_status filtr_test_set_device_plan(filtr_ctx *ctx, int32_t mode);
  * depend on it; it trades shared memory (occupancy) against load latency. */
 filtr_status filtr_test_set_search_ring(filtr_ctx *ctx, int32_t entries);
 
+/* Tiled batches a warp per row strip (intra-pair) instead of a warp per pair:
+ * 0 by batch size (the default), 1 never, 2 whenever the pairs have several
+ * strips and the workspace allows.  Results do not depend on it. */
+filtr_status filtr_test_set_split(filtr_ctx *ctx, int32_t mode);
+
 /* Cell width of the antidiagonal (X-drop / Z-drop) sweep: 0 the default (two
  * cells per register for affine pairs whose threshold leaves room, int32
  * otherwise), 1 int32 always, 2 two cells per register with the base score

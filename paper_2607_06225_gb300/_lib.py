@@ -178,6 +178,8 @@ def lib():
         L.filtr_test_set_first_width.argtypes = [C.c_void_p, C.c_int32]
         L.filtr_test_set_device_plan.restype = i32
         L.filtr_test_set_device_plan.argtypes = [C.c_void_p, C.c_int32]
+        L.filtr_test_set_split.restype = i32
+        L.filtr_test_set_split.argtypes = [C.c_void_p, C.c_int32]
         L.filtr_test_set_search_ring.restype = i32
         L.filtr_test_set_search_ring.argtypes = [C.c_void_p, C.c_int32]
         L.filtr_test_set_packed_sweep.restype = i32

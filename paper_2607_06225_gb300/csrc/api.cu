@@ -13,6 +13,7 @@
 
 #include "../../include/filtr_testing.h"
 #include "filtr_ctx.h"
+#include "k_split.cuh"
 #include "k_xdrop_layout.h"
 #include "plan.h"
 
@@ -178,6 +179,16 @@ int Ctx::graph_blocks_per_sm(int R, bool packed, const ScoreParams &sp) {
   return nb;
 }
 
+int Ctx::split_blocks_per_sm(bool packed, int R, const ScoreParams &sp) {
+  const auto key = std::make_tuple(R | (packed ? 0x500 : 0x400), sp.mode, sp.affine, sp.traceback,
+                                   sp.use_band, sp.alphabet);
+  auto it = occ_cache.find(key);
+  if (it != occ_cache.end()) return it->second;
+  const int nb = std::max(1, packed ? split_pack_blocks_per_sm(R, sp) : split_full_blocks_per_sm(sp));
+  occ_cache[key] = nb;
+  return nb;
+}
+
 cudaEvent_t Ctx::next_event() {
   if (ev_used == ev_pool.size()) {
     cudaEvent_t e = nullptr;
@@ -308,6 +319,13 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     return FILTR_ERR_NOMEM;
   }
   const ShapeCost *costs = ctx->tuned_costs(sp);
+  // Few pairs: a warp per strip instead of per pair (k_split.cuh), unless a tune
+  // table says which warp-per-pair shapes to use
+  int split = SPLIT_NONE;
+  const bool may_split = !plain && !sp.use_xdrop && !costs && ctx->split_mode != 1 &&
+                         (ctx->split_mode == 2 || n <= (sp.use_band ? SPLIT_MAX_BANDED : SPLIT_MAX_PAIRS));
+  if (may_split && (ctx->split_mode == 2 || sp.use_band || n <= SPLIT_LATENCY_PAIRS))
+    split = n <= SPLIT_LATENCY_PAIRS ? SPLIT_PACK8 : SPLIT_PACK8_16;
   if (!costs) costs = kDefaultShapeCost;
 
   // 2. residue validation, the device plan, and the lengths or the plan's
@@ -342,7 +360,7 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     pa.r_len = b.r_len;
     pa.n = n;
     pa.sp = sp;
-    pa.tab = make_shape_table(costs, sp);
+    pa.tab = make_shape_table(costs, sp, split);
     pa.state = d_ps;
     pa.key = d_pkey;
     pa.words = d_pwords;
@@ -439,15 +457,43 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     return FILTR_ERR_NOMEM;
   }
   const uint64_t tb_budget = (ctx->ws_bytes - c.used) / 4;
+  // The split launches' queues and hand-over slots sit between the staging and
+  // the traceback.  They are laid out once the plan's groups are known; a plan
+  // whose traceback and slots do not fit together (or whose slots would take a
+  // quarter of the workspace) is made again without splitting, so a split batch
+  // never needs workspace that a plain one did not.
+  const uint32_t split_stride = (uint32_t)max_n + 1;
+  SplitSpace split_spc[SHAPE_TILED];
+  auto split_fits = [&](const std::vector<Group> &groups, uint64_t tb_words, uint64_t *words) -> bool {
+    if (sp.traceback) {  // a pair the plain shapes may refuse for its traceback: they decide
+      ScoreParams full = sp;
+      full.use_band = 0;
+      const ShapeTable plain_tab = make_shape_table(costs, sp);
+      for (int i = 0; i < plain_tab.n_elig; ++i)
+        if (shape_tb_words(plain_tab, plain_tab.elig[i], (uint32_t)max_m, (uint32_t)max_n, full) > tb_budget)
+          return false;
+    }
+    size_t bytes = 0;
+    for (size_t g = 0; g < groups.size(); ++g) {
+      const uint64_t rows = split_rows(groups[g].family == FAM_PACK, groups[g].R);
+      const uint64_t ns = (max_m + rows - 1) / rows;
+      if (ns > SPLIT_MAX_STRIPS || g >= SHAPE_TILED) return false;
+      split_spc[g] = split_space(groups[g].end - groups[g].begin, ns, split_stride);
+      bytes += split_spc[g].bytes;
+    }
+    *words = (bytes + 3) / 4;
+    return bytes <= ctx->ws_bytes / 4 && tb_words + *words + 64 <= tb_budget;
+  };
+  uint64_t split_words = 0;
+  // one strip each: nothing to split (and 8 rows per lane is the shape of such pairs anyway)
+  const bool one_strip = max_m <= (uint64_t)split_rows(false, 8);
 
   // 4. the plan: the device's when its traceback fits one wave, else the host's
   Plan &P = ctx->plan;
   uint32_t n_main = 0, n_trivial = 0;
-  if (dev_plan && (!sp.traceback || dsum.tb_words <= tb_budget)) {
-    P.waves.clear();
-    P.trivial.clear();
-    Wave w;
-    w.tb_words = dsum.tb_words;
+  Wave w;
+  w.tb_words = dsum.tb_words;
+  if (dev_plan) {
     uint32_t at = 0;
     for (int k = 0; k < SHAPE_TILED; ++k) {
       if (!dsum.count[k]) continue;
@@ -462,6 +508,18 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
       w.groups.push_back(g);
     }
     n_main = at;
+  }
+  const bool dev_split = dev_plan && split != SPLIT_NONE && !one_strip;
+  // unbanded pairs planned a warp each, one of which would outlast the others:
+  // planned again on the host, a warp per strip
+  const bool tall = dev_plan && may_split && split == SPLIT_NONE && max_m > SPLIT_TALL_ROWS &&
+                    (double)max_m * (double)max_n > 2.0 * (double)dsum.cells / (10.0 * ctx->sms);
+  if (tall) split = SPLIT_PACK8_16;
+  if (dev_plan && !tall && (!sp.traceback || dsum.tb_words <= tb_budget) &&
+      (!dev_split || split_fits(w.groups, sp.traceback ? dsum.tb_words : 0, &split_words))) {
+    P.waves.clear();
+    P.trivial.clear();
+    if (!dev_split) split = SPLIT_NONE;
     n_trivial = dsum.count[KEY_TRIVIAL];
     w.walk_begin = 0;
     w.walk_end = n_main;
@@ -491,7 +549,15 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     const int w0 = ctx->xdrop_warps0 > 0 ? ctx->xdrop_warps0 : (swc ? swc->warps : 0);
     PlanInput in{&sp, n, ctx->h_ql.data(), ctx->h_rl.data(), tb_budget, 8, w0};
     in.shape_cost = costs;
-    if (!make_plan(in, &P)) return FILTR_ERR_NOMEM;
+    in.split = dev_split || one_strip ? SPLIT_NONE : split;  // a device plan has tried splitting
+    bool planned = false;
+    if (in.split != SPLIT_NONE) {
+      planned = make_plan(in, &P) && P.waves.size() == 1 &&
+                split_fits(P.waves[0].groups, sp.traceback ? P.waves[0].tb_words : 0, &split_words);
+      if (!planned) in.split = SPLIT_NONE;
+    }
+    split = in.split;
+    if (!planned && !make_plan(in, &P)) return FILTR_ERR_NOMEM;
     n_main = (uint32_t)P.order.size();
     n_trivial = (uint32_t)P.trivial.size();
     const size_t up_bytes = n * (4 + sizeof(TbLayout) + 8) + 64;
@@ -515,6 +581,14 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   ctx->last_dev_plan = dev_plan;
   const std::vector<uint32_t> &ql = ctx->h_ql, &rl = ctx->h_rl;
   ctx->last_host_plan_ms = ms_since(t_plan);
+
+  char *d_split = reinterpret_cast<char *>(d_tb);
+  if (split != SPLIT_NONE) {
+    d_tb += (split_words + 63) / 64 * 64;
+    // the groups of a split batch run at the same time, each on its own side stream
+    n_conc = P.waves.empty() ? 0 : (int)P.waves[0].groups.size();
+    if (n_conc < 2 || !ctx->ensure_side(n_conc)) n_conc = 0;
+  }
 
   FullArgs fa;
   fa.b = b;
@@ -607,6 +681,27 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     ++launches;
     return ce == cudaSuccess;
   };
+  // group gi of a split batch: a warp per strip
+  auto run_split = [&](const Group &g, int gi, cudaStream_t gs) -> bool {
+    SplitLaunch sl{};
+    sl.packed = g.family == FAM_PACK;
+    sl.R = g.R;
+    sl.count = g.end - g.begin;
+    const uint64_t rows = split_rows(sl.packed, g.R);
+    sl.max_strips = (uint32_t)((max_m + rows - 1) / rows);
+    const int64_t items = sl.count * (int64_t)sl.max_strips;
+    sl.grid = (int)std::min<int64_t>((int64_t)ctx->sms * ctx->split_blocks_per_sm(sl.packed, g.R, sp),
+                                     (items + FULL_WARPS - 1) / FULL_WARPS);
+    sl.a.f = fa;
+    sl.a.f.order = d_order + g.begin;
+    sl.a.timeout_ns = SPLIT_TIMEOUT_NS;
+    size_t at = 0;
+    for (int x = 0; x < gi; ++x) at += split_spc[x].bytes;
+    split_bind(&sl.a, d_split + at, split_spc[gi], split_stride);
+    ce = launch_split(sl, gs);
+    launches += 3;
+    return ce == cudaSuccess;
+  };
   // pairs that outgrew their window (list) and, from the packed sweep, pairs
   // that left its 16-bit range (list16); both counters come back in one copy
   auto read_overflow = [&](std::vector<uint32_t> *list, std::vector<uint32_t> *list16) -> bool {
@@ -649,24 +744,32 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
       ce = cudaMemsetAsync(d_novf, 0, 32, st);
       if (ce != cudaSuccess) return cuda_fail(ce, "overflow reset");
     }
-    if (n_conc) {  // fork: each shape on its own side stream and strip region; join on st
+    if (n_conc) {  // fork: each shape on its own side stream (and strip region); join on st
       ce = cudaEventRecord(ctx->fork_ev, st);
       int si = 0;
       for (const Group &g : w.groups) {
         if (ce != cudaSuccess) break;
         cudaStream_t s2 = ctx->side[si];
         ce = cudaStreamWaitEvent(s2, ctx->fork_ev, 0);
-        fa.strip_buf = d_strip + shape_strip[g.shape];
-        if (ce == cudaSuccess &&
-            !run_group(d_order + g.begin, g.end - g.begin, g.family, g.R, g.warps, s2,
-                       shape_grid[g.shape]))
-          return cuda_fail(ce, "forward kernel launch");
+        if (split != SPLIT_NONE) {
+          if (ce == cudaSuccess && !run_split(g, si, s2)) return cuda_fail(ce, "forward kernel launch");
+        } else {
+          fa.strip_buf = d_strip + shape_strip[g.shape];
+          if (ce == cudaSuccess &&
+              !run_group(d_order + g.begin, g.end - g.begin, g.family, g.R, g.warps, s2,
+                         shape_grid[g.shape]))
+            return cuda_fail(ce, "forward kernel launch");
+        }
         if (ce == cudaSuccess) ce = cudaEventRecord(ctx->join_ev[si], s2);
         ++si;
       }
       for (int i = 0; i < si && ce == cudaSuccess; ++i) ce = cudaStreamWaitEvent(st, ctx->join_ev[i], 0);
       fa.strip_buf = d_strip;
       if (ce != cudaSuccess) return cuda_fail(ce, "forking the forward launches");
+    } else if (split != SPLIT_NONE) {
+      int gi = 0;
+      for (const Group &g : w.groups)
+        if (!run_split(g, gi++, st)) return cuda_fail(ce, "forward kernel launch");
     } else {
       for (const Group &g : w.groups)
         if (!run_group(d_order + g.begin, g.end - g.begin, g.family, g.R, g.warps, st, grid_max))

@@ -36,6 +36,7 @@ struct Ctx {
   double last_host_wait_ms = 0, last_host_plan_ms = 0;
   Plan plan;                       // the last call's plan; its buffers are reused
   int dev_plan_mode = 0;           // 0: device planner by batch size, 1: never, 2: always
+  int split_mode = 0;              // a warp per strip: 0 by batch size, 1 never, 2 whenever possible
   int search_ring = 0;             // search score pass: shared-memory ring entries, 0 default
   bool last_dev_plan = false;      // the last call was planned on the device
   std::vector<uint32_t> h_ql, h_rl;  // the last call's lengths (host copies)
@@ -86,6 +87,7 @@ struct Ctx {
   int full_blocks_per_sm(int R, const ScoreParams &sp);
   int pack_blocks_per_sm(int R, const ScoreParams &sp);
   int graph_blocks_per_sm(int R, bool packed, const ScoreParams &sp);  // filtr_graph instances
+  int split_blocks_per_sm(bool packed, int R, const ScoreParams &sp);  // a warp per strip (k_split.cuh)
   bool ensure_host(size_t bytes);
   cudaEvent_t next_event();
   // open / close a timed span on stream st (no-ops when timing is off)

@@ -21,13 +21,6 @@ constexpr int32_t NEG = -(1 << 29);
 constexpr int32_t NEG_HALF = NEG / 2;
 constexpr int MAX_ALPHA = 20;
 constexpr int FULL_WARPS = 2;  // warps per CTA of the tiled wavefront kernel
-// Rows per lane of the intra-pair strip kernel (strips of 32 * LONG_R rows).
-// One long pair keeps only (strip width / strip height) strips in flight and
-// each strip's step is latency bound, so lower strips (shorter steps, more of
-// them in flight) finish sooner: an 80 kbp banded pair's forward took 48.2 ms
-// at 8 rows against 55.1 ms at 16.
-constexpr int LONG_R = 8;
-
 // Band limits on d = j - i (Sec. 7.1 prune axis), widened to hold both corners
 // unless the literal +-B band is asked for.
 FILTR_HD void band_limits(int64_t M, int64_t N, int64_t B, bool literal, int64_t *lo,
@@ -254,30 +247,7 @@ struct WalkArgs {
   const GraphDesc *gd = nullptr;  // captured pipeline: b, out and n_order from here
 };
 
-struct LaneBest;
-// One long pair across the whole grid (k_long.cu).
-struct LongArgs {
-  const uint8_t *q, *r;
-  int M, N;
-  int lo, hi;                 // band on j - i (unbanded: -M-1, N+1)
-  ScoreParams sp;
-  int2 *ring;                 // NW slots of ring_stride entries
-  uint32_t ring_stride;
-  unsigned long long *prog;   // NW progress words (strip << 32 | column), zeroed
-  int *err;                   // set to 1 when a wait times out
-  unsigned long long timeout_ns;
-  int withhold;               // test hook: strip 0 never publishes (forces the timeout)
-  uint32_t *tb;               // traceback words (nullptr without traceback)
-  const int64_t *strip_base;  // first traceback word of each strip
-  struct LaneBest *wbest;     // one per warp
-  int *end_h;                 // H(M, N)
-};
-
 // ---- launches (defined in the .cu files) -----------------------------------
-cudaError_t launch_long(const LongArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_long_finish(const LongArgs &a, int nw, uint64_t cells, filtr_result *out,
-                               FwdOut *fwd, cudaStream_t s);
-int long_blocks_per_sm(const ScoreParams &sp);
 cudaError_t launch_full(const FullArgs &a, int R, int grid, cudaStream_t s);
 int full_smem_bytes(int R, int alphabet);
 int full_max_blocks_per_sm(int R, const ScoreParams &sp, int alphabet);

@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "filtr_ctx.h"
+#include "k_split.cuh"
 
 namespace filtr {
 namespace {
@@ -32,12 +33,12 @@ __global__ void k_graph_desc(GraphDesc d, GraphDesc *dst) {
 // One thread: the checks filtr_align_batch makes on the host, and that every
 // pair's shape is one the graph launches (shapes_in: bit k for shape k).
 __global__ void k_graph_check(const DevPlanState *ps, GraphDesc *gd, uint32_t max_len,
-                              unsigned long long tb_cap, unsigned long long stage_cap,
-                              uint32_t shapes_in) {
+                              unsigned long long tb_cap, unsigned long long ref_cap,
+                              unsigned long long stage_cap, uint32_t shapes_in) {
   int32_t code = 0;
   if (ps->bad[0] != 0 || ps->sum.max_m > max_len || ps->sum.max_n > max_len)
     code = FILTR_ERR_INVALID;
-  else if (ps->sum.tb_words > tb_cap || ps->sum.stage_words > stage_cap)
+  else if (ps->sum.tb_words > tb_cap || ps->sum.tb_words_ref > ref_cap || ps->sum.stage_words > stage_cap)
     code = FILTR_ERR_NOMEM;
   for (int k = 0; k < SHAPE_TILED && code == 0; ++k)
     if (!(shapes_in >> k & 1u) && ps->sum.count[k] != 0) code = FILTR_ERR_UNSUPPORTED;
@@ -112,6 +113,9 @@ struct ShapeSet {
   int k[SHAPE_TILED];
   int grid[SHAPE_TILED];
   int n = 0;
+  int split = SPLIT_NONE;        // a warp per strip (k_split.cuh) instead of a warp per pair
+  SplitSpace space[SHAPE_TILED];
+  uint32_t strips[SHAPE_TILED];  // strips of max_len rows
 };
 // Shapes choose_shape can give some pair with both lengths at most max_len.
 // Within one block of 64 query rows every shape's strip count is fixed and its
@@ -157,21 +161,47 @@ void reachable_shapes(const ShapeTable &t, const ScoreParams &sp, uint32_t max_l
   }
 }
 
-ShapeSet graph_shapes(Ctx *c, const ScoreParams &sp, const ShapeCost *costs, uint32_t max_len) {
+ShapeSet graph_shapes(Ctx *c, const ScoreParams &sp, const ShapeCost *costs, uint32_t max_len,
+                      uint32_t max_pairs, int split) {
   ShapeSet ss;
+  ss.split = split;
   const bool pack_ok = !sp.use_band && sp.precision != FILTR_PREC_I32;
   bool reach[SHAPE_TILED];
-  reachable_shapes(make_shape_table(costs, sp), sp, max_len, reach);
+  reachable_shapes(make_shape_table(costs, sp, split), sp, max_len, reach);
   for (int k = 0; k < SHAPE_TILED; ++k) {
     if (costs[k].packed && !pack_ok) continue;
     if (!reach[k]) continue;
-    const int R = costs[k].R;
-    const int bps = c->graph_blocks_per_sm(R, costs[k].packed, sp);
-    ss.k[ss.n] = k;
-    ss.grid[ss.n] = c->sms * bps;
+    const int R = costs[k].R, i = ss.n;
+    ss.k[i] = k;
+    if (split == SPLIT_NONE) {
+      ss.grid[i] = c->sms * c->graph_blocks_per_sm(R, costs[k].packed, sp);
+    } else {
+      const uint32_t rows = (uint32_t)split_rows(costs[k].packed, R);
+      ss.strips[i] = (max_len + rows - 1) / rows;
+      ss.space[i] = split_space(max_pairs, ss.strips[i], (uint64_t)max_len + 1);
+      ss.grid[i] = c->sms * c->split_blocks_per_sm(costs[k].packed, R, sp);
+    }
     ++ss.n;
   }
   return ss;
+}
+
+// Device memory of shape i's forward launch: strip buffers or hand-over slots.
+size_t shape_bytes(const ShapeSet &ss, int i, uint32_t max_len) {
+  return ss.split != SPLIT_NONE ? ss.space[i].bytes
+                                : (size_t)ss.grid[i] * FULL_WARPS * (max_len + 2) * sizeof(int2);
+}
+// Most traceback words a pair within max_len can need in any of the shapes.
+uint64_t worst_tb_words(const ShapeSet &ss, const ShapeCost *costs, const ScoreParams &sp, uint32_t max_len) {
+  uint64_t w = 0;
+  ScoreParams full = sp;
+  full.use_band = 0;
+  for (int i = 0; i < ss.n; ++i) {
+    const int R = costs[ss.k[i]].R;
+    w = std::max(w, costs[ss.k[i]].packed ? strips_of(max_len, R) * pack_strip_tb_words(1, max_len, R)
+                                          : full_tb_words(max_len, max_len, R, full));
+  }
+  return w;
 }
 
 // Capture the pipeline on st into g->graph.  The shapes' kernels sit in
@@ -179,7 +209,7 @@ ShapeSet graph_shapes(Ctx *c, const ScoreParams &sp, const ShapeCost *costs, uin
 // queue counter), so a shape the plan leaves empty costs nothing and the
 // shapes' tails overlap.  Returns the first error.
 cudaError_t capture(Graph *g, const ShapeCost *costs, const ShapeSet &ss, uint64_t tb_words,
-                    uint64_t stage_cap, const GCarve &layout_in, cudaStream_t st,
+                    uint64_t ref_words, uint64_t stage_cap, const GCarve &layout_in, cudaStream_t st,
                     cudaStream_t st2) {
   const ScoreParams &sp = g->sp;
   const uint32_t NP = g->max_pairs;
@@ -196,9 +226,8 @@ cudaError_t capture(Graph *g, const ShapeCost *costs, const ShapeSet &ss, uint64
   uint64_t *d_pwords = cv.take<uint64_t>(NP);
   uint64_t *d_pblk = cv.take<uint64_t>((NP + DEV_PLAN_BLOCK - 1) / DEV_PLAN_BLOCK);
   const uint32_t strip_stride = g->max_len + 2;
-  int2 *d_strip[SHAPE_TILED];
-  for (int i = 0; i < ss.n; ++i)
-    d_strip[i] = cv.take<int2>((size_t)ss.grid[i] * FULL_WARPS * strip_stride);
+  char *d_strip[SHAPE_TILED];
+  for (int i = 0; i < ss.n; ++i) d_strip[i] = cv.take<char>(shape_bytes(ss, i, g->max_len));
   uint32_t *d_stage = sp.traceback ? cv.take<uint32_t>(stage_cap) : nullptr;
   uint32_t *d_tb = cv.take<uint32_t>(tb_words);
   uint32_t *d_bad = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(d_ps) +
@@ -216,7 +245,11 @@ cudaError_t capture(Graph *g, const ShapeCost *costs, const ShapeSet &ss, uint64
   DevPlanArgs pa{};
   pa.n = NP;
   pa.sp = sp;
-  pa.tab = make_shape_table(costs, sp);
+  pa.tab = make_shape_table(costs, sp, ss.split);
+  if (ss.split != SPLIT_NONE && sp.traceback) {
+    pa.ref_tab = make_shape_table(costs, sp);
+    pa.use_ref = 1;
+  }
   pa.state = d_ps;
   pa.key = d_pkey;
   pa.words = d_pwords;
@@ -230,6 +263,7 @@ cudaError_t capture(Graph *g, const ShapeCost *costs, const ShapeSet &ss, uint64
     uint32_t shapes_in = 0;
     for (int i = 0; i < ss.n; ++i) shapes_in |= 1u << ss.k[i];
     k_graph_check<<<1, 1, 0, st>>>(d_ps, g->d_gd, g->max_len, (unsigned long long)tb_words,
+                                   (unsigned long long)ref_words,
                                    (unsigned long long)(sp.traceback ? stage_cap : ~0ull),
                                    shapes_in);
     e = cudaGetLastError();
@@ -281,9 +315,22 @@ cudaError_t capture(Graph *g, const ShapeCost *costs, const ShapeSet &ss, uint64
     if (e != cudaSuccess) break;
     fa.counter = d_counters + k;
     fa.gshape = k;
-    fa.strip_buf = d_strip[i];
-    e = costs[k].packed ? launch_pack(fa, costs[k].R, ss.grid[i], st2)
-                        : launch_full(fa, costs[k].R, ss.grid[i], st2);
+    if (ss.split != SPLIT_NONE) {
+      SplitLaunch sl{};
+      sl.packed = costs[k].packed;
+      sl.R = costs[k].R;
+      sl.count = NP;
+      sl.max_strips = ss.strips[i];
+      sl.grid = ss.grid[i];
+      sl.a.f = fa;
+      sl.a.timeout_ns = SPLIT_TIMEOUT_NS;
+      split_bind(&sl.a, d_strip[i], ss.space[i], g->max_len + 1);
+      e = launch_split(sl, st2);
+    } else {
+      fa.strip_buf = reinterpret_cast<int2 *>(d_strip[i]);
+      e = costs[k].packed ? launch_pack(fa, costs[k].R, ss.grid[i], st2)
+                          : launch_full(fa, costs[k].R, ss.grid[i], st2);
+    }
     cudaGraph_t body = nullptr;
     const cudaError_t eb = cudaStreamEndCapture(st2, &body);
     if (e == cudaSuccess) e = eb;
@@ -364,10 +411,9 @@ filtr_status filtr_graph_create(filtr_ctx *ctx, const filtr_params *params, uint
 
   // layout: fixed parts (capacity-sized), strip buffers per shape, staging,
   // traceback
-  const ShapeSet ss = graph_shapes(c, sp, costs, max_len);
   const uint64_t stage_cap = sp.traceback ? (uint64_t)max_pairs * (2ull * max_len + 1) : 0;
-  GCarve probe{nullptr};  // the same sequence of parts as capture() carves
-  {
+  auto fixed_bytes = [&](const ShapeSet &s) {  // the same sequence of parts as capture() carves
+    GCarve probe{nullptr};
     probe.take<GraphDesc>(1);
     probe.take<DevPlanState>(1);
     probe.take<uint32_t>(max_pairs);
@@ -380,15 +426,36 @@ filtr_status filtr_graph_create(filtr_ctx *ctx, const filtr_params *params, uint
     probe.take<uint16_t>(max_pairs);
     probe.take<uint64_t>(max_pairs);
     probe.take<uint64_t>((max_pairs + DEV_PLAN_BLOCK - 1) / DEV_PLAN_BLOCK);
-    for (int i = 0; i < ss.n; ++i) probe.take<int2>((size_t)ss.grid[i] * FULL_WARPS * (max_len + 2));
+    for (int i = 0; i < s.n; ++i) probe.take<char>(shape_bytes(s, i, max_len));
     if (sp.traceback) probe.take<uint32_t>(stage_cap);
     probe.take<uint32_t>(0);
-  }
-  const size_t fixed = probe.used;
+    return probe.used;
+  };
+  ShapeSet ss = graph_shapes(c, sp, costs, max_len, max_pairs, SPLIT_NONE);
+  size_t fixed = fixed_bytes(ss);
   if (workspace_bytes < fixed + (sp.traceback ? 4096 : 0)) {
     set_error("filtr_graph_create: %zu bytes of workspace, the bounds need %zu before traceback",
               workspace_bytes, fixed);
     return FILTR_ERR_NOMEM;
+  }
+  // A graph of few pairs runs them a warp per strip, when the workspace holds any
+  // batch within the bounds that way.  Its shapes take more or less traceback
+  // than the warp-per-pair ones; which batches the traceback area holds stays
+  // what those need (the check node compares ref_words).
+  const uint64_t ref_words = sp.traceback ? (workspace_bytes - fixed) / 4 : 0;
+  if (max_len > 256 && !c->tuned_costs(sp) && c->split_mode != 1 && (c->split_mode == 2 || max_pairs <= (sp.use_band ? SPLIT_MAX_BANDED : SPLIT_LATENCY_PAIRS))) {
+    const int order[2] = {max_pairs <= SPLIT_LATENCY_PAIRS ? SPLIT_PACK8 : SPLIT_PACK8_16, SPLIT_PACK16};
+    for (int mode : order) {
+      const ShapeSet s = graph_shapes(c, sp, costs, max_len, max_pairs, mode);
+      const size_t f = fixed_bytes(s);
+      const uint64_t worst = sp.traceback ? max_pairs * worst_tb_words(s, costs, sp, max_len) : 0;
+      bool ok = f + worst * 4 + 4096 <= workspace_bytes;
+      for (int i = 0; i < s.n; ++i) ok = ok && s.strips[i] <= SPLIT_MAX_STRIPS;
+      if (!ok) continue;
+      ss = s;
+      fixed = f;
+      break;
+    }
   }
   const uint64_t tb_words = sp.traceback ? (workspace_bytes - fixed) / 4 : 0;
 
@@ -419,7 +486,7 @@ filtr_status filtr_graph_create(filtr_ctx *ctx, const filtr_params *params, uint
     graph_free(g);
     return cuda_fail(e, "cudaStreamCreate");
   }
-  e = capture(g, costs, ss, tb_words, stage_cap, lay, st, st2);
+  e = capture(g, costs, ss, tb_words, ref_words, stage_cap, lay, st, st2);
   cudaStreamDestroy(st);
   cudaStreamDestroy(st2);
   if (e != cudaSuccess) {

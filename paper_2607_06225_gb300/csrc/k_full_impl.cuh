@@ -19,11 +19,9 @@ namespace {
 // Strip I/O through one per-warp buffer (no cross-warp waits).
 struct WarpIO {
   int2 *buf;
-  __device__ bool wait(int) { return true; }
   static constexpr bool FETCH = false;
   __device__ int2 in(int j) { return buf[j]; }
   __device__ void out(int j, int H, int F) { buf[j] = make_int2(H, F); }
-  __device__ void done_col(int, int, int) {}
 };
 
 template <int R, bool LOCAL, bool AFFINE, bool TB, bool BAND, bool GR>

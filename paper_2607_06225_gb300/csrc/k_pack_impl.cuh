@@ -130,8 +130,19 @@ __device__ __forceinline__ void best_put(Best &b, int v, int i, int j) {
   }
 }
 
-template <int R, bool LOCAL, bool AFFINE, bool TB>
-__device__ __forceinline__ void pack_strip(const PackPair &PP, int s, int64_t tb_base, int2 *buf,
+// The strip above's bottom row, biased H in the low half and F in the high half
+// of a word per column, from a per-warp buffer: lane 0 reads, lane 31 writes.
+// An IO with FETCH set fetches ahead instead: fetch(j, jmax, v) gives lane x
+// column j + x for the n columns (1 <= n <= 32, up to jmax) that are ready.
+struct PackBuf {
+  static constexpr bool FETCH = false;
+  uint32_t *buf;
+  __device__ uint32_t in(int j) { return buf[j]; }
+  __device__ void out(int j, uint32_t hf) { buf[j] = hf; }
+};
+
+template <int R, bool LOCAL, bool AFFINE, bool TB, class IO>
+__device__ __forceinline__ void pack_strip(const PackPair &PP, int s, int64_t tb_base, IO &io,
                                            Best &best, int &endH) {
   constexpr int HS = 32 * R, P = R / 2, G = (P + 7) / 8, WPS = 2 * G;
   constexpr int PW = (P + 3) / 4, PS = pack_prof_stride(R);
@@ -209,6 +220,9 @@ __device__ __forceinline__ void pack_strip(const PackPair &PP, int s, int64_t tb
   uint32_t bestkey = ((uint32_t)(best.v + B) << 16) | 31u;
   int rc_lo = PP.r[0], rc_hi = rc_lo;
   int rc_next = PP.r[min(max(1 - 2 * lane, 1), N) - 1];
+  // columns fetched ahead (IO::FETCH): lane x of pv holds column pbase + x, x < pn
+  uint32_t pv = 0;
+  int pbase = 0, pn = 0;
 
   // one step; the steps where some lane has a half outside [1, N] (the first
   // 63 and those from N on) run the masked form, the steady ones the plain
@@ -220,6 +234,17 @@ __device__ __forceinline__ void pack_strip(const PackPair &PP, int s, int64_t tb
     const bool actH = !EDGE_STEP || (cH >= 1 && cH <= N);
     uint32_t sH = __shfl_up_sync(PFULL, outH, 1);
     uint32_t sF = __shfl_up_sync(PFULL, outF, 1);
+    uint32_t vin = 0;
+    if constexpr (IO::FETCH) {
+      const int j0 = 1 + t;  // lane 0's column
+      if (s > 0 && j0 <= N) {
+        if (j0 >= pbase + pn) {
+          pn = io.fetch(j0, N, pv);
+          pbase = j0;
+        }
+        vin = __shfl_sync(PFULL, pv, j0 - pbase);
+      }
+    }
     if (lane == 0) {
       // outside [1, N] the row above is a placeholder, but it must stay inside
       // the biased range: a half that wraps below 0 borrows from (or carries
@@ -229,9 +254,9 @@ __device__ __forceinline__ void pack_strip(const PackPair &PP, int s, int64_t tb
       if (s == 0 && actL) {
         hv = (uint32_t)(LOCAL ? B : B - o - cL * e) & 0xffffu;  // H(0, cL)
       } else if (actL) {
-        const int2 v = buf[cL];
-        hv = (uint32_t)v.x;
-        fv = (uint32_t)v.y;
+        if constexpr (!IO::FETCH) vin = io.in(cL);
+        hv = vin & 0xffffu;
+        fv = vin >> 16;
       }
       sH = hv << 16;
       sF = fv << 16;
@@ -339,7 +364,7 @@ __device__ __forceinline__ void pack_strip(const PackPair &PP, int s, int64_t tb
       for (int w = 0; w < WPS; ++w) PP.tb[tb_base + ((int64_t)t * WPS + w) * 32 + lane] = tbw[w];
     }
     if (lane == 31 && actH && s + 1 < nstrips)
-      buf[cH] = make_int2((int)(Hc[P - 1] >> 16), (int)(Fup >> 16));
+      io.out(cH, perm<0x7632>(Hc[P - 1], Fup));  // both high halves
     // best cell (local): a lane takes the step's largest key only if strictly
     // above its best key (equal keys: the same row at a later column, whose
     // smaller j already stands).  Rows past M stay below a valid cell of their
@@ -379,7 +404,7 @@ __global__ void __launch_bounds__(FULL_WARPS * 32) k_pack(const FullArgs a) {
   for (int t = threadIdx.x; t < A * A; t += blockDim.x) s_sub[t] = a.sp.subst[t];
   __syncthreads();
   const int gw = blockIdx.x * FULL_WARPS + wib;
-  int2 *buf = a.strip_buf + (size_t)gw * a.strip_stride;
+  PackBuf buf{reinterpret_cast<uint32_t *>(a.strip_buf + (size_t)gw * a.strip_stride)};
 
   for (;;) {
     uint32_t t0 = 0;

@@ -59,13 +59,14 @@ __global__ void __launch_bounds__(DEV_PLAN_BLOCK) k_plan_classify(const DevPlanA
   const PlanView V = plan_view(a);
   if (blockIdx.x * DEV_PLAN_BLOCK >= V.n) return;  // uniform over the block
   __shared__ uint32_t hist[PLAN_KEYS];
-  __shared__ unsigned long long part[5][DEV_PLAN_BLOCK / 32];
+  __shared__ unsigned long long part[6][DEV_PLAN_BLOCK / 32];
   __shared__ uint32_t pmax[2][DEV_PLAN_BLOCK / 32];
   for (int i = threadIdx.x; i < PLAN_KEYS; i += DEV_PLAN_BLOCK) hist[i] = 0;
   __syncthreads();
   const uint32_t p = blockIdx.x * DEV_PLAN_BLOCK + threadIdx.x;
-  // traceback words, cells, staging words, M + N, cells of int16x2 shapes
-  unsigned long long v[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
+  // traceback words, cells, staging words, M + N, cells of int16x2 shapes,
+  // traceback words in the reference shapes
+  unsigned long long v[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
   uint32_t mm = 0, mn = 0;
   if (p < V.n) {
     const uint32_t M = V.q_len[p], N = V.r_len[p];
@@ -81,6 +82,8 @@ __global__ void __launch_bounds__(DEV_PLAN_BLOCK) k_plan_classify(const DevPlanA
       if (a.sp.traceback) w = shape_tb_words(a.tab, k, M, N, a.sp);
       v[1] = cost;
       v[4] = a.tab.packed[k] ? cost : 0ull;
+      if (a.use_ref)
+        v[5] = shape_tb_words(a.ref_tab, choose_shape(a.ref_tab, a.sp, M, N), M, N, a.sp);
       key = k * 64 + cost_bucket_desc(cost);
     }
     v[0] = w;
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(DEV_PLAN_BLOCK) k_plan_classify(const DevPlanA
   }
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
+  for (int i = 0; i < 6; ++i) {
     unsigned long long x = v[i];
     for (int o = 16; o; o >>= 1) x += __shfl_down_sync(FULL_MASK, x, o);
     if (lane == 0) part[i][wp] = x;
@@ -103,7 +106,7 @@ __global__ void __launch_bounds__(DEV_PLAN_BLOCK) k_plan_classify(const DevPlanA
   }
   __syncthreads();
   DevPlanSummary &S = a.state->sum;
-  if (threadIdx.x < 5) {
+  if (threadIdx.x < 6) {
     unsigned long long x = 0;
     for (int k = 0; k < DEV_PLAN_BLOCK / 32; ++k) x += part[threadIdx.x][k];
     if (threadIdx.x == 2) a.blk[blockIdx.x] = x;
@@ -111,10 +114,11 @@ __global__ void __launch_bounds__(DEV_PLAN_BLOCK) k_plan_classify(const DevPlanA
                               : threadIdx.x == 1 ? &S.cells
                               : threadIdx.x == 2 ? &S.stage_words
                               : threadIdx.x == 3 ? &S.cigar_upper
-                                                 : &S.cells_packed;
+                                                 : threadIdx.x == 4 ? &S.cells_packed
+                                              : &S.tb_words_ref;
     if (x) atomicAdd(dst, x);
-  } else if (threadIdx.x < 7) {
-    const int t = threadIdx.x - 5;
+  } else if (threadIdx.x < 8) {
+    const int t = threadIdx.x - 6;
     uint32_t x = 0;
     for (int k = 0; k < DEV_PLAN_BLOCK / 32; ++k) x = max(x, pmax[t][k]);
     atomicMax(t ? &S.max_n : &S.max_m, x);

@@ -1,5 +1,5 @@
 // k_strip.cuh -- one row strip of the tiled wavefront (shared by the batched
-// kernel k_full and the intra-pair kernel k_long).
+// kernel k_full, a warp per pair, and the split kernel, a warp per strip).
 //
 // A strip is 32*R query rows; lane l owns rows [row0 + lR + 1, row0 + lR + R]
 // in registers.  At step t lane l updates column j = jlo + t - l of its rows,
@@ -124,22 +124,19 @@ struct LaneBest {
 };
 
 // Process strip s.  IO must provide (called by every lane unless noted):
-//   bool wait(int j)          -- before lane 0 reads column j of the strip
-//                                above; false aborts the strip (timeout)
-//   int2 in(int j)            -- lane 0 only: (H, F) of the strip above
 //   FETCH                     -- constexpr bool: lane 0's input row is
 //                                fetched ahead with fetch() instead of in()
-//   int fetch(int j, int jmax, int2 &v) -- (FETCH only) after wait(j): lane x
-//                                loads (H, F) of column j + x of the strip
-//                                above for the n columns (1 <= n <= 32, up to
-//                                jmax) known to be ready; returns n
+//   int2 in(int j)            -- (not FETCH) lane 0 only: (H, F) of the strip above
+//   int fetch(int j, int jmax, int2 &v) -- (FETCH) lane x loads (H, F) of column
+//                                j + x of the strip above for the n columns
+//                                (1 <= n <= 32, up to jmax) known to be ready,
+//                                waiting for the first; returns n
 //   void out(int j, int H, int F) -- lane 31 only: this strip's bottom row
-//   void done_col(int j, int jlo, int jhi) -- lane 31 only, after out(j)
 // prev_jlo / prev_jhi: the strip above's columns (empty for s == 0).
-// Returns false if IO aborted.  endH receives H(M, jhi) for the lane holding
-// row M when this is the last strip.
+// endH receives H(M, jhi) for the lane holding row M when this is the last
+// strip.
 template <int R, bool LOCAL, bool AFFINE, bool TB, bool BAND, class IO>
-__device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, int jhi, int prev_jlo,
+__device__ __forceinline__ void strip_pass(const StripPair &P, int s, int jlo, int jhi, int prev_jlo,
                                            int prev_jhi, int64_t tb_base, IO &io, LaneBest &best,
                                            int &endH) {
   constexpr int HS = 32 * R;
@@ -196,8 +193,13 @@ __device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, i
   } else if (s > 0) {
     const int jj = jlo - 1;
     if (jj >= prev_jlo && jj <= prev_jhi) {
-      if (!io.wait(jj)) return false;
-      if (lane == 0) dtop = io.in(jj).x;
+      if constexpr (IO::FETCH) {
+        int2 v;
+        io.fetch(jj, jj, v);
+        if (lane == 0) dtop = v.x;
+      } else {
+        if (lane == 0) dtop = io.in(jj).x;
+      }
     }
   }
 
@@ -205,7 +207,7 @@ __device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, i
   int upH = NEG, upF = NEG, prevIn = dtop;
   // lane 0's input row, fetched ahead (IO::FETCH): lane x of pv holds column
   // pbase + x of the strip above (x < pn), so a step waits on a load once per
-  // fetch.  A strip that follows the strip above closely (one long pair) would
+  // fetch.  A strip that follows the strip above closely (split pairs) would
   // otherwise wait on a load every step; with many warps per SM (batched
   // pairs) the loads' latency is hidden anyway, and the registers cost more.
   int2 pv = make_int2(NEG, NEG);
@@ -228,15 +230,12 @@ __device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, i
     if constexpr (IO::FETCH) {
       if (need) {
         if (j0 >= pbase + pn) {
-          if (!io.wait(j0)) return false;
           pn = io.fetch(j0, prev_jhi, pv);
           pbase = j0;
         }
         vin.x = __shfl_sync(STRIP_FULLMASK, pv.x, j0 - pbase);
         vin.y = AFFINE ? __shfl_sync(STRIP_FULLMASK, pv.y, j0 - pbase) : NEG;
       }
-    } else {
-      if (need && !io.wait(j0)) return false;
     }
     int inH = __shfl_up_sync(STRIP_FULLMASK, upH, 1);
     int inF = AFFINE ? __shfl_up_sync(STRIP_FULLMASK, upF, 1) : NEG;
@@ -315,10 +314,7 @@ __device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, i
 #pragma unroll
         for (int w = 0; w < WPS; ++w) P.tb[tb_base + ((int64_t)t * WPS + w) * 32 + lane] = tbw[w];
       }
-      if (lane == 31 && s + 1 < nstrips) {
-        io.out(j, Hup, Fup);
-        io.done_col(j, jlo, jhi);
-      }
+      if (lane == 31 && s + 1 < nstrips) io.out(j, Hup, Fup);
       // rows past M stay below a valid cell of their lane already seen, so
       // they never win; lanes wholly past M keep no best
       if (LOCAL && top <= M && mkey > bestkey) {
@@ -335,7 +331,6 @@ __device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, i
       if (top + k == M) endH = Hc[k];
   }
   __syncwarp();
-  return true;
 }
 
 // warp-wide reduction of LaneBest with the tie-break (all lanes get the result)

@@ -801,14 +801,17 @@ __global__ void k_compact(const WalkArgs a, uint32_t n, const uint64_t *offs, ui
 
 }  // namespace
 
+constexpr uint32_t WALK_WARP_PAIRS = 16384;
+
 cudaError_t launch_walk(const WalkArgs &a, cudaStream_t s) {
   if (a.n_order == 0) return cudaSuccess;
   // A warp per pair keeps more loads in flight for each pair but issues the
-  // serial walk as a whole warp's instructions: for one or a few pairs (plain
-  // per-pair calls, a long pair) it is the faster form; with thousands of pairs
-  // a thread per pair (32 pairs per instruction stream) is (2.5 ms against
-  // 3.4 ms for the 100,000-pair protein batch).
-  if (a.n_order <= 256)
+  // serial walk as a whole warp's instructions.  Up to about one warp per resident
+  // slot of the device (and some) it is the faster form: 4096 protein pairs of
+  // 100-1000 through the captured pipeline 3.3 -> 1.85 ms, 512 banded reads' walk
+  // about 27 -> 6 ms.  With many more pairs a thread per pair (32 pairs per
+  // instruction stream) is: 2.5 ms against 3.4 ms for 100,000 protein pairs.
+  if (a.n_order <= WALK_WARP_PAIRS)
     k_walk_tw<<<(a.n_order + 3) / 4, 128, 0, s>>>(a);
   else
     k_walk<<<(a.n_order + 127) / 128, 128, 0, s>>>(a);

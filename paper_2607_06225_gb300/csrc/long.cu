@@ -1,17 +1,17 @@
 // long.cu -- filtr_align_long: one long pair with every SM on it.
 //
 // X-drop pairs (and pairs with an empty side) run as a one-pair batch of the
-// antidiagonal kernel with a 4-warp first window (reruns widen it); the
-// antidiagonal order is inherently sequential, so one wide group is what the
-// pair can use.  Full-matrix and banded pairs run the cooperative strip kernel
-// (k_long.cu) across the whole grid, then the ordinary traceback walk.
+// antidiagonal kernel with a 4-warp first window (reruns widen it), or as a
+// segmented sweep; the antidiagonal order is inherently sequential, so one group
+// is what the pair can use.  Full-matrix and banded pairs run a warp per row
+// strip across the device (k_split.cuh), then the ordinary traceback walk.
 #include <algorithm>
 #include <cstring>
 #include <vector>
 
 #include "../../include/filtr_testing.h"
 #include "filtr_ctx.h"
-#include "k_strip.cuh"
+#include "k_split.cuh"
 #include "k_xdrop_layout.h"
 #include "plan.h"
 
@@ -34,7 +34,6 @@ struct Carve {
   }
 };
 
-constexpr unsigned long long LONG_TIMEOUT_NS = 20ull * 1000 * 1000 * 1000;  // 20 s without progress
 
 filtr_status validate_seq(Ctx *c, const uint8_t *q, uint32_t M, const uint8_t *r, uint32_t N,
                           int alphabet, cudaStream_t st) {
@@ -54,45 +53,33 @@ filtr_status validate_seq(Ctx *c, const uint8_t *q, uint32_t M, const uint8_t *r
   return FILTR_OK;
 }
 
-// the cooperative strip kernel; withhold != 0 is the timeout test
+// a warp per row strip of the int32 tile (k_split.cuh); withhold != 0 is the timeout test
 filtr_status run_long(Ctx *c, const ScoreParams &sp, const filtr_params *params, const uint8_t *q,
                       uint32_t M, const uint8_t *r, uint32_t N, filtr_result *out, uint32_t *cigar,
                       uint64_t cap, cudaStream_t st, int withhold, unsigned long long timeout_ns,
                       bool sync = true) {
-  constexpr int R = LONG_R, HS = 32 * R;
-  int64_t lo = -(int64_t)M - 1, hi = (int64_t)N + 1;
+  (void)params;
+  constexpr int R = 8, HS = 32 * R;
+  int64_t widest = N;
   if (sp.use_band) {
+    int64_t lo, hi;
     band_limits(M, N, sp.band, sp.band_literal, &lo, &hi);
-    lo = std::max<int64_t>(lo, -(int64_t)M - 1);
-    hi = std::min<int64_t>(hi, (int64_t)N + 1);
+    widest = std::max<int64_t>(1, std::min<int64_t>(N, hi - lo + HS));
   }
-  const int nstrips = (int)((M + HS - 1) / HS);
-  // strip geometry: widest strip and traceback bases
-  std::vector<int64_t> base(nstrips + 1, 0);
-  int64_t widest = 0;
-  for (int s = 0; s < nstrips; ++s) {
-    int64_t jl, jh;
-    strip_cols((int64_t)s * HS, HS, M, N, sp.use_band != 0, lo, hi, &jl, &jh);
-    widest = std::max<int64_t>(widest, jh >= jl ? jh - jl + 1 : 0);
-    base[s + 1] = base[s] + (sp.traceback ? strip_tb_words(jl, jh, R) : 0);
-  }
-  const uint64_t tb_words = (uint64_t)base[nstrips];
-  const int bps = std::max(1, long_blocks_per_sm(sp));
-  int grid = c->sms * bps;
-  grid = std::max(1, std::min(grid, (nstrips + FULL_WARPS - 1) / FULL_WARPS));
-  // the ring may use a quarter of the workspace
-  const uint64_t stride = (uint64_t)widest + 2;
-  while (grid > 1 && (uint64_t)grid * FULL_WARPS * stride * 8 > c->ws_bytes / 4) grid /= 2;
-  if (withhold) grid = std::max(grid, 2);
-  const int nw = grid * FULL_WARPS;
+  const uint32_t nstrips = (uint32_t)((M + (uint64_t)HS - 1) / HS);
+  const uint64_t tb_words = sp.traceback ? full_tb_words(M, N, R, sp) : 0;
+  // a banded strip starts HS columns after the one above, so only about
+  // widest / HS of them ever run at once; more warps would only wait
+  const int64_t in_flight = sp.use_band ? widest / HS + 6 : (int64_t)nstrips;
+  const int grid = (int)std::max<int64_t>(
+      withhold ? 2 : 1,
+      std::min<int64_t>((int64_t)c->sms * c->split_blocks_per_sm(false, R, sp),
+                        (std::min<int64_t>(in_flight, nstrips) + FULL_WARPS - 1) / FULL_WARPS));
+  const uint64_t stride = (uint64_t)widest + 1;
+  const SplitSpace space = split_space(1, nstrips, stride);
 
   Carve cv{c->ws, c->ws_bytes};
-  int2 *ring = cv.take<int2>((size_t)nw * stride);
-  unsigned long long *prog = cv.take<unsigned long long>(nw);
-  int *err = cv.take<int>(4);
-  LaneBest *wbest = cv.take<LaneBest>(nw);
-  int *end_h = cv.take<int>(4);
-  int64_t *d_base = cv.take<int64_t>(nstrips + 1);
+  char *d_split = cv.take<char>(space.bytes);
   FwdOut *d_fwd = cv.take<FwdOut>(1);
   uint32_t *d_one = cv.take<uint32_t>(16);  // order, lengths, offsets of the one-pair batch
   TbLayout *d_tbl = cv.take<TbLayout>(1);
@@ -106,7 +93,7 @@ filtr_status run_long(Ctx *c, const ScoreParams &sp, const filtr_params *params,
     return FILTR_ERR_NOMEM;
   }
   // host-side constants for the one-pair batch used by the walk
-  if (!c->ensure_host(4096 + (nstrips + 1) * 8)) return FILTR_ERR_NOMEM;
+  if (!c->ensure_host(4096)) return FILTR_ERR_NOMEM;
   char *h = reinterpret_cast<char *>(c->h_stage);
   uint32_t one[16] = {0, M, N};            // order[0] = 0, q_len = M, r_len = N
   TbLayout L{};
@@ -119,45 +106,36 @@ filtr_status run_long(Ctx *c, const ScoreParams &sp, const filtr_params *params,
   memcpy(h, one, sizeof one);
   memcpy(h + 64, &L, sizeof L);
   memcpy(h + 128, misc, sizeof misc);
-  memcpy(h + 256, base.data(), (nstrips + 1) * 8);
   cudaError_t e = cudaMemcpyAsync(d_one, h, sizeof one, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_tbl, h + 64, sizeof L, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_misc, h + 128, sizeof misc, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_base, h + 256, (nstrips + 1) * 8, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(prog, 0, nw * sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 16, st);
   if (e != cudaSuccess) return cuda_fail(e, "long-pair setup");
 
-  LongArgs a;
-  a.q = q;
-  a.r = r;
-  a.M = (int)M;
-  a.N = (int)N;
-  a.lo = (int)lo;
-  a.hi = (int)hi;
-  a.sp = sp;
-  a.ring = ring;
-  a.ring_stride = (uint32_t)stride;
-  a.prog = prog;
-  a.err = err;
-  a.timeout_ns = timeout_ns;
-  a.withhold = withhold;
-  a.tb = sp.traceback ? d_tb : nullptr;
-  a.strip_base = d_base;
-  a.wbest = wbest;
-  a.end_h = end_h;
+  const uint64_t *d_off = d_misc + 1;
+  const BatchDev b{q, r, d_off, d_off + 1, d_one + 1, d_one + 2};
+  SplitLaunch sl{};
+  sl.packed = false;
+  sl.R = R;
+  sl.count = 1;
+  sl.max_strips = nstrips;
+  sl.grid = grid;
+  sl.a.f.b = b;
+  sl.a.f.sp = sp;
+  sl.a.f.order = d_one;
+  sl.a.f.out = out;
+  sl.a.f.fwd = d_fwd;
+  sl.a.f.tb = d_tb;
+  sl.a.f.tbl = d_tbl;
+  sl.a.timeout_ns = timeout_ns;
+  sl.a.withhold = withhold;
+  split_bind(&sl.a, d_split, space, (uint32_t)stride);
+  const int *err = sl.a.err;
   c->span_begin(Ctx::PH_FORWARD, st);
-  e = launch_long(a, grid, st);
+  e = launch_split(sl, st);
   c->span_end(st);
   if (e != cudaSuccess) return cuda_fail(e, "long-pair kernel launch");
-  const uint64_t cells = band_cells(M, N, sp);
-  e = launch_long_finish(a, nw, cells, out, d_fwd, st);
-  if (e != cudaSuccess) return cuda_fail(e, "long-pair finish");
-  uint32_t launches = 2;
+  uint32_t launches = 3;
   if (sp.traceback && !withhold) {
-    const uint64_t *d_off = d_misc + 1;
-    BatchDev b{q, r, d_off, d_off + 1, d_one + 1, d_one + 2};
     WalkArgs wa;
     wa.b = b;
     wa.sp = sp;
@@ -430,7 +408,7 @@ filtr_status long_pair_async(Ctx *c, const ScoreParams &sp, const filtr_params *
   c->ev_used = 0;
   c->spans.clear();
   const filtr_status rc =
-      run_long(c, sp, params, q, M, r, N, out, cigar, cap, st, 0, LONG_TIMEOUT_NS, false);
+      run_long(c, sp, params, q, M, r, N, out, cigar, cap, st, 0, SPLIT_TIMEOUT_NS, false);
   if (!c->done_ev) cudaEventCreateWithFlags(&c->done_ev, cudaEventDisableTiming);
   if (c->done_ev) cudaEventRecord(c->done_ev, st);
   return rc;
@@ -504,7 +482,7 @@ filtr_status filtr_align_long(filtr_ctx *ctx, const filtr_params *params, const 
     c->xdrop_warps0 = w0;
     return rc;
   }
-  rc = run_long(c, sp, params, q, M, r, N, out, cigar, cigar_cap, st, 0, LONG_TIMEOUT_NS);
+  rc = run_long(c, sp, params, q, M, r, N, out, cigar, cigar_cap, st, 0, SPLIT_TIMEOUT_NS);
   if (!c->done_ev) cudaEventCreateWithFlags(&c->done_ev, cudaEventDisableTiming);
   if (c->done_ev) cudaEventRecord(c->done_ev, st);
   return rc;
@@ -535,6 +513,15 @@ filtr_status filtr_test_set_device_plan(filtr_ctx *ctx, int32_t mode) {
     return FILTR_ERR_INVALID;
   }
   reinterpret_cast<Ctx *>(ctx)->dev_plan_mode = mode;
+  return FILTR_OK;
+}
+
+filtr_status filtr_test_set_split(filtr_ctx *ctx, int32_t mode) {
+  if (!ctx || mode < 0 || mode > 2) {
+    set_error("filtr_test_set_split: bad arguments");
+    return FILTR_ERR_INVALID;
+  }
+  reinterpret_cast<Ctx *>(ctx)->split_mode = mode;
   return FILTR_OK;
 }
 

@@ -98,7 +98,7 @@ bool make_plan(const PlanInput &in, Plan *P) {
   // shape keys: 0..3 the int32 tiled kernel with R = 32, 24, 16, 8; 4..7 the
   // int16x2 tiled kernel with R = 32, 24, 16, 8; 8 the X-drop kernel
   const ShapeCost *costs = in.shape_cost ? in.shape_cost : kDefaultShapeCost;
-  const ShapeTable tab = make_shape_table(costs, sp);
+  const ShapeTable tab = make_shape_table(costs, sp, in.split);
   P->s_bucket.resize(n);
   P->s_shape.resize(n);
   P->s_words.resize(n);

@@ -53,6 +53,7 @@ struct PlanInput {
   int xdrop_slots;                // slots per lane of the X-drop kernel
   int xdrop_warps;                // first window width of X-drop pairs (warps), 0: estimated
   const ShapeCost *shape_cost = nullptr;  // nullptr: kDefaultShapeCost
+  int split = SPLIT_NONE;                 // shapes of pairs run a warp per strip
 };
 
 // First group width (warps) for X-drop / Z-drop pairs, from the expected width
@@ -88,6 +89,7 @@ struct DevPlanSummary {
   unsigned long long stage_words;   // sum of M + N + 1 (traceback on)
   unsigned long long cigar_upper;   // sum of M + N
   unsigned long long cells_packed;  // cells of the pairs given an int16x2 shape
+  unsigned long long tb_words_ref;  // traceback words of all pairs in ref_tab's shapes (use_ref)
 };
 
 // Zeroed before each call.  The host reads back bad[] and sum with one copy.
@@ -104,6 +106,8 @@ struct DevPlanArgs {
   uint32_t n;
   ScoreParams sp;
   ShapeTable tab;
+  ShapeTable ref_tab;   // with use_ref: other shapes, whose traceback words are summed too
+  int use_ref = 0;
   DevPlanState *state;
   uint16_t *key;        // per pair: shape * 64 + bucket
   uint64_t *words;      // per pair: traceback words

@@ -112,7 +112,16 @@ struct ShapeTable {
   int n_elig, n_elig_packed;
 };
 
-inline ShapeTable make_shape_table(const ShapeCost *costs, const ScoreParams &sp) {
+// Which shapes a batch may use when its pairs run a warp per strip (k_split.cuh):
+// the int32 tile of 8 rows, and the packed tile of 8 rows, of 16, or either.
+enum SplitShapes : int { SPLIT_NONE = 0, SPLIT_PACK8, SPLIT_PACK16, SPLIT_PACK8_16 };
+FILTR_HD bool split_shape_ok(int split, bool packed, int R) {
+  if (split == SPLIT_NONE) return true;
+  if (!packed) return R == 8;
+  return (R == 8 && split != SPLIT_PACK16) || (R == 16 && split != SPLIT_PACK8);
+}
+
+inline ShapeTable make_shape_table(const ShapeCost *costs, const ScoreParams &sp, int split = SPLIT_NONE) {
   ShapeTable t{};
   const bool pack_ok = !sp.use_band && !sp.use_xdrop && sp.precision != FILTR_PREC_I32;
   for (int k = 0; k < SHAPE_TILED; ++k) {
@@ -121,6 +130,7 @@ inline ShapeTable make_shape_table(const ShapeCost *costs, const ScoreParams &sp
     t.R[k] = costs[k].R;
     t.packed[k] = costs[k].packed ? 1 : 0;
     if (costs[k].packed && !pack_ok) continue;
+    if (!split_shape_ok(split, costs[k].packed, costs[k].R)) continue;
     t.elig[t.n_elig++] = k;
     t.n_elig_packed += costs[k].packed ? 1 : 0;
   }

@@ -1,0 +1,164 @@
+"""Tiled pairs with a warp per row strip (k_split.cuh) against the warp-per-pair
+kernels and the oracle, bit for bit: strip edges (256 and 512 rows), references
+from 1 column, bands whose strips start past the first column or hold no cell,
+pairs of very uneven height in one queue, both planners, the captured pipeline,
+and workspaces that leave no room for the hand-over slots."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+DNA_S = synth.dna_subst(2, -4)
+PROT_S = synth.protein_subst(np.random.default_rng(2))
+ROWS = [1, 255, 256, 257, 511, 512, 513, 769, 1024, 1025, 1300]
+COLS = [1, 2, 31, 32, 33, 63, 64, 65, 300, 700]
+
+
+@pytest.fixture(scope="module")
+def F():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2607_06225_gb300 as F
+
+    return F
+
+
+@pytest.fixture(scope="module")
+def ctx(F):
+    c = F.Context(0, 8 << 30)
+    yield c
+    F.lib().filtr_test_set_split(c.handle, 0)
+    c.close()
+
+
+def pairs(alphabet, seed, sizes):
+    rng = np.random.default_rng(seed)
+    qs, rs = [], []
+    for m, n in sizes:
+        r = rng.integers(0, alphabet, n).astype(np.uint8)
+        q = synth.mutate(rng, r, 0.1, 0.05, 0.05, 0.7, alphabet)[:m]
+        qs.append(np.concatenate([q, rng.integers(0, alphabet, m - len(q)).astype(np.uint8)]))
+        rs.append(r)
+    return synth.pack(qs, rs, alphabet, DNA_S if alphabet == 4 else PROT_S)
+
+
+def run(F, ctx, b, sc, mode, **kw):
+    assert F.lib().filtr_test_set_split(ctx.handle, mode) == F.OK
+    res, cig, rc = F.align_batch(ctx, F.make_params(b.subst, **sc), b, **kw)
+    assert rc == 0, F.last_error()
+    n = int(res["cigar_len"].sum()) if sc.get("traceback") else 0
+    return res, cig[:n]
+
+
+def same(a, b):
+    assert a[0].tobytes() == b[0].tobytes()
+    assert np.array_equal(a[1], b[1])
+
+
+KINDS = {
+    "global": dict(mode="global"),
+    "local": dict(mode="local"),
+    "global_linear": dict(mode="global", affine=False),
+    "local_linear": dict(mode="local", affine=False),
+    "band": dict(mode="global", band=20),
+    "band_local": dict(mode="local", band=40),
+    "band_literal": dict(mode="global", band=300, band_literal=True),
+    "int32": dict(mode="global", precision=1),
+}
+
+
+@pytest.mark.parametrize("alphabet", [4, 20])
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("kind", list(KINDS))
+def test_edges(F, ctx, kind, tb, alphabet):
+    sc = dict(dict(affine=True, gap_open=11 if alphabet == 20 else 4, gap_extend=2), **KINDS[kind],
+              traceback=tb)
+    b = pairs(alphabet, 5, [(m, n) for m in ROWS for n in COLS])
+    got = run(F, ctx, b, sc, 2)
+    same(got, run(F, ctx, b, sc, 1))
+    pick = list(range(0, b.n, 7))
+    osc = {k: v for k, v in sc.items() if k != "precision"}
+    ores = oracle.align_batch(b.subset(pick), **osc)[0]
+    assert np.array_equal(got[0]["score"][pick].astype(np.int64), ores["score"])
+    assert np.array_equal(got[0]["cells"][pick].astype(np.int64), ores["cells"])
+
+
+@pytest.mark.parametrize("n", [1, 2, 300, 700])
+@pytest.mark.parametrize("kind", ["local", "band"])
+def test_uneven_heights(F, ctx, n, kind):
+    """One tall pair among short ones; host (n < 256) and device plans, and both
+    packed strip heights."""
+    rng = np.random.default_rng(n)
+    sizes = [(6000, 5500)] + [(int(rng.integers(1, 900)), int(rng.integers(1, 900))) for _ in range(n - 1)]
+    sc = dict(dict(affine=True, gap_open=4, gap_extend=2, traceback=True), **KINDS[kind])
+    b = pairs(4, 6, sizes)
+    same(run(F, ctx, b, sc, 2), run(F, ctx, b, sc, 1))
+
+
+def test_both_widths(F, ctx):
+    """Pairs whose scores fit 15 bits beside pairs whose do not: two queues; the
+    tall ones have more strips than a warp has lanes."""
+    b = pairs(20, 7, [(700, 800)] * 5 + [(9000, 6000)] * 2 + [(300, 5000)] * 3)
+    sc = dict(mode="local", affine=True, gap_open=11, gap_extend=1, traceback=True)
+    same(run(F, ctx, b, sc, 2), run(F, ctx, b, sc, 1))
+
+
+@pytest.mark.parametrize("sc", [dict(mode="global", precision=1), dict(mode="local"),
+                                dict(mode="global", band=3000)])
+def test_many_strips_at_once(F, ctx, sc):
+    """One pair of 80 strips, all of them waiting in line from the start."""
+    sc = dict(dict(affine=True, gap_open=4, gap_extend=2, traceback=True), **sc)
+    b = pairs(4, 10, [(20400, 1500)])
+    same(run(F, ctx, b, sc, 2), run(F, ctx, b, sc, 1))
+
+
+def test_small_workspace(F):
+    """No room for the slots, or only for less traceback: the warp-per-pair form."""
+    b = pairs(4, 8, [(1100, 1000)] * 40)
+    sc = dict(mode="local", affine=True, gap_open=4, gap_extend=2, traceback=True)
+    big = F.Context(0, 1 << 30)
+    want = run(F, big, b, sc, 1)
+    big.close()
+    for ws in (3 << 20, 8 << 20, 24 << 20, 40 << 20):
+        small = F.Context(0, ws)
+        try:
+            same(run(F, small, b, sc, 2), want)
+        finally:
+            small.close()
+
+
+@pytest.mark.parametrize("kind", ["local", "band", "global"])
+def test_graph(F, ctx, kind):
+    sc = dict(dict(affine=True, gap_open=4, gap_extend=2, traceback=True), **KINDS[kind])
+    for n, room in ((40, 1 << 30), (900, 2 << 30)):
+        rng = np.random.default_rng(n)
+        b = pairs(4, 9, [(int(rng.integers(0, 1000)), int(rng.integers(0, 1000))) for _ in range(n)])
+        want = run(F, ctx, b, sc, 1)
+        for mode in (0, 2):
+            F.lib().filtr_test_set_split(ctx.handle, mode)
+            g = F.Graph(ctx, F.make_params(b.subst, **sc), n + 3, 1000, room)
+            for _ in range(2):
+                res, cig, st = F.graph_align(g, b)
+                assert st == F.OK
+                same((res, cig[:int(res["cigar_len"].sum())]), want)
+            sub = b.subset([n // 2])
+            res, cig, st = F.graph_align(g, sub)
+            same((res, cig[:int(res["cigar_len"].sum())]), run(F, ctx, sub, sc, 1))
+            g.close()
+
+
+def test_tall_pair_in_a_batch(F, ctx):
+    """300 unbanded pairs of a few hundred rows and one of 5000: the default rule
+    plans them again, a warp per strip."""
+    rng = np.random.default_rng(11)
+    sizes = [(5000, 4000)] + [(int(rng.integers(100, 400)), int(rng.integers(100, 400))) for _ in range(300)]
+    sc = dict(mode="local", affine=True, gap_open=11, gap_extend=1, traceback=True)
+    b = pairs(20, 12, sizes)
+    got = run(F, ctx, b, sc, 0)
+    assert ctx.last_stats()["device_plan"] == 0
+    same(got, run(F, ctx, b, sc, 1))

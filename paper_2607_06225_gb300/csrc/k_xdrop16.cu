@@ -1,6 +1,6 @@
 // k_xdrop16.cu -- the X-drop instances of the packed antidiagonal sweep
-// (k_xdrop16_impl.cuh).
-#include "k_xdrop16_impl.cuh"
+// (k_sweep16_impl.cuh).
+#include "k_sweep16_impl.cuh"
 
 namespace filtr {
 

@@ -1,7 +1,7 @@
 // k_zdrop16.cu -- the Z-drop instances of the packed antidiagonal sweep
-// (k_xdrop16_impl.cuh), in a translation unit of their own so the two sets
+// (k_sweep16_impl.cuh), in a translation unit of their own so the two sets
 // compile in parallel.
-#include "k_xdrop16_impl.cuh"
+#include "k_sweep16_impl.cuh"
 
 namespace filtr {
 

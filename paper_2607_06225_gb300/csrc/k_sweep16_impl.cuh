@@ -77,16 +77,13 @@ constexpr int X16_C0 = 16384;
 constexpr int X16_BLOCK = 16;  // antidiagonals per block (8 of each phase)
 constexpr uint32_t X16_K80 = 0x80008000u;
 
-struct alignas(16) Edge16 {
-  uint32_t x, o;  // phase A reads the next thread's (Fn, Ho), phase B the previous thread's (En, Ho)
-  uint32_t pad[2];
-};
-
 template <int W>
 struct alignas(16) X16Shared {
-  int red[2][W][4];  // per warp: max H (packed), lowest live slot, highest live slot, slot of the max
-  Edge16 first[2][W];
-  Edge16 last[2][W];
+  int4 red[2][W];       // per warp: max H (packed), lowest live slot, highest live slot, slot of the max
+  // a warp's edge values, [0] its first thread's (Fn, Ho), which the warp before
+  // reads in phase A, [1] its last thread's (En, Ho), which the warp after reads in phase B
+  uint2 edge[2][W][2];
+  int tmp[2][W];
   uint32_t pair;
   unsigned long long rsv;
   uint4 move[W > 1 ? W * 32 : 1];  // state on its way to other threads
@@ -158,6 +155,8 @@ enum : int { X16_GO = 0, X16_END, X16_WIDE, X16_OVF };  // how a step ended
 template <int W, int G, bool LOCAL, bool TB, bool ZD, bool UNI>
 struct Sweep16 {
   static constexpr int S = 8 * G, P = 4 * G, WIN = W * 32 * S, ROW = WIN / 8;
+  // a fast step needs k and c itself (else a fast block counts them as a whole)
+  static constexpr bool STEP_K = LOCAL || ZD || W > 1 || !UNI;
   // parameters of the pair and the thread
   X16Shared<W> &sh;
   const int8_t *s_sub;
@@ -181,6 +180,7 @@ struct Sweep16 {
   int bv, bi, bj;      // best cell so far
   int k;               // the last antidiagonal
   uint64_t cells;
+  int span;            // sum of ph - pl over the steps of a fast block
   int cornerH;
   bool corner;
 
@@ -236,14 +236,43 @@ struct Sweep16 {
 
   // the last antidiagonal's reductions over the group's warps
   __device__ __forceinline__ void combine() {
-    if constexpr (W > 1) {
-      const int nb = k & 1;
-      const int v0 = lane < W ? sh.red[nb][lane][0] : 0;
-      b2 = (uint32_t)__reduce_max_sync(X16_FULL, (unsigned)v0);
-      pl = __reduce_min_sync(X16_FULL, lane < W ? sh.red[nb][lane][1] : INT_MAX);
-      ph = __reduce_max_sync(X16_FULL, lane < W ? sh.red[nb][lane][2] : INT_MIN);
-      if (need_bs) pbs = __reduce_max_sync(X16_FULL, (lane < W && (uint32_t)v0 == b2) ? sh.red[nb][lane][3] : -1);
+    const int nb = k & 1;
+    if constexpr (W > 1 && W <= 4) {  // a few warps: one broadcast load each, no warp reductions
+      int4 v[W];
+#pragma unroll
+      for (int x = 0; x < W; ++x) v[x] = sh.red[nb][x];
+      int best = v[0].x, l = v[0].y, h = v[0].z;
+#pragma unroll
+      for (int x = 1; x < W; ++x) {
+        best = max(best, v[x].x);
+        l = min(l, v[x].y);
+        h = max(h, v[x].z);
+      }
+      b2 = (uint32_t)best;
+      pl = l;
+      ph = h;
+      if (need_bs) {
+        int s = -1;
+#pragma unroll
+        for (int x = 0; x < W; ++x)
+          if (v[x].x == best) s = max(s, v[x].w);
+        pbs = s;
+      }
+    } else if constexpr (W > 4) {
+      const int4 v = lane < W ? sh.red[nb][lane] : make_int4(0, INT_MAX, INT_MIN, -1);
+      b2 = (uint32_t)__reduce_max_sync(X16_FULL, v.x);
+      pl = __reduce_min_sync(X16_FULL, v.y);
+      ph = __reduce_max_sync(X16_FULL, v.z);
+      if (need_bs) pbs = __reduce_max_sync(X16_FULL, (uint32_t)v.x == b2 ? v.w : -1);
     }
+  }
+  // this warp's reductions and edge values of antidiagonal k, for the others
+  __device__ __forceinline__ void publish() {
+    const int nb = k & 1;
+    if (lane == 0) sh.red[nb][warp] = make_int4((int)b2, pl, ph, pbs);
+    if (lane == 0 || lane == 31)
+      sh.edge[nb][warp][lane & 1] = make_uint2(lane ? En[P - 1] : Fn[0], lane ? Ho[P - 1] : Ho[0]);
+    __syncthreads();
   }
   // the group's largest slot whose H equals the best (smallest row)
   __device__ __forceinline__ int best_slot_of(const uint32_t (&H)[P], uint32_t best2) const {
@@ -295,12 +324,18 @@ struct Sweep16 {
       }
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        const uint32_t t = (qw[g] ^ rw[g]) + 0x33333333u;  // bit 2 of a nibble: codes differ
-#pragma unroll
-        for (int rq = 0; rq < 4; ++rq) {
-          const uint32_t ne = x16_halfmask(t * (1u << (13 - 4 * rq)));
-          s2[4 * g + rq] = (ne & MI2) | (~ne & MA2);
-        }
+        // bit 3 of a nibble: codes differ.  An odd slot's is a byte's sign, so one byte
+        // permute spreads a register's two flags; a shift brings the even slots' there
+        const uint32_t t1 = (qw[g] ^ rw[g]) + 0x77777777u, t0 = t1 << 4;
+        uint32_t n0, n1, n2, n3;
+        asm("prmt.b32 %0, %1, 0, 0xaa88;" : "=r"(n0) : "r"(t0));
+        asm("prmt.b32 %0, %1, 0, 0xaa88;" : "=r"(n1) : "r"(t1));
+        asm("prmt.b32 %0, %1, 0, 0xbb99;" : "=r"(n2) : "r"(t0));
+        asm("prmt.b32 %0, %1, 0, 0xbb99;" : "=r"(n3) : "r"(t1));
+        s2[4 * g] = (n0 & MI2) | (~n0 & MA2);
+        s2[4 * g + 1] = (n1 & MI2) | (~n1 & MA2);
+        s2[4 * g + 2] = (n2 & MI2) | (~n2 & MA2);
+        s2[4 * g + 3] = (n3 & MI2) | (~n3 & MA2);
       }
     } else {
       if (PH == 0) {
@@ -349,18 +384,18 @@ struct Sweep16 {
       if (PH == 0) {
         nx = __shfl_down_sync(X16_FULL, Fn[0], 1);
         no = __shfl_down_sync(X16_FULL, Ho[0], 1);
-        if (lane == 31) {
-          const bool in = W > 1 && warp < W - 1;
-          nx = in ? sh.first[buf][in ? warp + 1 : 0].x : 0u;
-          no = in ? sh.first[buf][in ? warp + 1 : 0].o : 0u;
+        if ((SLOW || W > 1) && lane == 31) {  // (in a fast block the last thread of one warp is dead)
+          const uint2 v = W > 1 && warp < W - 1 ? sh.edge[buf][warp + 1][0] : make_uint2(0u, 0u);
+          nx = v.x;
+          no = v.y;
         }
       } else {
         nx = __shfl_up_sync(X16_FULL, En[P - 1], 1);
         no = __shfl_up_sync(X16_FULL, Ho[P - 1], 1);
-        if (lane == 0) {
-          const bool in = W > 1 && warp > 0;
-          nx = in ? sh.last[buf][in ? warp - 1 : 0].x : 0u;
-          no = in ? sh.last[buf][in ? warp - 1 : 0].o : 0u;
+        if ((SLOW || W > 1) && lane == 0) {
+          const uint2 v = W > 1 && warp > 0 ? sh.edge[buf][warp - 1][1] : make_uint2(0u, 0u);
+          nx = v.x;
+          no = v.y;
         }
       }
       uint32_t nib[G];
@@ -426,13 +461,14 @@ struct Sweep16 {
 
     // ---- antidiagonal k: its reductions, and what k + 1 takes from them --------------
     combine();
-    if (b2 == 0) return X16_END;  // nothing alive on k: the sweep ends there
+    // nothing alive on k: the sweep ends there (in a fast block pl is then above every ol)
+    if ((SLOW || LOCAL || ZD || W > 1) && b2 == 0) return X16_END;
     settle(Hp);
     if (xrun) brun2 = max(brun2, b2);
     if (SLOW && k == M + N) corner = true;
     const int kk = k + 1, cn = c + (PH == 0 ? 1 : 0);
     int low = PH == 0 ? pl - 1 : pl, high = PH == 0 ? ph : ph + 1;  // the candidate slots
-    bool cut = LOCAL || ol < low || oh > high;
+    const bool cut = SLOW || LOCAL || ol < low || oh > high;
     if (SLOW) {
       const int jA = max(max(0, kk - M), max(cn + low, (kk + band_lo + 1) >> 1));
       const int jB = min(min(N, kk), min(cn + high, (kk + band_hi) >> 1));
@@ -446,15 +482,14 @@ struct Sweep16 {
       if (bp > pceil || tmin < pfloor) return X16_OVF;
       const int a0 = max(jA, 1), b0 = min(jB, kk - 1);
       cells += (uint64_t)max(b0 - a0 + 1, 0);
-      cut = true;
-    } else {
-      cells += (uint32_t)(high - low + 1);
     }
-    ol = pl;
-    oh = ph;
     // ---- prune k + 1 -----------------------------------------------------------------
     const uint32_t K = CX2 - (xrun ? brun2 : b2);  // 0x8000 - threshold in each half
     uint32_t t2 = 0, am = 0;
+    if (cut && !(SLOW || LOCAL || ZD || W > 1) && b2 == 0) return X16_END;
+    if (!SLOW) span += ph - pl;  // high - low + 1 = ph - pl + 2 cells
+    ol = pl;
+    oh = ph;
     if (!idle) {
       if (cut) {
         const int vA = low - base_slot, vB = high - base_slot;
@@ -496,8 +531,10 @@ struct Sweep16 {
       t2 = __vimax_s16x2_relu(t2, __byte_perm(t2, t2, 0x1032));
     }
     // ---- reductions of k + 1 (consumed after the next raw update) -----------------------
-    k = kk;
-    c = cn;
+    if (SLOW || STEP_K) {
+      k = kk;
+      c = cn;
+    }
     b2 = __reduce_max_sync(X16_FULL, t2);
     pl = __reduce_min_sync(X16_FULL, am ? base_slot + __ffs(am) - 1 : INT_MAX);
     ph = __reduce_max_sync(X16_FULL, am ? base_slot + 31 - __clz(am) : INT_MIN);
@@ -514,22 +551,7 @@ struct Sweep16 {
         cornerH = v ? v - X16_C0 + base : NEG;
       }
     }
-    if constexpr (W > 1) {
-      const int nb = k & 1;
-      if (lane == 0) {
-        sh.red[nb][warp][0] = (int)b2;
-        sh.red[nb][warp][1] = pl;
-        sh.red[nb][warp][2] = ph;
-        sh.red[nb][warp][3] = pbs;
-        sh.first[nb][warp].x = Fn[0];
-        sh.first[nb][warp].o = Ho[0];
-      }
-      if (lane == 31) {
-        sh.last[nb][warp].x = En[P - 1];
-        sh.last[nb][warp].o = Ho[P - 1];
-      }
-      __syncthreads();
-    }
+    if constexpr (W > 1) publish();
     return X16_GO;
   }
 
@@ -581,23 +603,11 @@ struct Sweep16 {
       ol -= t * S;
       oh -= t * S;
     }
-    if constexpr (W > 1) {  // the next step reads its neighbours' edges and the warps' reductions
-      const int nb = k & 1;
+    if constexpr (W > 1) {
+      // the next step reads its neighbours' edges and the warps' reductions (the
+      // group's values stand for each warp's: they are combined again)
       __syncthreads();
-      if (lane == 0) {
-        // the group's values stand for each warp's: they are combined again
-        sh.red[nb][warp][0] = (int)b2;
-        sh.red[nb][warp][1] = pl;
-        sh.red[nb][warp][2] = ph;
-        sh.red[nb][warp][3] = pbs;
-        sh.first[nb][warp].x = Fn[0];
-        sh.first[nb][warp].o = Ho[0];
-      }
-      if (lane == 31) {
-        sh.last[nb][warp].x = En[P - 1];
-        sh.last[nb][warp].o = Ho[P - 1];
-      }
-      __syncthreads();
+      publish();
     }
   }
 };
@@ -826,8 +836,10 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
         }
       }
       if (LOCAL) w.Z2 = x16_splat(min(max(X16_C0 - w.base, 0), 0x7fff));
-      // eight slots of room on each side (a block moves an end by 8), and the new codes
-      constexpr int ROOM = X16_BLOCK / 2 + 2;
+      // room on each side (a block moves an end by 8 slots), and the new codes
+      // (in one-warp groups the first and last thread stay dead besides: a fast
+      // step does not clear the edge values that wrap around to them)
+      constexpr int ROOM = X16_BLOCK / 2 + 1 + (W == 1 ? S : 1);
       if (w.pl < ROOM || w.ph > WIN - 1 - ROOM) {
         const int mid = (w.pl + w.ph) >> 1;
         const int t = (mid - WIN / 2) / S;
@@ -871,12 +883,22 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
                         dlo >= w.band_lo && dhi <= w.band_hi && bp + 9 * w.smax <= w.pceil &&
                         rp - w.X - (ZD ? max(dhi, w.dbest) - min(dlo, w.dbest) : 0) - X16_BLOCK * w.oe >= w.pfloor;
       if (fast) {
+        w.span = 0;
+        int x = 0;
 #pragma unroll 1
-        for (int x = 0; x < X16_BLOCK / 2; ++x) {
+        for (; x < X16_BLOCK; x += 2) {
           stop = w.template step<0, false>(w.Ha, w.Hb);
           if (stop != X16_GO) break;
           stop = w.template step<1, false>(w.Hb, w.Ha);
-          if (stop != X16_GO) break;
+          if (stop != X16_GO) {
+            ++x;
+            break;
+          }
+        }
+        w.cells += (uint64_t)(uint32_t)(w.span + 2 * x);
+        if (!SW::STEP_K) {
+          w.k += x;
+          w.c += (x + 1) >> 1;
         }
       } else {
         int x = phase_b ? 1 : 0;
@@ -936,10 +958,10 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
       int ch = __reduce_max_sync(X16_FULL, cornerH);
       if (W > 1) {
         __syncthreads();
-        if (lane == 0) sh.red[1][w.warp][0] = ch;
+        if (lane == 0) sh.tmp[0][w.warp] = ch;
         __syncthreads();
         ch = INT_MIN;
-        for (int x = 0; x < W; ++x) ch = max(ch, sh.red[1][x][0]);
+        for (int x = 0; x < W; ++x) ch = max(ch, sh.tmp[0][x]);
       }
       cornerH = ch;
     }
@@ -965,13 +987,13 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
       if (W > 1) {
         __syncthreads();
         if (lane == 0) {
-          sh.red[0][w.warp][0] = used;
-          sh.red[0][w.warp][1] = first;
+          sh.tmp[0][w.warp] = used;
+          sh.tmp[1][w.warp] = first;
         }
         __syncthreads();
         for (int x = 0; x < W; ++x) {
-          used = max(used, sh.red[0][x][0]);
-          first = min(first, sh.red[0][x][1]);
+          used = max(used, sh.tmp[0][x]);
+          first = min(first, sh.tmp[1][x]);
         }
       }
       const int drop = first == INT_MAX ? 0 : first >> 3;  // eight-slot threads
@@ -1077,13 +1099,12 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
 }
 // Group widths: W = 1 (256 slots) runs one warp per pair (8 slots per thread,
 // four pairs per 128-thread block).  W = 2 (512 slots) runs one warp of 16-slot
-// threads for batched pairs, where the bookkeeping done once per warp and the
-// absence of block barriers pay, and two warps of 8-slot threads for the
-// segments of one long pair (a.ck), where the shorter chain of two half-loaded
-// warps gives the lower latency per antidiagonal.  The traceback rows and the
-// checkpoint records of W = 2 are the same in either form: thread t of the
-// one-warp group writes words 2t and 2t + 1.  W >= 4 runs W warps of 8-slot
-// threads.
+// threads: bookkeeping done once per warp and no block barriers.  (Two warps of
+// 8-slot threads have half the cell work each, but exchanging edges and
+// reductions every antidiagonal costs more: the megabase pair's forward took
+// 670 ms that way, 601 ms on one warp.)  The traceback rows and the checkpoint
+// records are those of 8-slot threads: thread t of the one-warp group writes
+// words 2t and 2t + 1.  W >= 4 runs W warps of 8-slot threads.
 template <int KW, int G, bool LOCAL, bool TB, bool ZD>
 cudaError_t x16_launch(const FullArgs &a, int grid, uint32_t *ovf, uint32_t *novf, X16Knobs kn,
                        cudaStream_t s) {
@@ -1125,8 +1146,7 @@ cudaError_t x16_launch_any(const FullArgs &a, int W, int grid, uint32_t *ovf, ui
                            cudaStream_t s) {
   switch (W) {
     case 1: return x16_dispatch<1, 1, ZD>(a, grid, ovf, novf, kn, s);
-    case 2: return a.ck ? x16_dispatch<2, 1, ZD>(a, grid, ovf, novf, kn, s)
-                        : x16_dispatch<1, 2, ZD>(a, grid, ovf, novf, kn, s);
+    case 2: return x16_dispatch<1, 2, ZD>(a, grid, ovf, novf, kn, s);
     case 4: return x16_dispatch<4, 1, ZD>(a, grid, ovf, novf, kn, s);
     case 8: return x16_dispatch<8, 1, ZD>(a, grid, ovf, novf, kn, s);
     case 16: return x16_dispatch<16, 1, ZD>(a, grid, ovf, novf, kn, s);

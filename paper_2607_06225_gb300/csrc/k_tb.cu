@@ -8,6 +8,8 @@
 // or column 0 finish with the forced gap.  A scan then places every pair's
 // CIGAR in pair order and a warp per pair copies it forward into the caller's
 // buffer.
+#include <climits>
+
 #include "filtr_internal.h"
 #include "k_xdrop_layout.h"
 
@@ -21,18 +23,24 @@ struct FullGeom {
   bool band;
   int64_t lo, hi;
   int64_t base;   // first word of strip `s`
-  int s;          // current strip
+  int s;          // current strip (or one past the last)
   int64_t jlo;    // first column of strip s
   int64_t nsteps; // steps of strip s
 };
 
 __device__ __forceinline__ void geom_seek(FullGeom &g, int s) {
-  // strips are visited upward only; move `base` from strip g.s to strip s
-  while (g.s > s) {
-    --g.s;
+  while (g.s != s) {  // move `base` strip by strip
     int64_t jl, jh;
-    strip_cols((int64_t)g.s * g.HS, g.HS, g.M, g.N, g.band, g.lo, g.hi, &jl, &jh);
-    g.base -= strip_tb_words(jl, jh, g.R);
+    if (g.s < s) {
+      strip_cols((int64_t)g.s * g.HS, g.HS, g.M, g.N, g.band, g.lo, g.hi, &jl, &jh);
+      g.base += strip_tb_words(jl, jh, g.R);
+      ++g.s;
+      strip_cols((int64_t)g.s * g.HS, g.HS, g.M, g.N, g.band, g.lo, g.hi, &jl, &jh);
+    } else {
+      --g.s;
+      strip_cols((int64_t)g.s * g.HS, g.HS, g.M, g.N, g.band, g.lo, g.hi, &jl, &jh);
+      g.base -= strip_tb_words(jl, jh, g.R);
+    }
     g.jlo = jl;
     g.nsteps = jh >= jl ? (jh - jl + 1) + 31 : 0;
   }
@@ -64,9 +72,8 @@ __device__ __forceinline__ void geom_init(FullGeom &g, int R, int M, int N, cons
   }
 }
 
-// Choice bits of cell (i, j) of an int32 tile (banded or not).  The cursor g
-// only moves up, so successive calls on one cursor must ask for rows that do
-// not increase.
+// Choice bits of cell (i, j) of an int32 tile (banded or not).  Successive calls
+// on one cursor should ask for rows near each other.
 __device__ __forceinline__ uint32_t full_bits(const uint32_t *tb, FullGeom &g, int i, int j) {
   const int s = (i - 1) / g.HS;
   geom_seek(g, s);
@@ -98,17 +105,6 @@ __device__ __forceinline__ uint32_t pack_bits(const uint32_t *tb, const PackGeom
   const int c = k & 7;
   return (((w >> c) & 1u) << 3) | (((w >> (8 + c)) & 1u) << 2) | (((w >> (16 + c)) & 1u) << 1) |
          ((w >> (24 + c)) & 1u);
-}
-
-// Choice bits of cell (i, j) of an unbanded int32 tile: every strip has N + 31
-// steps of R / 8 words per lane.
-__device__ __forceinline__ uint32_t full_bits_unbanded(const uint32_t *tb, int R, int N, int i,
-                                                       int j) {
-  const int HS = 32 * R, s = (i - 1) / HS, rho = (i - 1) - s * HS;
-  const int l = rho / R, k = rho - l * R, wps = R / 8;
-  const int64_t t = (int64_t)j - 1 + l;
-  const int64_t base = (int64_t)s * strip_tb_words(1, N, R);
-  return tb_nibble(__ldg(tb + base + (t * wps + (k >> 3)) * 32 + l), k);
 }
 
 struct Emitter {
@@ -243,199 +239,174 @@ __global__ void k_walk(const WalkArgs a) {
   walk_thread(a, gd ? gd->b : a.b, gd ? gd->out : a.out, a.order[t]);
 }
 
-// ---- warp walks over the antidiagonal (X-drop) layout ------------------------
-// The walk itself is serial, and one thread per pair spends it waiting on two
-// dependent loads per step (the window origin c_k, then the traceback word).
-// A warp prefetches instead: from the current cell (i0, j0) on antidiagonal
-// k0, lane L loads c of antidiagonal k0 - L and the words holding the slots a
-// path from (i0, j0) can reach there -- every step lowers i + j by 1 or 2 and
-// j by at most 1, so on k0 - L the path's column lies in [j0 - L, j0]: at most
-// 32 slots, 5 words.  Lane 0 then walks through shared memory until the path
-// leaves the 32 cached antidiagonals, and the warp refills.
-
-constexpr int XW = 5;  // cached words per antidiagonal
+// ---- warp walks ----------------------------------------------------------------
+// The walk is serial, and one thread per pair spends it waiting on a dependent
+// load per step.  A warp keeps a band of choice bits on chip instead: 32 rows
+// (iw - 31 .. iw) by the eight diagonals d0 - 4 .. d0 + 3 around the path, lane x
+// loading the eight cells of row iw - x.  While the path crosses these rows the
+// next 32 are already being loaded, around the diagonal the path entered this
+// window on (and for the antidiagonal layout, whose words are found through the
+// window origins, the origins of the rows after those).  A path that drifts off
+// the band is loaded again around where it is.
+//
+// The state of the walk is the same in every lane.  A run of diagonal steps (matches and
+// mismatches, H taken from the diagonal) is taken in one go: lane d looks at the
+// cell d steps down the diagonal, a ballot finds where the run ends (a gap, row or
+// column 0, the band's edge, or for local alignments the first cell of value 0,
+// found by a warp scan of the scores), and another tells '=' from 'X'.  A gap's
+// extension bits are looked at the same way, along the row or the column.
+//
+// Measured against windows of 32 antidiagonals loaded when the path enters them
+// (antidiagonal layout) and three cached lines of 32 cells (tiles), walked by lane
+// 0 but for the diagonal runs: see the figures at launch_walk.
 
 struct WalkCore {
   const uint8_t *q, *r;
   const int8_t *subst;
   int A, e, oe;
-  bool local;
+  bool local, mid;  // mid: a gap that opened leaves through a diagonal step (state 3)
   int i, j, v, state;
-  Emitter em;
-  bool mid = false;  // Table 1's M/I/D: a gap that opened leaves through a diagonal step (state 3)
+  uint32_t *st;     // staged ops
+  uint32_t n, run;  // ops staged; length of the op being grown
+  int cur;
+  __device__ __forceinline__ void put(int op, uint32_t len) {
+    if (op == cur) {
+      run += len;
+    } else {
+      flush();
+      cur = op;
+      run = len;
+    }
+  }
+  __device__ __forceinline__ void flush() {
+    if (cur >= 0) {
+      if ((threadIdx.x & 31) == 0) st[n] = (run << 4) | (uint32_t)cur;
+      ++n;
+    }
+    cur = -1;
+  }
+  __device__ __forceinline__ void store(filtr_result *res) {  // the finished walk
+    flush();
+    if ((threadIdx.x & 31) == 0) {
+      res->q_begin = i;
+      res->r_begin = j;
+      res->cigar_len = n;
+    }
+  }
 };
 
-// One step of the walk (those of k_walk): 1 when the alignment's start is
-// reached, 2 when the current cell's antidiagonal is <= k_stop or < k_low or
-// its bits are not cached (state kept), else 0.  Codes gives the residue codes
-// of the diagonal steps (cached by the warp beside the bits).
-template <class Bits, class Codes>
-__device__ __forceinline__ int walk_step(WalkCore &w, const Bits &bits, int64_t k_stop, int64_t k_low,
-                                         const Codes &codes) {
-  if (w.state == 0) {
-    if ((w.i == 0 && w.j == 0) || (w.local && w.v == 0)) return 1;
-    if (w.i == 0) {
-      w.em.put(OP_D, (uint32_t)w.j);
-      w.j = 0;
-      return 1;
-    }
-    if (w.j == 0) {
-      w.em.put(OP_I, (uint32_t)w.i);
-      w.i = 0;
-      return 1;
-    }
-  }
-  const int64_t k = (int64_t)w.i + w.j;
-  if (k <= k_stop || k < k_low) return 2;
-  if (w.state == 0) {
-    const uint32_t nib = bits(w.i, w.j);
-    if (nib > 15u) return 2;  // not cached: the warp refills around (i, j)
-    if (nib & TB_PF) {
-      w.state = 2;
-    } else if (nib & TB_PE) {
-      w.state = 1;
-    } else {
-      const int qc = codes.q(w, w.i), rc = codes.r(w, w.j);
-      w.em.put(qc == rc ? OP_EQ : OP_X, 1);
-      w.v -= w.subst[qc * w.A + rc];
-      --w.i;
-      --w.j;
-    }
-  } else if (w.state == 1) {
-    if (w.j == 0) {
-      w.state = 0;
-      return 0;
-    }
-    const uint32_t nib = bits(w.i, w.j);
-    if (nib > 15u) return 2;
-    w.em.put(OP_D, 1);
-    if (nib & TB_EEXT) {
-      w.v += w.e;
-    } else {
-      w.v += w.oe;
-      w.state = w.mid ? 3 : 0;
-    }
-    --w.j;
-  } else if (w.state == 2) {
-    if (w.i == 0) {
-      w.state = 0;
-      return 0;
-    }
-    const uint32_t nib = bits(w.i, w.j);
-    if (nib > 15u) return 2;
-    w.em.put(OP_I, 1);
-    if (nib & TB_FEXT) {
-      w.v += w.e;
-    } else {
-      w.v += w.oe;
-      w.state = w.mid ? 3 : 0;
-    }
-    --w.i;
-  } else {  // state 3: the gap opened from M here, so this cell is a diagonal step
-    if (w.i == 0 && w.j == 0) return 1;
-    const int qc = codes.q(w, w.i), rc = codes.r(w, w.j);
-    w.em.put(qc == rc ? OP_EQ : OP_X, 1);
-    w.v -= w.subst[qc * w.A + rc];
-    --w.i;
-    --w.j;
-    w.state = 0;
-  }
-  return 0;
+__device__ __forceinline__ WalkCore walk_core(const WalkArgs &a, const BatchDev &b, uint32_t p, const int8_t *subst) {
+  WalkCore w;
+  w.q = b.q_seq + b.q_off[p];
+  w.r = b.r_seq + b.r_off[p];
+  w.subst = subst;
+  w.A = a.sp.alphabet;
+  w.e = a.sp.e;
+  w.oe = a.sp.o + a.sp.e;
+  w.local = a.sp.mode == FILTR_LOCAL;
+  w.mid = a.sp.mid != 0;
+  w.st = a.stage + a.stage_off[p];
+  w.n = w.run = 0;
+  w.cur = -1;
+  w.state = 0;
+  return w;
 }
 
-// Walks until the alignment's start is reached (returns true), or until the
-// current cell's antidiagonal is <= k_stop or < k_low or its bits are not
-// cached (returns false, state kept), with the whole warp (every lane calls
-// it; w is lane 0's).  A
-// run of diagonal steps (matches and mismatches, H taken from the diagonal) is
-// taken in one go: lane d looks at the cell d steps down the diagonal, a ballot
-// finds where the run ends (a gap, row or column 0, the window's edge, or for
-// local alignments the first cell of value 0), a warp scan gives the value
-// change, and lane 0 emits the run's '=' / 'X' ops.  Lane 0 walks the other
-// steps alone.
-template <class Bits, class Codes>
-__device__ __forceinline__ bool walk_coop(WalkCore &w, const Bits &bits, int64_t k_stop,
-                                          int64_t k_low, const Codes &codes) {
-  constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  for (;;) {
-    const int i = __shfl_sync(FULL, w.i, 0), j = __shfl_sync(FULL, w.j, 0);
-    const int v = __shfl_sync(FULL, w.v, 0), st = __shfl_sync(FULL, w.state, 0);
-    if (st == 0) {
-      const int ii = i - lane, jj = j - lane;
-      const int64_t kk = (int64_t)ii + jj;
-      bool ok = ii >= 1 && jj >= 1 && kk > k_stop && kk >= k_low;
-      int qc = 0, rc = 1, sc = 0;
-      if (ok) {
-        ok = (bits(ii, jj) & (TB_PE | TB_PF)) == 0u;
-        qc = codes.q(w, ii);
-        rc = codes.r(w, jj);
-        sc = w.subst[qc * w.A + rc];
-      }
-      int pre = sc;  // inclusive scan of the scores down the diagonal
+constexpr int WB = 8;       // diagonals of the band
+constexpr int WB_MID = 4;   // the path's diagonal when the band is loaded around it
+struct WalkBand {
+  uint8_t nb[32][WB];       // choice bits: row iw - x, diagonal d0 - WB_MID + y
+  int32_t c[96];            // antidiagonal layout: origins of kc, kc - 1, ...
+};
+
+// Loaders keep the raw words of one window in registers between issue() and
+// commit().
+//
+// Tiled layouts: a word of each cell of the lane's row.
+struct TileLoader {
+  const uint32_t *tb;
+  bool pk, fb;
+  PackGeom pg;
+  FullGeom g;    // banded int32 tiles: this lane's strip cursor
+  int R, M, N;
+  int s, row0;   // this lane's strip and its first row (0-based)
+  uint32_t raw[WB];
+  int sub;       // the cells' place in their words
+  __device__ __forceinline__ void start(WalkBand &, int, int) {}
+  __device__ __forceinline__ void ahead(WalkBand &, int, int) {}
+  __device__ __forceinline__ void issue(WalkBand &, int iw, int d0) {
+    const int i = iw - (int)(threadIdx.x & 31), j0 = i + d0 - WB_MID;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(FULL, pre, o);
-        if (lane >= o) pre += t;
+    for (int y = 0; y < WB; ++y) raw[y] = 0;
+    if (i < 1) return;
+    const int HS = 32 * R;
+    while (i <= row0) row0 -= HS, --s;  // the rows move a window at a time
+    while (i > row0 + HS) row0 += HS, ++s;
+    const int rho = i - 1 - row0, l = rho * ((1 << 20) / R + 1) >> 20, k = rho - l * R;  // rho / R, rho < 1024
+    int64_t at;
+    int stride, steps, t;
+    if (pk) {
+      const int P = R >> 1, h = k >= P ? 1 : 0, kk = k - h * P, G = (P + 7) >> 3;
+      t = j0 - 1 + 2 * l + h;
+      at = (int64_t)s * pg.strip_words + (h * G + (kk >> 3)) * 32 + l;
+      stride = 64 * G;
+      steps = N + 63;
+      sub = kk & 7;
+    } else {
+      int64_t base;
+      int jlo = 1;
+      steps = N + 31;
+      if (fb) {
+        geom_seek(g, s);
+        base = g.base;
+        jlo = (int)g.jlo;
+        steps = (int)g.nsteps;
+      } else {
+        base = (int64_t)s * strip_tb_words(1, N, R);
       }
-      if (w.local && v - (pre - sc) == 0) ok = false;  // the value at cell d
-      const unsigned okm = __ballot_sync(FULL, ok);
-      const int L = (okm == FULL) ? 32 : __ffs(~okm) - 1;
-      if (L > 0) {
-        const unsigned eqm = __ballot_sync(FULL, qc == rc);
-        const int dv = __shfl_sync(FULL, pre, L - 1);
-        if (lane == 0) {
-          int d = 0;
-          while (d < L) {
-            const unsigned rest = eqm >> d;
-            const bool eq = (rest & 1u) != 0u;
-            const unsigned stop = eq ? ~rest : rest;
-            const int len = min(stop ? __ffs(stop) - 1 : 32 - d, L - d);
-            w.em.put(eq ? OP_EQ : OP_X, (uint32_t)len);
-            d += len;
-          }
-          w.v -= dv;
-          w.i -= L;
-          w.j -= L;
-        }
-        continue;
-      }
+      t = j0 - jlo + l;
+      at = base + (k >> 3) * 32 + l;
+      stride = 4 * R;
+      sub = 4 * (7 - (k & 7));
     }
-    int r = 0;
-    if (lane == 0) r = walk_step(w, bits, k_stop, k_low, codes);
-    r = __shfl_sync(FULL, r, 0);
-    if (r == 1) return true;
-    if (r == 2) return false;
+    const uint32_t *w = tb + at + (int64_t)t * stride;
+    if (j0 >= 1 && j0 + WB - 1 <= N && t >= 0 && t + WB - 1 < steps) {
+#pragma unroll
+      for (int y = 0; y < WB; ++y) raw[y] = __ldg(w + y * stride);
+    } else {
+#pragma unroll
+      for (int y = 0; y < WB; ++y)
+        if (j0 + y >= 1 && j0 + y <= N && t + y >= 0 && t + y < steps) raw[y] = __ldg(w + y * stride);
+    }
   }
-}
-
-struct XdCache {
-  uint32_t w[32 * XW];
-  int32_t c[32], b[32];
-  // the 32 query / reference codes below the window's first cell (i0, j0):
-  // qc[x] = q[i0 - 1 - x], rc[x] = r[j0 - 1 - x] (a walk inside the window
-  // steps diagonally only from cells with i > i0 - 32, j > j0 - 32)
-  uint8_t qc[32], rc[32];
-  int32_t i0, j0;
+  __device__ __forceinline__ void commit(WalkBand &C) {
+    uint32_t lo = 0, hi = 0;
+#pragma unroll
+    for (int y = 0; y < WB; ++y) {
+      const uint32_t x = raw[y] >> sub;
+      const uint32_t nib = pk ? ((x & 1u) << 3) | ((x >> 8 & 1u) << 2) | ((x >> 16 & 1u) << 1) | (x >> 24 & 1u)
+                              : x & 15u;
+      if (y < 4)
+        lo |= nib << (8 * y);
+      else
+        hi |= nib << (8 * (y - 4));
+    }
+    __syncwarp();  // the last window's readers are done
+    *reinterpret_cast<uint2 *>(C.nb[threadIdx.x & 31]) = make_uint2(lo, hi);
+    __syncwarp();
+  }
 };
-struct XdCacheCodes {
-  const XdCache *C;
-  __device__ int q(const WalkCore &, int i) const { return C->qc[C->i0 - i]; }
-  __device__ int r(const WalkCore &, int j) const { return C->rc[C->j0 - j]; }
-};
 
-// Where antidiagonal k's window origin and traceback row live.
+// Where antidiagonal k's window origin and traceback row live (antidiagonals stay
+// below 2^31).  run(k): row k's words, with those of the rows around it in the
+// range (lo, hi] at multiples of wpk.
 struct XdRows {  // one pair's own layout or a recomputed segment: row = k - row_off
   const int32_t *ck;
   const uint32_t *tb;
-  int wpk;
-  int64_t row_off;
-  __device__ void at(int64_t k, int &c, const uint32_t *&row, int &w) const {
-    const int64_t i = k - row_off;
-    c = __ldg(ck + i);
-    row = tb + i * wpk;
-    w = wpk;
-  }
+  int wpk, row_off;
+  int lo, hi;
+  __device__ __forceinline__ int origin(int k) const { return __ldg(ck + (k - row_off)); }
+  __device__ __forceinline__ const uint32_t *run(int k) { return tb + (int64_t)(k - row_off) * wpk; }
 };
 struct XdPoolRows {  // single-pass segmented sweep: segment s = (k - 1) / C
   const uint32_t *pool;
@@ -443,60 +414,252 @@ struct XdPoolRows {  // single-pass segmented sweep: segment s = (k - 1) / C
   const uint64_t *seg_off;
   const int32_t *seg_w;
   int C;
-  __device__ void at(int64_t k, int &c, const uint32_t *&row, int &w) const {
-    const int km = (int)(k - 1);  // antidiagonals stay below 2^31
-    const int s = km / C, i = km - s * C;
-    w = xd_words_per_k(__ldg(seg_w + s), 8);
-    c = __ldg(seg_ck_all + (int64_t)s * C + i);
-    row = pool + __ldg(seg_off + s) + (int64_t)i * w;
+  int wpk, lo, hi;  // the segment looked up last
+  const uint32_t *base;
+  __device__ __forceinline__ int origin(int k) const { return __ldg(seg_ck_all + (k - 1)); }
+  __device__ __forceinline__ const uint32_t *run(int k) {
+    if (k <= lo || k > hi) {
+      const int s = (k - 1) / C;
+      wpk = xd_words_per_k(__ldg(seg_w + s), 8);
+      base = pool + __ldg(seg_off + s);
+      lo = s * C;
+      hi = lo + C;
+    }
+    return base + (int64_t)(k - 1 - lo) * wpk;
   }
 };
 
-// All lanes: cache antidiagonals k0 - lane (those > k_min) around column j0,
-// and the residue codes the walk reads below (i0, j0).
+// Antidiagonal layout: the word of cell (i, j) sits in the row of antidiagonal
+// i + j, at the slot the row's origin tells.  The origins of a window's 70
+// antidiagonals (and eight on each side, for a band loaded a few diagonals off)
+// are loaded one window earlier than its words.
 template <class Rows>
-__device__ __forceinline__ void xd_fill(XdCache &C, const Rows &rows, int64_t k0, int j0,
-                                        int64_t k_min, const WalkCore &w) {
-  const int lane = threadIdx.x & 31;
-  const int i0 = (int)(k0 - j0);
-  C.qc[lane] = (i0 - 1 - lane >= 0) ? w.q[i0 - 1 - lane] : 0;
-  C.rc[lane] = (j0 - 1 - lane >= 0) ? w.r[j0 - 1 - lane] : 0;
-  if (lane == 0) {
-    C.i0 = i0;
-    C.j0 = j0;
-  }
-  const int64_t kk = k0 - lane;
-  if (kk > k_min) {
-    int c, wpk;
-    const uint32_t *row;
-    rows.at(kk, c, row, wpk);
-    const int plo = max(j0 - lane - c, 0), phi = j0 - c;
-    const int w0 = plo >> 3, w1 = min(phi >> 3, wpk - 1);
+struct XdLoader {
+  Rows rows;
+  int k_min, k_max;  // antidiagonals that have a row: k_min < k <= k_max
+  int cn[3];         // origins on their way: kn, kn - 1, ... (lane + 32 z)
+  int kn, kc;        // top of cn; top of the band's c
+  uint32_t raw[WB];
+  uint32_t sub;      // 4 bits per cell: its slot within its word
+  __device__ __forceinline__ void load_origins(int iw, int d0) {
+    kn = 2 * iw + d0 + (WB - 1 - WB_MID) + 8;
 #pragma unroll
-    for (int x = 0; x < XW; ++x)
-      if (w0 + x <= w1) C.w[lane * XW + x] = __ldg(row + w0 + x);
-    C.c[lane] = c;
-    C.b[lane] = w0;
+    for (int z = 0; z < 3; ++z) {
+      const int k = kn - (int)(threadIdx.x & 31) - 32 * z;
+      cn[z] = k > k_min && k <= k_max ? rows.origin(k) : 0;
+    }
   }
-  __syncwarp();
+  __device__ __forceinline__ void store_origins(WalkBand &C) {
+    __syncwarp();
+#pragma unroll
+    for (int z = 0; z < 3; ++z) C.c[(threadIdx.x & 31) + 32 * z] = cn[z];
+    kc = kn;
+    __syncwarp();
+  }
+  // the first window of a band at (iw, d0): its origins, waited for
+  __device__ __forceinline__ void start(WalkBand &C, int iw, int d0) {
+    load_origins(iw, d0);
+    store_origins(C);
+  }
+  // the window after the one about to be issued at (iw, d0)
+  __device__ __forceinline__ void ahead(WalkBand &C, int iw, int d0) { load_origins(iw, d0); }
+  __device__ __forceinline__ void issue(WalkBand &C, int iw, int d0) {
+    const int i = iw - (int)(threadIdx.x & 31), j0 = i + d0 - WB_MID, k0 = i + j0, x0 = kc - k0;
+    sub = 0;
+    // (the bounds on x0 always hold: a band is issued at most 3 diagonals off its origins)
+    if (i >= 1 && j0 >= 1 && k0 > k_min && k0 + WB - 1 <= k_max && x0 >= WB - 1 && x0 < 96) {
+      const uint32_t *row = rows.run(k0);
+      const bool one = k0 > rows.lo && k0 + WB - 1 <= rows.hi;
+#pragma unroll
+      for (int y = 0; y < WB; ++y) {
+        if (!one && y) row = rows.run(k0 + y);
+        const int p = j0 + y - C.c[x0 - y];
+        raw[y] = (unsigned)p < 8u * (unsigned)rows.wpk ? __ldg(row + (p >> 3)) : 0u;
+        sub |= (uint32_t)(p & 7) << (4 * y);
+        row += rows.wpk;
+      }
+    } else {
+#pragma unroll
+      for (int y = 0; y < WB; ++y) {
+        const int j = j0 + y, k = k0 + y, x = x0 - y;
+        raw[y] = 0;
+        if (i >= 1 && j >= 1 && k > k_min && k <= k_max && x >= 0 && x < 96) {
+          const uint32_t *row = rows.run(k);
+          const int p = j - C.c[x];
+          if ((unsigned)p < 8u * (unsigned)rows.wpk) raw[y] = __ldg(row + (p >> 3));
+          sub |= (uint32_t)(p & 7) << (4 * y);
+        }
+      }
+    }
+  }
+  __device__ __forceinline__ void commit(WalkBand &C) {
+    uint32_t lo = 0, hi = 0;
+#pragma unroll
+    for (int y = 0; y < WB; ++y) {
+      const uint32_t nib = raw[y] >> (28 - 4 * (sub >> (4 * y) & 7u)) & 15u;
+      if (y < 4)
+        lo |= nib << (8 * y);
+      else
+        hi |= nib << (8 * (y - 4));
+    }
+    __syncwarp();  // the last window's readers are done
+    *reinterpret_cast<uint2 *>(C.nb[threadIdx.x & 31]) = make_uint2(lo, hi);
+    __syncwarp();
+  }
+};
+template <class L>
+struct WalkAhead {  // a window's origins must be stored before its words are issued
+  static __device__ __forceinline__ void next(L &ld, WalkBand &C, int iw, int d0) { ld.issue(C, iw, d0); }
+};
+template <class Rows>
+struct WalkAhead<XdLoader<Rows>> {
+  static __device__ __forceinline__ void next(XdLoader<Rows> &ld, WalkBand &C, int iw, int d0) {
+    ld.store_origins(C);
+    ld.issue(C, iw, d0);
+    ld.ahead(C, iw - 32, d0);
+  }
+};
+
+// Walks until the alignment's start is reached (true), or until the current cell
+// is on antidiagonal k_stop or before (false, state kept).
+template <class L>
+__device__ __forceinline__ bool walk_band(WalkCore &w, L &ld, WalkBand &C, int k_stop) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  int iw = 0, d0 = 0, dn = 0;  // this window; the diagonal the next is issued around
+  bool open = false;
+  for (;;) {
+    if (w.state == 0) {
+      if ((w.i == 0 && w.j == 0) || (w.local && w.v == 0)) return true;
+      if (w.i == 0) {
+        w.put(OP_D, (uint32_t)w.j);
+        w.j = 0;
+        return true;
+      }
+      if (w.j == 0) {
+        w.put(OP_I, (uint32_t)w.i);
+        w.i = 0;
+        return true;
+      }
+    }
+    if (w.i + w.j <= k_stop) return false;
+    if (w.state == 1 && w.j == 0) {
+      w.state = 0;
+      continue;
+    }
+    if (w.state == 2 && w.i == 0) {
+      w.state = 0;
+      continue;
+    }
+    if (w.state == 3) {  // the gap opened from M here, so this cell is a diagonal step
+      if (w.i == 0 && w.j == 0) return true;
+      const int qc = w.q[w.i - 1], rc = w.r[w.j - 1];
+      w.put(qc == rc ? OP_EQ : OP_X, 1);
+      w.v -= w.subst[qc * w.A + rc];
+      --w.i;
+      --w.j;
+      w.state = 0;
+      continue;
+    }
+    // ---- the window that holds (i, j) ---------------------------------------------
+    int x0 = iw - w.i, y0 = w.j - w.i - d0 + WB_MID;
+    if (!open || x0 >= 32 || y0 < 0 || y0 >= WB) {
+      const int d = w.j - w.i, yn = d - dn + WB_MID;
+      if (open && x0 == 32 && yn >= 1 && yn < WB - 1) {  // the next one, on its way since this one was entered
+        iw -= 32;
+        d0 = dn;
+      } else {
+        iw = w.i;
+        d0 = d;
+        ld.start(C, iw, d0);
+        ld.issue(C, iw, d0);
+        ld.ahead(C, iw - 32, d);
+        open = true;
+      }
+      ld.commit(C);
+      dn = d;
+      WalkAhead<L>::next(ld, C, iw - 32, d);
+      if (lane < 2) {  // the residues of the rows after those
+        const uint8_t *s = lane ? w.r + w.j : w.q + w.i;
+        if ((lane ? w.j : w.i) > 192) asm volatile("prefetch.global.L1 [%0];" ::"l"(s - 192));
+      }
+      x0 = iw - w.i;
+      y0 = d - d0 + WB_MID;
+    }
+    if (w.state == 0) {  // a run down the diagonal
+      const int ii = w.i - lane, jj = w.j - lane;
+      bool ok = ii >= 1 && jj >= 1 && ii + jj > k_stop && x0 + lane < 32;
+      uint32_t nib = 0;
+      int qc = 0, rc = 1, sc = 0;
+      if (ok) {
+        nib = C.nb[x0 + lane][y0];
+        ok = (nib & (TB_PE | TB_PF)) == 0u;
+        qc = __ldg(w.q + ii - 1);
+        rc = __ldg(w.r + jj - 1);
+      }
+      int dv = 0;
+      if (w.local) {
+        if (ok) sc = w.subst[qc * w.A + rc];
+        int pre = sc;  // inclusive scan of the scores down the diagonal
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(FULL, pre, o);
+          if (lane >= o) pre += t;
+        }
+        if (w.v - (pre - sc) == 0) ok = false;  // the value at cell d
+        dv = pre;
+      }
+      const unsigned okm = __ballot_sync(FULL, ok);
+      const int n = okm == FULL ? 32 : __ffs(~okm) - 1;
+      if (n > 0) {
+        const unsigned eqm = __ballot_sync(FULL, qc == rc);
+        if (w.local) w.v -= __shfl_sync(FULL, dv, n - 1);
+        int d = 0;
+        while (d < n) {
+          const unsigned rest = eqm >> d;
+          const bool eq = (rest & 1u) != 0u;
+          const unsigned stop = eq ? ~rest : rest;
+          const int len = min(stop ? __ffs(stop) - 1 : 32 - d, n - d);
+          w.put(eq ? OP_EQ : OP_X, (uint32_t)len);
+          d += len;
+        }
+        w.i -= n;
+        w.j -= n;
+        continue;
+      }
+      nib = __shfl_sync(FULL, nib, 0);
+      w.state = nib & TB_PF ? 2 : 1;
+    }
+    // ---- a gap: lane t looks at its t-th residue's extension bit --------------------
+    const bool down = w.state == 2;  // along the column (query residues), else the row
+    const int ii = down ? w.i - lane : w.i, jj = down ? w.j : w.j - lane;
+    const int x = down ? x0 + lane : x0, y = down ? y0 + lane : y0 - lane;
+    const bool in = ii >= 1 && jj >= 1 && ii + jj > k_stop && x < 32 && y >= 0 && y < WB;
+    const bool ext = in && (C.nb[in ? x : 0][in ? y : 0] & (down ? TB_FEXT : TB_EEXT)) != 0u;
+    const unsigned extm = __ballot_sync(FULL, ext), inm = __ballot_sync(FULL, in);
+    const int n = extm == FULL ? 32 : __ffs(~extm) - 1;    // residues that extend
+    const bool opens = n < 32 && (inm >> n & 1u) != 0u;   // and then one that opens the gap
+    const int len = n + (opens ? 1 : 0);
+    if (len > 0) w.put(down ? OP_I : OP_D, (uint32_t)len);
+    w.v += n * w.e + (opens ? w.oe : 0);
+    if (down)
+      w.i -= len;
+    else
+      w.j -= len;
+    if (opens) w.state = w.mid ? 3 : 0;
+  }
 }
 
-struct XdCacheBits {
-  const XdCache *C;
-  int64_t k0;
-  __device__ uint32_t operator()(int ii, int jj) const {
-    const int L = (int)(k0 - ((int64_t)ii + jj));
-    const int p = jj - C->c[L];
-    return tb_nibble(C->w[L * XW + (p >> 3) - C->b[L]], p);
-  }
-};
+__device__ __forceinline__ void load_subst(int8_t *s_sub, const ScoreParams &sp) {
+  for (int x = threadIdx.x; x < sp.alphabet * sp.alphabet; x += blockDim.x) s_sub[x] = sp.subst[x];
+  __syncthreads();
+}
 
 // One warp per pair of a batched X-drop call (4 pairs per 128-thread block).
 __global__ void __launch_bounds__(128) k_walk_xdw(const WalkArgs a) {
-  __shared__ XdCache cache[4];
+  __shared__ WalkBand band[4];
   __shared__ int8_t s_sub[MAX_ALPHA * MAX_ALPHA];
-  for (int x = threadIdx.x; x < a.sp.alphabet * a.sp.alphabet; x += blockDim.x) s_sub[x] = a.sp.subst[x];
-  __syncthreads();
+  load_subst(s_sub, a.sp);
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t t = blockIdx.x * 4 + wib;
   if (t >= a.n_order) return;
@@ -509,82 +672,24 @@ __global__ void __launch_bounds__(128) k_walk_xdw(const WalkArgs a) {
   }
   const int M = (int)a.b.q_len[p], N = (int)a.b.r_len[p];
   const uint32_t *base = a.tb + L.off;
-  const int32_t *ck = reinterpret_cast<const int32_t *>(base);
-  const uint32_t *tbw = base + xd_origin_words(M, N);
-  const int wpk = xd_words_per_k(L.warps, L.R);
-  WalkCore w{a.b.q_seq + a.b.q_off[p], a.b.r_seq + a.b.r_off[p], s_sub, a.sp.alphabet,
-             a.sp.e, a.sp.o + a.sp.e, a.sp.mode == FILTR_LOCAL, f.end_i, f.end_j, f.score, 0,
-             Emitter{a.stage + a.stage_off[p], 0, -1, 0}, a.sp.mid != 0};
-  XdCache &C = cache[wib];
-  bool done = false;
-  for (;;) {
-    const int i0 = __shfl_sync(0xffffffffu, w.i, 0), j0 = __shfl_sync(0xffffffffu, w.j, 0);
-    if (__shfl_sync(0xffffffffu, (int)done, 0)) break;
-    const int64_t k0 = (int64_t)i0 + j0;
-    xd_fill(C, XdRows{ck, tbw, wpk, 0}, k0, j0, 0, w);
-    done = walk_coop(w, XdCacheBits{&C, k0}, -1, k0 - 31, XdCacheCodes{&C});
-    __syncwarp();
-  }
-  if (lane == 0) {
-    w.em.flush();
-    filtr_result *res = a.out + p;
-    res->q_begin = w.i;
-    res->r_begin = w.j;
-    res->cigar_len = w.em.n;
-  }
+  WalkCore w = walk_core(a, a.b, p, s_sub);
+  w.i = f.end_i;
+  w.j = f.end_j;
+  w.v = f.score;
+  XdLoader<XdRows> ld;
+  ld.rows = XdRows{reinterpret_cast<const int32_t *>(base), base + xd_origin_words(M, N),
+                   xd_words_per_k(L.warps, L.R), 0, INT_MIN, INT_MAX};
+  ld.k_min = 0;
+  ld.k_max = w.i + w.j;
+  walk_band(w, ld, band[wib], -1);
+  w.store(a.out + p);
 }
 
-// ---- warp walk over the tiled layouts ---------------------------------------
-// One thread per pair waits on one dependent load per step.  A warp instead
-// caches, from the current cell (i0, j0), the choice bits of three lines of 32
-// cells: the diagonal (i0 - d, j0 - d), the row (i0, j0 - d) and the column
-// (i0 - d, j0) -- lane d loads its three words at once.  Matches and
-// mismatches follow the diagonal, a gap the row or the column, so lane 0 walks
-// from the cache until the path leaves all three lines (a gap's start or end),
-// and the warp refills there: about two refills per gap instead of a load per
-// step.  Runs of diagonal steps along the cached diagonal are taken by the
-// whole warp (walk_coop), with the 32 codes below (i0, j0) cached beside the
-// bits.  In a banded int32 tile the strips' offsets depend on the band, so
-// every lane keeps two strip cursors: one for row i0 and one for row i0 - d.
-// Both rows never increase from one refill to the next, and a cursor only
-// moves up.
-
-struct TileCache {
-  uint8_t d[32], row[32], col[32];
-  // qc[x] = q[i0 - 1 - x], rc[x] = r[j0 - 1 - x]: the codes of the diagonal
-  // line's cells (and of the row's and the column's)
-  uint8_t qc[32], rc[32];
-  int32_t i0, j0;
-};
-struct TileCacheCodes {  // cached codes; cells further from (i0, j0) read the sequences
-  const TileCache *C;
-  __device__ int q(const WalkCore &w, int i) const {
-    const int x = C->i0 - i;
-    return x < 32 ? C->qc[x] : w.q[i - 1];
-  }
-  __device__ int r(const WalkCore &w, int j) const {
-    const int x = C->j0 - j;
-    return x < 32 ? C->rc[x] : w.r[j - 1];
-  }
-};
-
-struct TileCacheBits {
-  const TileCache *C;
-  int i0, j0;
-  __device__ uint32_t operator()(int ii, int jj) const {
-    const int di = i0 - ii, dj = j0 - jj;
-    if (di == dj && di < 32) return C->d[di];
-    if (di == 0 && dj < 32) return C->row[dj];
-    if (dj == 0 && di < 32) return C->col[di];
-    return 0xffu;  // not cached
-  }
-};
-
+// One warp per pair over the tiled layouts.
 __global__ void __launch_bounds__(128) k_walk_tw(const WalkArgs a) {
-  __shared__ TileCache cache[4];
+  __shared__ WalkBand band[4];
   __shared__ int8_t s_sub[MAX_ALPHA * MAX_ALPHA];
-  for (int x = threadIdx.x; x < a.sp.alphabet * a.sp.alphabet; x += blockDim.x) s_sub[x] = a.sp.subst[x];
-  __syncthreads();
+  load_subst(s_sub, a.sp);
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t t = blockIdx.x * 4 + wib;
   const GraphDesc *gd = a.gd;  // captured pipeline: batch, outputs and count from here
@@ -599,56 +704,28 @@ __global__ void __launch_bounds__(128) k_walk_tw(const WalkArgs a) {
     if (lane == 0) walk_thread(a, b, out, p);  // empty pairs
     return;
   }
-  const bool fb = !pk && a.sp.use_band;
   const FwdOut f = a.fwd[p];
   if (f.status != FILTR_ST_OK && f.status != FILTR_ST_DROPPED) {
     if (lane == 0) out[p].cigar_len = 0;
     return;
   }
-  const int N = (int)b.r_len[p];
-  const uint32_t *tb = a.tb + L.off;
-  const PackGeom pg{L.R, (int64_t)pack_strip_tb_words(1, N, L.R)};
-  WalkCore w{b.q_seq + b.q_off[p], b.r_seq + b.r_off[p], s_sub, a.sp.alphabet,
-             a.sp.e, a.sp.o + a.sp.e, a.sp.mode == FILTR_LOCAL, f.end_i, f.end_j, f.score, 0,
-             Emitter{a.stage + a.stage_off[p], 0, -1, 0}, a.sp.mid != 0};
-  TileCache &C = cache[wib];
-  bool done = false;
-  FullGeom g_row, g_lane;  // banded int32 tiles: cursors for rows i0 and i0 - lane
-  if (fb) {
-    geom_init(g_row, L.R, (int)b.q_len[p], N, a.sp);
-    g_lane = g_row;
-  }
-  auto cell = [&](FullGeom &g, int ii, int jj) -> uint8_t {
-    if (ii < 1 || jj < 1) return 0;
-    if (pk) return (uint8_t)pack_bits(tb, pg, ii, jj);
-    if (fb) return (uint8_t)full_bits(tb, g, ii, jj);
-    return (uint8_t)full_bits_unbanded(tb, L.R, N, ii, jj);
-  };
-  for (;;) {
-    const int i0 = __shfl_sync(0xffffffffu, w.i, 0), j0 = __shfl_sync(0xffffffffu, w.j, 0);
-    if (__shfl_sync(0xffffffffu, (int)done, 0)) break;
-    const uint8_t cr = cell(g_row, i0, j0 - lane), cd = cell(g_lane, i0 - lane, j0 - lane),
-                  cc = cell(g_lane, i0 - lane, j0);
-    C.d[lane] = cd;
-    C.row[lane] = cr;
-    C.col[lane] = cc;
-    C.qc[lane] = (i0 - 1 - lane >= 0) ? w.q[i0 - 1 - lane] : 0;
-    C.rc[lane] = (j0 - 1 - lane >= 0) ? w.r[j0 - 1 - lane] : 0;
-    if (lane == 0) {
-      C.i0 = i0;
-      C.j0 = j0;
-    }
-    __syncwarp();
-    done = walk_coop(w, TileCacheBits{&C, i0, j0}, -1, INT64_MIN, TileCacheCodes{&C});
-    __syncwarp();
-  }
-  if (lane == 0) {
-    w.em.flush();
-    filtr_result *res = out + p;
-    res->q_begin = w.i;
-    res->r_begin = w.j;
-    res->cigar_len = w.em.n;
-  }
+  WalkCore w = walk_core(a, b, p, s_sub);
+  w.i = f.end_i;
+  w.j = f.end_j;
+  w.v = f.score;
+  TileLoader ld;
+  ld.tb = a.tb + L.off;
+  ld.pk = pk;
+  ld.fb = !pk && a.sp.use_band;
+  ld.R = L.R;
+  ld.M = (int)b.q_len[p];
+  ld.N = (int)b.r_len[p];
+  ld.s = 0;
+  ld.row0 = 0;
+  ld.pg = PackGeom{L.R, (int64_t)pack_strip_tb_words(1, ld.N, L.R)};
+  if (ld.fb) geom_init(ld.g, L.R, ld.M, ld.N, a.sp);
+  walk_band(w, ld, band[wib], -1);
+  w.store(out + p);
 }
 
 // Resumable walk over one recomputed segment (antidiagonals (k_start, k_end])
@@ -657,82 +734,65 @@ __global__ void __launch_bounds__(128) k_walk_tw(const WalkArgs a) {
 // when the alignment's start is reached.
 __global__ void k_walk_segw(const WalkArgs a, const uint32_t *seg_tb, const int32_t *seg_ck,
                             int k_start, int wpk, WalkState *ws) {
-  __shared__ XdCache C;
+  __shared__ WalkBand band;
   __shared__ int8_t s_sub[MAX_ALPHA * MAX_ALPHA];
-  for (int x = threadIdx.x; x < a.sp.alphabet * a.sp.alphabet; x += blockDim.x) s_sub[x] = a.sp.subst[x];
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
+  load_subst(s_sub, a.sp);
   if (blockIdx.x != 0 || threadIdx.x >= 32) return;
   const WalkState st = *ws;
   if (st.done) return;
   const uint32_t p = a.order[0];
-  WalkCore w{a.b.q_seq + a.b.q_off[p], a.b.r_seq + a.b.r_off[p], s_sub, a.sp.alphabet,
-             a.sp.e, a.sp.o + a.sp.e, a.sp.mode == FILTR_LOCAL, st.i, st.j, st.v, st.state,
-             Emitter{a.stage + a.stage_off[p], st.n, st.cur, st.run}, a.sp.mid != 0};
-  bool done = false;
-  for (;;) {
-    const int i0 = __shfl_sync(0xffffffffu, w.i, 0), j0 = __shfl_sync(0xffffffffu, w.j, 0);
-    const bool d = __shfl_sync(0xffffffffu, (int)done, 0) != 0;
-    const int64_t k0 = (int64_t)i0 + j0;
-    if (d || k0 <= k_start) break;
-    xd_fill(C, XdRows{seg_ck, seg_tb, wpk, (int64_t)k_start + 1}, k0, j0, k_start, w);
-    done = walk_coop(w, XdCacheBits{&C, k0}, k_start, k0 - 31, XdCacheCodes{&C});
-    __syncwarp();
-  }
-  if (lane == 0) {
-    if (done) {
-      w.em.flush();
-      filtr_result *res = a.out + p;
-      res->q_begin = w.i;
-      res->r_begin = w.j;
-      res->cigar_len = w.em.n;
-    }
+  WalkCore w = walk_core(a, a.b, p, s_sub);
+  w.i = st.i;
+  w.j = st.j;
+  w.v = st.v;
+  w.state = st.state;
+  w.n = st.n;
+  w.cur = st.cur;
+  w.run = st.run;
+  XdLoader<XdRows> ld;
+  ld.rows = XdRows{seg_ck, seg_tb, wpk, k_start + 1, INT_MIN, INT_MAX};
+  ld.k_min = k_start;
+  ld.k_max = w.i + w.j;
+  // (a walk in a gap stops on k_start as well; 0 is the start itself)
+  const bool done = walk_band(w, ld, band, k_start > 0 ? k_start : -1);
+  __syncwarp();
+  if (done) w.store(a.out + p);
+  if (threadIdx.x == 0) {
     WalkState o;
     o.i = w.i;
     o.j = w.j;
     o.v = w.v;
     o.state = w.state;
     o.done = done ? 1 : 0;
-    o.n = w.em.n;
-    o.cur = w.em.cur;
-    o.run = w.em.run;
+    o.n = w.n;
+    o.cur = w.cur;
+    o.run = w.run;
     *ws = o;
   }
 }
 
 // The whole traceback of a single-pass segmented sweep; one warp.
 __global__ void k_walk_poolw(const WalkArgs a, const XdPoolRows rows) {
-  __shared__ XdCache C;
+  __shared__ WalkBand band;
   __shared__ int8_t s_sub[MAX_ALPHA * MAX_ALPHA];
-  for (int x = threadIdx.x; x < a.sp.alphabet * a.sp.alphabet; x += blockDim.x) s_sub[x] = a.sp.subst[x];
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
+  load_subst(s_sub, a.sp);
   if (blockIdx.x != 0 || threadIdx.x >= 32) return;
   const uint32_t p = a.order[0];
   const FwdOut f = a.fwd[p];
   if (f.status != FILTR_ST_OK && f.status != FILTR_ST_DROPPED) {
-    if (lane == 0) a.out[p].cigar_len = 0;
+    if (threadIdx.x == 0) a.out[p].cigar_len = 0;
     return;
   }
-  WalkCore w{a.b.q_seq + a.b.q_off[p], a.b.r_seq + a.b.r_off[p], s_sub, a.sp.alphabet,
-             a.sp.e, a.sp.o + a.sp.e, a.sp.mode == FILTR_LOCAL, f.end_i, f.end_j, f.score, 0,
-             Emitter{a.stage + a.stage_off[p], 0, -1, 0}, a.sp.mid != 0};
-  bool done = false;
-  for (;;) {
-    const int i0 = __shfl_sync(0xffffffffu, w.i, 0), j0 = __shfl_sync(0xffffffffu, w.j, 0);
-    if (__shfl_sync(0xffffffffu, (int)done, 0)) break;
-    const int64_t k0 = (int64_t)i0 + j0;
-    xd_fill(C, rows, k0, j0, 0, w);
-    done = walk_coop(w, XdCacheBits{&C, k0}, -1, k0 - 31, XdCacheCodes{&C});
-    __syncwarp();
-  }
-  if (lane == 0) {
-    w.em.flush();
-    filtr_result *res = a.out + p;
-    res->q_begin = w.i;
-    res->r_begin = w.j;
-    res->cigar_len = w.em.n;
-  }
+  WalkCore w = walk_core(a, a.b, p, s_sub);
+  w.i = f.end_i;
+  w.j = f.end_j;
+  w.v = f.score;
+  XdLoader<XdPoolRows> ld;
+  ld.rows = rows;
+  ld.k_min = 0;
+  ld.k_max = w.i + w.j;
+  walk_band(w, ld, band, -1);
+  w.store(a.out + p);
 }
 
 // Exclusive scan of cigar_len (pair order) into offs; *total = sum.  One CTA.
@@ -807,10 +867,12 @@ cudaError_t launch_walk(const WalkArgs &a, cudaStream_t s) {
   if (a.n_order == 0) return cudaSuccess;
   // A warp per pair keeps more loads in flight for each pair but issues the
   // serial walk as a whole warp's instructions.  Up to about one warp per resident
-  // slot of the device (and some) it is the faster form: 4096 protein pairs of
-  // 100-1000 through the captured pipeline 3.3 -> 1.85 ms, 512 banded reads' walk
-  // about 27 -> 6 ms.  With many more pairs a thread per pair (32 pairs per
-  // instruction stream) is: 2.5 ms against 3.4 ms for 100,000 protein pairs.
+  // slot of the device (and some) it is the faster form; with many more pairs a
+  // thread per pair (32 pairs per instruction stream) is: 2.5 ms against 3.4 ms
+  // for 100,000 protein pairs.  The band windows of walk_band took the walk of 64
+  // protein pairs from 0.17 to 0.10 ms, of 512 banded reads from 6.2 (a thread
+  // per pair: about 27) to 2.1, of an 80 kbp banded pair from 21.3 to 7.4, of a
+  // megabase X-drop pair from 144 to 54 and of 10,000 long reads from 17.2 to 14.5.
   if (a.n_order <= WALK_WARP_PAIRS)
     k_walk_tw<<<(a.n_order + 3) / 4, 128, 0, s>>>(a);
   else
@@ -827,7 +889,7 @@ cudaError_t launch_walk_xd(const WalkArgs &a, cudaStream_t s) {
 
 cudaError_t launch_walk_pool(const WalkArgs &a, const uint32_t *pool, const int32_t *seg_ck_all,
                              const uint64_t *seg_off, const int32_t *seg_w, int C, cudaStream_t s) {
-  k_walk_poolw<<<1, 32, 0, s>>>(a, XdPoolRows{pool, seg_ck_all, seg_off, seg_w, C});
+  k_walk_poolw<<<1, 32, 0, s>>>(a, XdPoolRows{pool, seg_ck_all, seg_off, seg_w, C, 0, 0, 0, nullptr});
   return cudaGetLastError();
 }
 

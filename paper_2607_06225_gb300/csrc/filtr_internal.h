@@ -219,7 +219,8 @@ struct FullArgs {
   uint32_t strip_stride;
   uint32_t max_n;          // 0, or the longest reference the strip buffers hold
   uint32_t max_m;          // 0, or the longest query accepted
-  const struct XdCkpt *ck; // X-drop kernel: checkpoint mode (nullptr = normal)
+  const struct XdCkpt *ck; // X-drop kernel: checkpoint mode (nullptr = normal): n_ck descriptors
+  uint32_t n_ck = 1;
   // packed X-drop sweep: pairs that left the 16-bit range (rerun in int32),
   // and the base move distance (<= 0: never, a test hook)
   uint32_t *ovf16 = nullptr;

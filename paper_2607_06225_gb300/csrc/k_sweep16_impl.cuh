@@ -85,7 +85,6 @@ struct alignas(16) X16Shared {
   uint2 edge[2][W][2];
   int tmp[2][W];
   uint32_t pair;
-  unsigned long long rsv;
   uint4 move[W > 1 ? W * 32 : 1];  // state on its way to other threads
 };
 
@@ -659,12 +658,13 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
       __syncthreads();
   };
 
+  const uint32_t ck_i = blockIdx.x * GROUPS + grp;
   bool first_item = true;
   for (;;) {
     // ---- next pair ------------------------------------------------------------
     uint32_t t0 = 0;
-    if (a.ck) {
-      t0 = (first_item && grp == 0) ? 0u : a.n_order;
+    if (a.ck) {  // a descriptor per group
+      t0 = (first_item && ck_i < a.n_ck) ? 0u : a.n_order;
       first_item = false;
     } else if (W == 1) {
       if (lane == 0) t0 = atomicAdd(a.counter, 1u);
@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
     w.band_lo = (int)max(blo, -(int64_t)M);
     w.band_hi = (int)min(bhi, (int64_t)N);
 
-    const XdCkpt *ck = a.ck;
+    const XdCkpt *ck = a.ck ? a.ck + ck_i : nullptr;
     const int ckmode = ck ? ck->mode : 0;
     const int seg = ck ? ck->k_start / ck->C : 0;
     if (ckmode == 3) {
@@ -698,28 +698,10 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
     }
     uint32_t *tbp = nullptr;
     int32_t *ckp = nullptr;
-    unsigned long long rsv = 0;
     if (TB) {
       if (ckmode == 2) {
         ckp = ck->seg_ck;
         tbp = ck->seg_tb;
-      } else if (ckmode == 3) {
-        const unsigned long long need = (unsigned long long)ck->C * (WIN / 8);
-        if (W == 1) {
-          if (lane == 0) rsv = atomicAdd(ck->pool_next, need);
-          rsv = __shfl_sync(X16_FULL, rsv, 0);
-        } else {
-          if (threadIdx.x == 0) sh.rsv = atomicAdd(ck->pool_next, need);
-          __syncthreads();
-          rsv = sh.rsv;
-          __syncthreads();
-        }
-        if (rsv + need > ck->pool_words) {
-          if (tid == 0) ck->flags[0] = 2;
-          break;
-        }
-        ckp = ck->seg_ck_all + (int64_t)seg * ck->C;
-        tbp = ck->pool + rsv;
       } else {
         ckp = reinterpret_cast<int32_t *>(a.tb + a.tbl[p].off);
         tbp = a.tb + a.tbl[p].off + (uint64_t)xd_origin_words(M, N);
@@ -1031,10 +1013,6 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
         rec[XCK_BJ] = w.bj;
         rec[XCK_CELLS_LO] = (int32_t)(uint32_t)w.cells;
         rec[XCK_CELLS_HI] = (int32_t)(uint32_t)(w.cells >> 32);
-        if (TB) {
-          ck->seg_off[seg] = rsv;
-          ck->seg_w[seg] = WCODE;
-        }
         ck->flags[1 + seg] = WCODE;
       }
       gsync();
@@ -1042,10 +1020,6 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
     }
     if (tid == 0 && ckmode != 2) {
       if (ckmode == 3) {
-        if (TB && status != FILTR_ST_TOO_WIDE) {
-          ck->seg_off[seg] = rsv;
-          ck->seg_w[seg] = WCODE;
-        }
         ck->flags[0] = 1;
         if (status != FILTR_ST_TOO_WIDE) ck->flags[1 + seg] = WCODE;
       }

@@ -51,7 +51,6 @@ struct alignas(16) XdShared {
   Edge first[2][W];      // slot 0 of the warp (lane 0) after each antidiagonal
   Edge last[2][W];       // slot 31*S + S-1 of the warp (lane 31)
   uint32_t pair;         // work item of the group
-  unsigned long long rsv;  // traceback rows reserved by the group (checkpointed sweep)
 };
 
 __device__ __forceinline__ int code_at(const uint32_t (&w)[2], int s) {
@@ -158,12 +157,13 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
       __syncthreads();
   };
 
+  const uint32_t ck_i = blockIdx.x * (W == 1 ? 4 : 1) + grp;
   bool first_item = true;
   for (;;) {
     // ---- next pair --------------------------------------------------------------
     uint32_t t0 = 0;
-    if (a.ck) {  // checkpointed sweep: one pair, taken once by group 0
-      t0 = (first_item && grp == 0) ? 0u : a.n_order;
+    if (a.ck) {  // checkpointed sweep of one pair: a descriptor per group
+      t0 = (first_item && ck_i < a.n_ck) ? 0u : a.n_order;
       first_item = false;
     } else if (W == 1) {
       if (lane == 0) t0 = atomicAdd(a.counter, 1u);
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
     if (a.sp.use_band) band_limits(M, N, a.sp.band, a.sp.band_literal, &blo, &bhi);
     const int band_lo = (int)max(blo, -(int64_t)M), band_hi = (int)min(bhi, (int64_t)N);
 
-    const XdCkpt *ck = a.ck;
+    const XdCkpt *ck = a.ck ? a.ck + ck_i : nullptr;
     const int ckmode = ck ? ck->mode : 0;
     const int seg = ck ? ck->k_start / ck->C : 0;
     if (ckmode == 3) {
@@ -196,28 +196,10 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
     }
     uint32_t *tbp = nullptr;
     int32_t *ckp = nullptr;
-    unsigned long long rsv = 0;
     if (TB) {
       if (ckmode == 2) {  // rows indexed by k - k_start - 1
         ckp = ck->seg_ck;
         tbp = ck->seg_tb;
-      } else if (ckmode == 3) {  // rows from the pool, indexed by k - k_start - 1
-        const unsigned long long need = (unsigned long long)ck->C * (WIN / 8);
-        if (W == 1) {
-          if (lane == 0) rsv = atomicAdd(ck->pool_next, need);
-          rsv = __shfl_sync(FULLMASK, rsv, 0);
-        } else {
-          if (threadIdx.x == 0) sh.rsv = atomicAdd(ck->pool_next, need);
-          __syncthreads();
-          rsv = sh.rsv;
-          __syncthreads();
-        }
-        if (rsv + need > ck->pool_words) {  // every thread sees the same rsv
-          if (tid == 0) ck->flags[0] = 2;
-          break;
-        }
-        ckp = ck->seg_ck_all + (int64_t)seg * ck->C;
-        tbp = ck->pool + rsv;
       } else {
         ckp = reinterpret_cast<int32_t *>(a.tb + a.tbl[p].off);
         tbp = a.tb + a.tbl[p].off + (uint64_t)xd_origin_words(M, N);
@@ -579,10 +561,6 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
         rec[XCK_BJ] = bj;
         rec[XCK_CELLS_LO] = (int32_t)(uint32_t)cells;
         rec[XCK_CELLS_HI] = (int32_t)(uint32_t)(cells >> 32);
-        if (TB) {
-          ck->seg_off[seg] = rsv;
-          ck->seg_w[seg] = W;
-        }
         ck->flags[1 + seg] = W;
       }
       gsync();
@@ -590,10 +568,6 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
     }
     if (tid == 0 && ckmode != 2) {
       if (ckmode == 3) {  // the sweep ends in this segment (or outgrew the widest window)
-        if (TB && status != FILTR_ST_TOO_WIDE) {
-          ck->seg_off[seg] = rsv;
-          ck->seg_w[seg] = W;
-        }
         ck->flags[0] = 1;
         if (status != FILTR_ST_TOO_WIDE) ck->flags[1 + seg] = W;
       }

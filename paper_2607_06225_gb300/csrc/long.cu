@@ -189,6 +189,9 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   static const int kLadder[] = {1, 2, 4, 8, 16, XD_MAX_WARPS};
   Carve cv{c->ws, c->ws_bytes};
   int32_t *ck_buf = cv.take<int32_t>((size_t)(nseg + 1) * xd_ckpt_stride());
+  // single pass: every segment of the path is recomputed with traceback at once,
+  // into a pool (the rest of the workspace), and walked once; when the pool does
+  // not hold them, one segment at a time is recomputed and walked
   const bool single = sp.traceback && !c->ckpt_recompute;
   uint32_t *seg_tb = (sp.traceback && !single)
                          ? cv.take<uint32_t>((size_t)C * xd_words_per_k(XD_MAX_WARPS, 8))
@@ -203,13 +206,9 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   uint64_t *d_misc = cv.take<uint64_t>(8);   // stage_off, offsets, CIGAR offset
   uint32_t *d_ovf = cv.take<uint32_t>(4);
   uint32_t *d_stage = sp.traceback ? cv.take<uint32_t>((size_t)M + N + 1) : nullptr;
-  // single pass: every segment's traceback rows kept in a pool (the rest of
-  // the workspace), walked once at the end; if the pool runs out the sweep
-  // stops and runs again without traceback, with the segments recomputed
   int32_t *seg_ck_all = single ? cv.take<int32_t>((size_t)nseg * C) : nullptr;
   uint64_t *seg_off = single ? cv.take<uint64_t>(nseg) : nullptr;
   int32_t *seg_wd = single ? cv.take<int32_t>(nseg) : nullptr;
-  unsigned long long *pool_next = single ? cv.take<unsigned long long>(4) : nullptr;
   if (cv.used > c->ws_bytes) {
     set_error("checkpointed traceback needs %zu workspace bytes; the context has %zu", cv.used,
               c->ws_bytes);
@@ -221,10 +220,12 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
     pool = cv.take<uint32_t>(0);
     pool_words = cv.used < c->ws_bytes ? (c->ws_bytes - cv.used) / 4 : 0;
   }
-  // host staging: the one-pair batch, the segment descriptors, the flags
+  // host staging: the one-pair batch, the segment descriptors, the flags, and the
+  // segments' places in the pool
   const size_t desc_off = 4096;
   const size_t flags_off = desc_off + (size_t)(2 * nseg + 1) * sizeof(XdCkpt);
-  if (!c->ensure_host(flags_off + (size_t)(nseg + 1) * 4 + 64)) return FILTR_ERR_NOMEM;
+  const size_t off_off = (flags_off + (size_t)(nseg + 1) * 4 + 63) / 64 * 64;
+  if (!c->ensure_host(off_off + (size_t)nseg * 12 + 64)) return FILTR_ERR_NOMEM;
   char *h = reinterpret_cast<char *>(c->h_stage);
   uint32_t one[16] = {0, M, N};  // order, q_len, r_len
   TbLayout L{};
@@ -234,11 +235,9 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   memcpy(h + 128, misc, sizeof misc);
   XdCkpt *hk = reinterpret_cast<XdCkpt *>(h + desc_off);
   for (int64_t sgi = 0; sgi < nseg; ++sgi)
-    hk[sgi] = XdCkpt{3,      C,          ck_buf,    (int)(sgi * C),
-                     (int)std::min<int64_t>((sgi + 1) * C, K), nullptr, nullptr, d_flags,
-                     pool,   pool_words, pool_next, seg_ck_all, seg_off, seg_wd};
+    hk[sgi] = XdCkpt{3, C, ck_buf, (int)(sgi * C), (int)std::min<int64_t>((sgi + 1) * C, K), nullptr, nullptr,
+                     d_flags};
   cudaError_t e = cudaMemcpyAsync(d_one, h, sizeof one, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && single) e = cudaMemsetAsync(pool_next, 0, 8, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_tbl, h + 64, sizeof L, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_misc, h + 128, sizeof misc, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
@@ -251,7 +250,7 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   FullArgs fa;
   fa.b = b;
   fa.sp = sp;
-  fa.sp.traceback = single ? 1 : 0;  // else the forward sweep keeps checkpoints only
+  fa.sp.traceback = 0;  // the forward sweep keeps checkpoints only
   fa.order = d_one;
   fa.n_order = 1;
   fa.counter = nullptr;  // unused with checkpoints
@@ -296,13 +295,6 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   }
   c->last_xd16 = sp.xd16 ? 1u : 0u;
   c->last_xd16_rerun = 0;
-  if (single && hflags[0] == 2) {  // the pool ran out: recompute the segments instead
-    const bool saved = c->ckpt_recompute;
-    c->ckpt_recompute = true;
-    const filtr_status rc = run_xdrop_ckpt(c, sp, params, q, M, r, N, out, cigar, cap, st, C);
-    c->ckpt_recompute = saved;
-    return rc;
-  }
   if (!sp.traceback || (f.status != FILTR_ST_OK && f.status != FILTR_ST_DROPPED)) return FILTR_OK;
   WalkArgs wp;
   wp.b = b;
@@ -315,9 +307,61 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   wp.tbl = d_tbl;
   wp.stage = d_stage;
   wp.stage_off = d_misc;
-  if (single) {  // one walk over the kept traceback
+  const int64_t ke = (int64_t)f.end_i + f.end_j;
+  if (single) {
+    // The forward sweep is one chain, each antidiagonal waiting for the last; the
+    // segments of the path, given their checkpoints, are not.  So the forward goes
+    // without traceback (a megabase pair: 475 ms instead of 579), and all segments
+    // are recomputed with it side by side, a launch per width.
+    const int64_t n_path = (ke + C - 1) / C;
+    uint64_t *h_off = reinterpret_cast<uint64_t *>(h + off_off);
+    int32_t *h_wd = reinterpret_cast<int32_t *>(h_off + nseg);
+    uint64_t words = 0;
+    for (int64_t sgi = 0; sgi < n_path; ++sgi) {
+      h_wd[sgi] = hflags[1 + sgi];
+      if (h_wd[sgi] <= 0) {
+        set_error("checkpointed sweep: segment %lld has no width", (long long)sgi);
+        return FILTR_ERR_CUDA;
+      }
+      h_off[sgi] = words;
+      words += (uint64_t)C * xd_words_per_k(h_wd[sgi], 8);
+    }
+    if (words > pool_words) {  // one segment at a time instead
+      const bool saved = c->ckpt_recompute;
+      c->ckpt_recompute = true;
+      const filtr_status rc = run_xdrop_ckpt(c, sp, params, q, M, r, N, out, cigar, cap, st, C);
+      c->ckpt_recompute = saved;
+      return rc;
+    }
+    FullArgs ra = fa;
+    ra.sp = sp;  // traceback on
+    ra.out = reinterpret_cast<filtr_result *>(c->d_small + 3072);  // mode 2 writes no result
+    e = cudaMemcpyAsync(seg_off, h_off, n_path * 8, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(seg_wd, h_wd, n_path * 4, cudaMemcpyHostToDevice, st);
+    XdCkpt *hb = hk + nseg;
+    int64_t nb = 0, first[7];
+    for (int wi = 0; wi < 6; ++wi) {
+      first[wi] = nb;
+      for (int64_t sgi = 0; sgi < n_path; ++sgi)
+        if (h_wd[sgi] == kLadder[wi])
+          hb[nb++] = XdCkpt{2, C, ck_buf, (int)(sgi * C), (int)std::min<int64_t>((sgi + 1) * C, ke),
+                            pool + h_off[sgi], seg_ck_all + sgi * C, d_flags};
+    }
+    first[6] = nb;
+    if (e == cudaSuccess && nb)
+      e = cudaMemcpyAsync(d_ck + nseg, hb, nb * sizeof(XdCkpt), cudaMemcpyHostToDevice, st);
+    c->span_begin(Ctx::PH_FORWARD, st);
+    for (int wi = 5; wi >= 0 && e == cudaSuccess; --wi) {
+      if (first[wi + 1] == first[wi]) continue;
+      ra.ck = d_ck + nseg + first[wi];
+      ra.n_ck = (uint32_t)(first[wi + 1] - first[wi]);
+      const int per = xd_pairs_per_cta(kLadder[wi], ra.sp);
+      e = launch_xdrop(ra, kLadder[wi], (int)((ra.n_ck + per - 1) / per), d_ovf, d_ovf + 1, st);
+      ++launches;
+    }
+    c->span_end(st);
     c->span_begin(Ctx::PH_WALK, st);
-    e = launch_walk_pool(wp, pool, seg_ck_all, seg_off, seg_wd, C, st);
+    if (e == cudaSuccess) e = launch_walk_pool(wp, pool, seg_ck_all, seg_off, seg_wd, C, st);
     c->span_end(st);
     uint64_t *d_offs = d_misc + 4;
     if (e == cudaSuccess) e = cudaMemsetAsync(d_offs, 0, 8, st);
@@ -339,7 +383,6 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   WalkState w0{f.end_i, f.end_j, f.score, 0, 0, -1, 0, 0};
   WalkState *hw = reinterpret_cast<WalkState *>(h + 512);
   *hw = w0;
-  const int64_t ke = (int64_t)f.end_i + f.end_j;
   XdCkpt *hb = hk + nseg;
   std::vector<int> seg_w;
   int64_t nb = 0;

@@ -49,6 +49,12 @@ filtr_status filtr_test_set_device_plan(filtr_ctx *ctx, int32_t mode);
  * depend on it; it trades shared memory (occupancy) against load latency. */
 filtr_status filtr_test_set_search_ring(filtr_ctx *ctx, int32_t entries);
 
+/* Most 32-bit words (a multiple of 4; 0 restores the default, whatever the
+ * workspace holds) that a warp of the search with traceback keeps of a pair's
+ * wavefronts.  Pairs that need more take the second pass; results do not depend
+ * on it. */
+filtr_status filtr_test_set_search_keep(filtr_ctx *ctx, int64_t words);
+
 /* Tiled batches a warp per row strip (intra-pair) instead of a warp per pair:
  * 0 by batch size (the default), 1 never, 2 whenever the pairs have several
  * strips and the workspace allows.  Results do not depend on it. */

@@ -182,6 +182,8 @@ def lib():
         L.filtr_test_set_split.argtypes = [C.c_void_p, C.c_int32]
         L.filtr_test_set_search_ring.restype = i32
         L.filtr_test_set_search_ring.argtypes = [C.c_void_p, C.c_int32]
+        L.filtr_test_set_search_keep.restype = i32
+        L.filtr_test_set_search_keep.argtypes = [C.c_void_p, C.c_int64]
         L.filtr_test_set_packed_sweep.restype = i32
         L.filtr_test_set_packed_sweep.argtypes = [C.c_void_p, C.c_int32]
         L.filtr_test_plan_host.restype = i32

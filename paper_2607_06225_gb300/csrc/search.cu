@@ -17,13 +17,29 @@
 // exceeds the wavefront's smallest by more than max_dist, from the first
 // wavefront that spans min_len diagonals.
 //
-// Score pass: the previous and current wavefronts live in a per-warp ring in
-// global memory (index d + M, so no copy when the domain moves).  Traceback
-// pass: every wavefront is kept (per score its bounds, then its values), its
-// size known from the score pass, and one lane walks back from (M, N), taking
-// at each score the first of mismatch, insertion, deletion that gives the
-// level's value; the ops go to the CIGAR staging area reversed, as the other
-// walks leave them.
+// Score pass, a warp per pair: the previous and current wavefronts live in a small
+// ring in shared memory.  A pair whose wavefront outgrows it first gets an upper
+// bound on its score: the search runs on in a window of 32 diagonals that follows
+// its leading cell.  From there on only diagonals are formed from which (M, N) is
+// within that bound, a diamond instead of a triangle.  That changes no result: a
+// cell of the diamond has all its predecessors in the diamond, so its value is
+// the same, and a path of the score lies inside.  (`cells` counts the whole
+// wavefronts; with WFA-Adapt, whose thresholds look at whole wavefronts, all is formed.)
+//
+// With traceback the pass also keeps every wavefront (its values, and per score its
+// bounds) in the warp's slot of the workspace -- past the ring they are the only copy --
+// and the warp walks back from (M, N) as soon as the pair is done, taking at each
+// score the first of mismatch, insertion, deletion that gives the level's value;
+// the ops go to the CIGAR staging area reversed, as the other walks leave them.
+// Only a pair whose wavefronts outgrow the slot goes through a traceback pass of
+// its own: every wavefront once more, into a store whose size the score pass tells.
+//
+// What bounds it: instruction issue, some 60 per 32 diagonals and a comparison
+// loop as long as the longest of 32 runs of matches; more warps than the 64 registers
+// leave (32 per SM) make it slower (48: 1.3 -> 1.6 ms before the bound was used).
+// Measured with traceback, 8192 pairs of 4000 residues at 5%: 3.26 ms for the call when a
+// second pass formed all wavefronts again for the walk, 1.95 ms with the wavefronts
+// kept, 1.51 ms with the bound; 2000 pairs of 2000 at 30%, the kernels alone: 3.3 -> 2.1 ms.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -38,7 +54,6 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int UNREACHED = -1;
 constexpr uint32_t OP_I = 1, OP_D = 2, OP_EQ = 7, OP_X = 8;
-constexpr int SEARCH_CHUNKS = 4;  // chunks of 32 diagonals a warp has in flight per iteration
 
 struct SearchArgs {
   BatchDev b;
@@ -46,7 +61,10 @@ struct SearchArgs {
   const uint32_t *order;
   uint32_t *counter;          // work-queue cursor (zeroed before the launch)
   filtr_result *out;
-  uint64_t *need;             // score pass: words the traceback pass stores per pair
+  uint64_t *need;             // score pass: words the traceback pass stores per pair, 0: none
+  int *keep;                  // score pass: per warp slot, keep_words for the wavefronts
+  uint64_t keep_words;        // (0: no traceback, or no room)
+  uint32_t *n_left;           // score pass: pairs left to the traceback pass
   int *ring;                  // score pass: per warp slot, two wavefronts of ring_half ints
   uint32_t ring_half;         // >= M + N + 1 of every pair
   int *arena;                 // traceback pass: wavefront store
@@ -54,6 +72,7 @@ struct SearchArgs {
   uint32_t *stage;            // traceback pass: reversed CIGAR ops, per pair id
   const uint64_t *stage_off;
   uint32_t q_words, r_words;  // shared-memory staging per warp (32-bit words)
+  uint32_t warp_words;        // score pass: shared memory per warp, with the rings
   uint32_t ring_c;            // score pass: entries of each shared-memory ring (power of two)
   int band;                   // < 0: none
   int adapt_min, adapt_max;   // adapt_min == 0: exact
@@ -168,6 +187,15 @@ __device__ __forceinline__ int terms(const int *pv, int off, uint32_t mask, int 
   return best;
 }
 
+// The same from the three values themselves (UNREACHED: none), without the choice.
+__device__ __forceinline__ int best_row(int vc, int vr, int vl, int d, int M, int N) {
+  int row = UNREACHED;
+  if (vc >= 0 && vc + 1 <= M && vc + 1 + d <= N) row = vc + 1;  // mismatch
+  if (vr >= 0 && vr + 1 <= M && vr + 1 > row) row = vr + 1;     // insertion
+  if (vl >= 0 && vl + d <= N && vl > row) row = vl;             // deletion
+  return row;
+}
+
 // WFA-Adapt: the diagonals of [lo, hi] that survive -- reached, and remaining
 // distance max(M - i, N - j) within amax of the wavefront's smallest; the
 // bounds move inwards to the outermost survivors.
@@ -244,85 +272,252 @@ __device__ __forceinline__ PairView stage_pair(const SearchArgs &a, uint32_t p, 
   return v;
 }
 
-// Progress of one pair's search.
+// Progress of one pair's search.  Level s spans diagonals [flo, fhi] (what cells
+// counts); [lo, hi] of them are formed: those on which (M, N) is within reach of
+// a score of at most ub.
+constexpr int NO_UB = 1 << 28;  // (above any score, and no sum with a diagonal overflows)
 struct Lev {
-  int lo, hi, s;
+  int lo, hi, flo, fhi, s;
+  int ub;     // a score that is enough for the pair, or NO_UB
   uint64_t cells;
   int state;  // 0 running, 1 reached (M, N), 2 gave up (not expected)
 };
 
-// Score levels from L.s on, until (M, N) is reached or -- in a shared-memory
-// ring of C entries -- the next wavefront would not fit (state stays 0).
-template <bool SMEM, int CH, bool P2>
-__device__ __forceinline__ void levels(Lev &L, const Wf &w, int C, const PairView &v, int amin,
-                                       int amax, int lane) {
+// The wavefronts kept for the walk: values from the slot's start, level after
+// level, and the bounds of level s (lo, hi, alive lo, alive hi) in the int4 s + 1
+// before its end.
+struct Keep {
+  int *slot;
+  uint64_t words;
+  uint64_t used;   // value words so far
+  bool ok;         // everything still fits
+  __device__ int4 *meta(int s) const { return reinterpret_cast<int4 *>(slot + words) - (s + 1); }
+};
+
+// CH chunks of 32 diagonals of the level after pv, from d0 to nhi: one load per
+// diagonal of pv (alive ones only); the neighbours d - 1 and d + 1 by two rotating
+// shuffles, in which lane 31 (lane 0) hands lane 0 (lane 31) the last (first)
+// diagonal of the chunk before (after) instead of its own.  True in the lane that
+// reaches (M, N).
+template <int CH, bool P2, bool BOTH>
+__device__ __forceinline__ bool chunks(const int *pv, int *nv, int *kv, uint32_t mk, const PairView &v,
+                                       int alo, int ahi, int d0, int nhi, int lane) {
   const int M = v.M, N = v.N;
+  bool done = false;
+  int vc[CH];
+#pragma unroll
+  for (int u = 0; u < CH; ++u) {
+    const int d = d0 + 32 * u + lane;
+    vc[u] = (d >= alo && d <= ahi) ? pv[at(d, 0, mk)] : UNREACHED;
+  }
+  const int dl = d0 - 1, dr = d0 + 32 * CH;  // outer edges: lane 31 / lane 0 load them
+  const int el = (lane == 31 && dl >= alo && dl <= ahi) ? pv[at(dl, 0, mk)] : UNREACHED;
+  const int er = (lane == 0 && dr >= alo && dr <= ahi) ? pv[at(dr, 0, mk)] : UNREACHED;
+#pragma unroll
+  for (int u = 0; u < CH; ++u) {
+    const int d = d0 + 32 * u + lane;
+    const int to_right = lane == 31 ? (u > 0 ? vc[u > 0 ? u - 1 : 0] : el) : vc[u];
+    const int to_left = lane == 0 ? (u + 1 < CH ? vc[u + 1 < CH ? u + 1 : 0] : er) : vc[u];
+    const int vl = __shfl_sync(FULL, to_right, (lane + 31) & 31);  // F[s][d - 1]
+    const int vr = __shfl_sync(FULL, to_left, (lane + 1) & 31);    // F[s][d + 1]
+    const int row = best_row(vc[u], vr, vl, d, M, N);
+    if (d <= nhi) {
+      const int f = row >= 0 ? extend<P2>(v.q, v.r, row, d, M, N) : UNREACHED;
+      nv[at(d, 0, mk)] = f;
+      if (BOTH && kv) kv[d] = f;
+      done |= d == v.target && f >= M;
+    }
+  }
+  return done;
+}
+
+// Score levels from L.s on (its values at pv), until (M, N) is reached or -- in a
+// shared-memory ring of C entries -- the next wavefront would not fit (state stays
+// 0).  In global memory a level's values go to the kept wavefronts alone while
+// these fit, else to the two buffers of w.
+template <bool SMEM, bool P2, bool KEEP>
+__device__ __forceinline__ void levels(Lev &L, const int *pv, const Wf &w, int C, const PairView &v,
+                                       int amin, int amax, int lane, Keep &kp) {
+  const int M = v.M, N = v.N;
+  const uint32_t mk = SMEM ? w.mask : 0xffffffffu;
+  bool done = v.target >= L.lo && v.target <= L.hi && pv[at(v.target, 0, mk)] >= M;
   for (;;) {
-    const int *cv = level_buf(w, L.s);
-    bool done = false;
-    if (lane == 0 && v.target >= L.lo && v.target <= L.hi)
-      done = cv[at(v.target, w.off, w.mask)] >= M;
-    done = __shfl_sync(FULL, done, 0);
     if (done) {
       L.state = 1;
       return;
     }
     int alo = L.lo, ahi = L.hi;
-    if (amin > 0 && L.hi - L.lo + 1 >= amin)
-      adapt_bounds(cv, w.off, w.mask, L.lo, L.hi, M, N, amax, lane, &alo, &ahi);
+    if (amin > 0) {
+      if (L.hi - L.lo + 1 >= amin) adapt_bounds(pv, 0, mk, L.lo, L.hi, M, N, amax, lane, &alo, &ahi);
+      L.flo = alo;
+      L.fhi = ahi;
+    }
     if (L.s >= M + N + 1 || alo > ahi) {  // the leading diagonal always survives
       L.state = 2;
       return;
     }
-    const int nlo = max(alo - 1, v.dlo), nhi = min(ahi + 1, v.dhi);
+    const int flo = max(L.flo - 1, v.dlo), fhi = min(L.fhi + 1, v.dhi);
+    int nlo = flo, nhi = fhi;
     if (SMEM && nhi - nlo + 1 > C) return;
-    int *nv = level_buf(w, L.s + 1);
-    // CH chunks of 32 diagonals per iteration: one load per diagonal of the
-    // previous wavefront (alive diagonals only); the neighbours d - 1 and d + 1
-    // by two rotating shuffles, in which lane 31 (lane 0) hands lane 0 (lane 31)
-    // the last (first) diagonal of the chunk before (after) instead of its own
-    const uint32_t mk = SMEM ? w.mask : 0xffffffffu;
-    for (int d0 = nlo; d0 <= nhi; d0 += 32 * CH) {
-      int vc[CH];
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        const int d = d0 + 32 * u + lane;
-        vc[u] = (d >= alo && d <= ahi) ? cv[at(d, w.off, mk)] : UNREACHED;
-      }
-      const int dl = d0 - 1, dr = d0 + 32 * CH;  // outer edges: lane 31 / lane 0 load them
-      const int el = (lane == 31 && dl >= alo && dl <= ahi) ? cv[at(dl, w.off, mk)] : UNREACHED;
-      const int er = (lane == 0 && dr >= alo && dr <= ahi) ? cv[at(dr, w.off, mk)] : UNREACHED;
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        const int d = d0 + 32 * u + lane;
-        const int to_right = lane == 31 ? (u > 0 ? vc[u > 0 ? u - 1 : 0] : el) : vc[u];
-        const int to_left = lane == 0 ? (u + 1 < CH ? vc[u + 1 < CH ? u + 1 : 0] : er) : vc[u];
-        const int vl = __shfl_sync(FULL, to_right, (lane + 31) & 31);  // F[s][d - 1]
-        const int vr = __shfl_sync(FULL, to_left, (lane + 1) & 31);    // F[s][d + 1]
-        int row = UNREACHED;
-        if (vc[u] >= 0 && vc[u] + 1 <= M && vc[u] + 1 + d <= N) row = vc[u] + 1;  // mismatch
-        if (vr >= 0 && vr + 1 <= M && vr + 1 > row) row = vr + 1;                // insertion
-        if (vl >= 0 && vl + d <= N && vl > row) row = vl;                        // deletion
-        if (d <= nhi) nv[at(d, w.off, mk)] = row >= 0 ? extend<P2>(v.q, v.r, row, d, M, N) : UNREACHED;
+    if (!SMEM) {  // what is left of ub bounds the distance to the target's diagonal
+      nlo = max(nlo, v.target - (L.ub - L.s - 1));
+      nhi = min(nhi, v.target + (L.ub - L.s - 1));
+      if (nlo > nhi) {  // not expected: ub is enough
+        L.state = 2;
+        return;
       }
     }
+    int *nv = level_buf(w, L.s + 1) + (SMEM ? 0 : w.off);
+    int *kv = nullptr;  // diagonal d of level L.s + 1 at kv[d]
+    if (KEEP) {
+      if (kp.ok && lane == 0) *kp.meta(L.s) = make_int4(L.lo, L.hi, alo, ahi);
+      // the values of level L.s + 1 and the bounds of levels up to L.s + 2
+      kp.ok = kp.ok && kp.used + (uint64_t)(nhi - nlo + 1) + 4ull * (uint64_t)(L.s + 3) <= kp.words;
+      if (kp.ok) {
+        kv = kp.slot + kp.used - nlo;
+        if (!SMEM) nv = kv;
+      }
+      kp.used += (uint64_t)(nhi - nlo + 1);
+    }
+    int d0 = nlo;
+    if (!SMEM) {
+      for (; d0 + 96 <= nhi; d0 += 128) done |= chunks<4, P2, false>(pv, nv, kv, mk, v, alo, ahi, d0, nhi, lane);
+      if (d0 + 32 <= nhi) {
+        done |= chunks<2, P2, false>(pv, nv, kv, mk, v, alo, ahi, d0, nhi, lane);
+        d0 += 64;
+      }
+    }
+    for (; d0 <= nhi; d0 += 32) done |= chunks<1, P2, SMEM && KEEP>(pv, nv, kv, mk, v, alo, ahi, d0, nhi, lane);
     __syncwarp();
-    L.cells += (uint64_t)(nhi - nlo + 1);
+    done = __any_sync(FULL, done);
+    L.cells += (uint64_t)(fhi - flo + 1);
     L.lo = nlo;
     L.hi = nhi;
+    L.flo = flo;
+    L.fhi = fhi;
     ++L.s;
+    pv = nv;
   }
 }
 
-// Score pass: distance and wavefront cells of every pair, and the words its
-// traceback pass would store.  Per warp in shared memory: the two sequences,
+// A score that is enough for the pair: the search goes on from level L.s in a
+// window of 32 diagonals alone, which follows the cell that is furthest along.
+// Any way from there to (M, N) will do; it is rarely dearer than the best one.
+// The leader is two or more diagonals from the window's edges wherever the domain
+// goes on there, and one of its moves is open unless it is at (M, N): every level
+// brings it further, and the straight way (max(M, N) edits) ends the search.
+template <bool P2>
+__device__ __forceinline__ int enough(const Lev &L, const int *pv, uint32_t mk, const PairView &v, int lane) {
+  const int M = v.M, N = v.N, most = max(M, N);
+  int w0 = min(max((L.lo + L.hi) / 2 - 15, L.lo), L.hi), f;
+  {
+    const int d = w0 + lane;
+    f = d >= L.lo && d <= L.hi ? pv[at(d, 0, mk)] : UNREACHED;
+  }
+  for (int s = L.s; s < most;) {
+    // the leader's lane: the largest i + j, the lowest lane on ties
+    const int far = f >= 0 ? 2 * f + w0 + lane : -1;
+    const int top = __reduce_max_sync(FULL, far);
+    if (top < 0) return most;  // (no cell of the window is reached)
+    const int lead = __ffs(__ballot_sync(FULL, far == top)) - 1;
+    const int sh = lead < 6 ? -8 : (lead > 25 ? 8 : 0);
+    if (sh != 0) {
+      const int t = __shfl_sync(FULL, f, (lane + sh) & 31);
+      f = (unsigned)(lane + sh) < 32u ? t : UNREACHED;
+      w0 += sh;
+    }
+    const int d = w0 + lane;
+    const int up = __shfl_down_sync(FULL, f, 1), dn = __shfl_up_sync(FULL, f, 1);
+    const int row = best_row(f, lane == 31 ? UNREACHED : up, lane == 0 ? UNREACHED : dn, d, M, N);
+    f = row >= 0 && d >= v.dlo && d <= v.dhi ? extend<P2>(v.q, v.r, row, d, M, N) : UNREACHED;
+    ++s;
+    if (__any_sync(FULL, d == v.target && f >= M)) return s;
+  }
+  return most;
+}
+
+// Walk back from (M, N) through the kept wavefronts of a finished pair (score S):
+// per score, the matches after the edit, then the edit.  Ten levels at a time: the
+// path moves at most one diagonal per level, so the warp loads the 2x + 3 values
+// around the current diagonal of the x-th level below (their bounds first) at
+// once, and lane 0 walks them in shared memory.
+constexpr int BACK = 10, BACK_W = 2 * BACK + 3;
+struct BackBuf {
+  int4 m[BACK];
+  int v[BACK][BACK_W];
+  int pad[2];  // whole int4s, as the next warp's buffer follows
+};
+static_assert(sizeof(BackBuf) % 16 == 0, "warps' buffers are 16-byte aligned");
+__device__ __forceinline__ uint32_t walk_back(const Keep &kp, BackBuf &bb, uint32_t *dst, int S, int M, int N,
+                                              int lane) {
+  RevEmitter em{dst};
+  int d = N - M, i = M;
+  uint64_t at_s = kp.used;  // one past level S's values
+  {
+    const int4 t = *kp.meta(S);
+    at_s -= (uint64_t)(t.y - t.x + 1);  // level S's first value
+  }
+  for (int s = S; s > 0;) {
+    const int nb = min(BACK, s);
+    int4 m = make_int4(0, -1, 0, -1);
+    if (lane < nb) {
+      m = *kp.meta(s - 1 - lane);
+      bb.m[lane] = m;
+    }
+    // level s - 1 - x starts x + 1 levels' widths before level s's first value
+    uint32_t wsum = (uint32_t)(m.y - m.x + 1);
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL, wsum, o);
+      if (lane >= o) wsum += t;
+    }
+    const int d0 = __shfl_sync(FULL, d, 0);
+#pragma unroll
+    for (int x = 0; x < BACK; ++x) {
+      const uint32_t down = __shfl_sync(FULL, wsum, x);
+      const int lo = __shfl_sync(FULL, m.x, x), hi = __shfl_sync(FULL, m.y, x);
+      const int dd = d0 - BACK - 1 + lane;
+      if (x < nb && lane < BACK_W && dd >= lo && dd <= hi) bb.v[x][lane] = kp.slot[at_s - down + (uint64_t)(dd - lo)];
+    }
+    __syncwarp();
+    if (lane == 0) {
+      for (int x = 0; x < nb; ++x) {
+        int which;
+        const int4 t = bb.m[x];
+        const int row = terms(bb.v[x], BACK + 1 - d0, 0xffffffffu, t.z, t.w, d, M, N, &which);
+        em.put(OP_EQ, (uint32_t)(i - row));
+        if (which == 0) {
+          em.put(OP_X, 1);
+          i = row - 1;
+        } else if (which == 1) {
+          em.put(OP_I, 1);
+          i = row - 1;
+          d = d + 1;
+        } else {
+          em.put(OP_D, 1);
+          i = row;
+          d = d - 1;
+        }
+      }
+    }
+    __syncwarp();
+    at_s -= __shfl_sync(FULL, wsum, nb - 1);
+    s -= nb;
+  }
+  if (lane == 0) em.put(OP_EQ, (uint32_t)i);
+  em.flush();
+  return em.n;
+}
+
+// Score pass: distance and wavefront cells of every pair, and (KEEP) its CIGAR or
+// the words its traceback pass stores.  Per warp in shared memory: the two sequences,
 // then two rings of ring_c entries; a pair whose wavefront outgrows them moves
 // to the warp's buffers in global memory.
-template <bool P2>
+template <bool P2, bool KEEP>
 __global__ void __launch_bounds__(128) k_search_score(const SearchArgs a) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  uint32_t *sq = smem + (size_t)wib * (a.q_words + a.r_words + 2 * a.ring_c);
+  uint32_t *sq = smem + (size_t)wib * a.warp_words;
   uint32_t *sr = sq + a.q_words;
   int *ra = reinterpret_cast<int *>(sr + a.r_words), *rb = ra + a.ring_c;
   const uint64_t slot = (uint64_t)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -336,19 +531,36 @@ __global__ void __launch_bounds__(128) k_search_score(const SearchArgs a) {
     if (t >= a.n) return;
     const uint32_t p = a.order ? a.order[t] : t;
     const PairView v = stage_pair<P2>(a, p, sq, sr, lane);
+    Keep kp{KEEP ? a.keep + slot * a.keep_words : nullptr, a.keep_words, 1ull, KEEP && a.keep_words >= 16};
     // score 0: the origin and its run of matches
-    if (lane == 0) ra[at(0, ws.off, ws.mask)] = extend<P2>(v.q, v.r, 0, 0, v.M, v.N);
+    if (lane == 0) {
+      const int f = extend<P2>(v.q, v.r, 0, 0, v.M, v.N);
+      ra[at(0, ws.off, ws.mask)] = f;
+      if (KEEP && kp.ok) kp.slot[0] = f;
+    }
     __syncwarp();
-    Lev L{0, 0, 0, 1ull, 0};
-    levels<true, SEARCH_CHUNKS, P2>(L, ws, (int)a.ring_c, v, a.adapt_min, a.adapt_max, lane);
-    if (L.state == 0) {  // level L.s to global memory, then on from there
-      const Wf wg{g, g + a.ring_half, v.M, 0xffffffffu};
+    Lev L{0, 0, 0, 0, 0, NO_UB, 1ull, 0};
+    levels<true, P2, KEEP>(L, ra, ws, (int)a.ring_c, v, a.adapt_min, a.adapt_max, lane, kp);
+    if (L.state == 0) {  // level L.s in global memory, then on from there
       const int *src = level_buf(ws, L.s);
-      int *dst = level_buf(wg, L.s);
-      for (int d = L.lo + lane; d <= L.hi; d += 32)
-        dst[at(d, wg.off, wg.mask)] = src[at(d, ws.off, ws.mask)];
+      const Wf wg{g, g + a.ring_half, v.M, 0xffffffffu};
+      const int *pv;
+      if (a.adapt_min == 0) L.ub = enough<P2>(L, src, ws.mask, v, lane);
+      if (KEEP && kp.ok) {
+        pv = kp.slot + kp.used - (L.hi + 1);
+      } else {
+        int *dst = level_buf(wg, L.s) + wg.off;
+        for (int d = L.lo + lane; d <= L.hi; d += 32) dst[d] = src[at(d, 0, ws.mask)];
+        pv = dst;
+      }
       __syncwarp();
-      levels<false, SEARCH_CHUNKS, P2>(L, wg, 0, v, a.adapt_min, a.adapt_max, lane);
+      levels<false, P2, KEEP>(L, pv, wg, 0, v, a.adapt_min, a.adapt_max, lane, kp);
+    }
+    uint32_t n_ops = 0;
+    if (KEEP && L.state == 1 && kp.ok) {
+      if (lane == 0) *kp.meta(L.s) = make_int4(L.lo, L.hi, L.lo, L.hi);
+      __syncwarp();
+      n_ops = walk_back(kp, *reinterpret_cast<BackBuf *>(sq), a.stage + a.stage_off[p], L.s, v.M, v.N, lane);
     }
     if (lane == 0) {
       const bool ok = L.state == 1;
@@ -359,12 +571,16 @@ __global__ void __launch_bounds__(128) k_search_score(const SearchArgs a) {
       r.r_begin = 0;
       r.r_end = v.N;
       r.status = ok ? FILTR_ST_OK : FILTR_ST_TOO_WIDE;
-      r.cigar_len = 0;
+      r.cigar_len = n_ops;
       r.reserved = 0;
       r.cigar_off = 0;
       r.cells = L.cells;
       a.out[p] = r;
-      if (a.need) a.need[p] = ok ? 4ull * (uint64_t)(L.s + 1) + L.cells : 0ull;
+      if (KEEP) {
+        const bool left = ok && !kp.ok;
+        a.need[p] = left ? 4ull * (uint64_t)(L.s + 1) + L.cells : 0ull;
+        if (left) atomicAdd(a.n_left, 1u);
+      }
     }
     __syncwarp();
   }
@@ -386,10 +602,7 @@ __global__ void __launch_bounds__(128) k_search_tb(const SearchArgs a) {
     t = __shfl_sync(FULL, t, 0);
     if (t >= a.n) return;
     const uint32_t p = a.order ? a.order[t] : t;
-    if (a.out[p].status != FILTR_ST_OK) {  // the score pass gave up on it (not expected)
-      if (lane == 0) a.out[p].cigar_len = 0;
-      continue;
-    }
+    if (a.out[p].status != FILTR_ST_OK) continue;  // the score pass gave up on it (not expected)
     const PairView v = stage_pair<P2>(a, p, sq, sr, lane);
     const int M = v.M, N = v.N;
     const int S = -a.out[p].score;
@@ -422,7 +635,15 @@ __global__ void __launch_bounds__(128) k_search_tb(const SearchArgs a) {
       }
       const int *pv = cv;
       const int pbase = lo;
-      const int nlo = max(alo - 1, v.dlo), nhi = min(ahi + 1, v.dhi);
+      int nlo = max(alo - 1, v.dlo), nhi = min(ahi + 1, v.dhi);
+      if (a.adapt_min == 0) {  // what can still reach (M, N)
+        nlo = max(nlo, v.target - (S - s - 1));
+        nhi = min(nhi, v.target + (S - s - 1));
+        if (nlo > nhi) {  // not expected
+          ok = false;
+          break;
+        }
+      }
       woff += (uint64_t)(hi - lo + 1);
       cv = waves + woff;
       for (int d0 = nlo; d0 <= nhi; d0 += 32) {
@@ -610,14 +831,20 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
   a.r_words = p2 ? (max_n + 48) / 64 * 4 + 4 : (max_n + 48) / 16 * 4;
   a.ring_half = max_m + max_n + 1;
   // shared-memory rings: small, so they cost little occupancy; a pair whose
-  // wavefront grows wider continues in global memory
-  const uint32_t ring_cap = ctx->search_ring > 0 ? (uint32_t)ctx->search_ring : 32u;
+  // wavefront grows wider continues in global memory, where a bound on its score
+  // first halves what is left.  8192 pairs of 4000 residues at 5% (1%) divergence with
+  // 32, 64, 128 and 256 entries: 1.34, 1.31, 1.30, 1.36 ms (0.26, 0.25, 0.24, 0.24)
+  const uint32_t ring_cap = ctx->search_ring > 0 ? (uint32_t)ctx->search_ring : 64u;
   a.ring_c = 32;
   while (a.ring_c < a.ring_half && a.ring_c < ring_cap) a.ring_c <<= 1;
   LaunchCfg cfg_score, cfg_tb;
-  auto k_score = p2 ? k_search_score<true> : k_search_score<false>;
+  auto k_score = tb ? (p2 ? k_search_score<true, true> : k_search_score<false, true>)
+                    : (p2 ? k_search_score<true, false> : k_search_score<false, false>);
   auto k_tb = p2 ? k_search_tb<true> : k_search_tb<false>;
-  ce = pick_cfg(k_score, (size_t)(a.q_words + a.r_words + 2 * a.ring_c) * 4, &cfg_score);
+  // (the walk's window takes the place of the sequences and the rings)
+  a.warp_words = a.q_words + a.r_words + 2 * a.ring_c;
+  if (tb) a.warp_words = std::max<uint32_t>(a.warp_words, sizeof(BackBuf) / 4);
+  ce = pick_cfg(k_score, (size_t)a.warp_words * 4, &cfg_score);
   if (ce == cudaSuccess && tb) ce = pick_cfg(k_tb, (size_t)(a.q_words + a.r_words) * 4, &cfg_tb);
   if (ce != cudaSuccess) return cuda_fail(ce, "search kernel occupancy");
 
@@ -646,22 +873,67 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
               ring_base + (size_t)slot_bytes * wpb);
     return FILTR_ERR_NOMEM;
   }
+  // half of what is left of the workspace holds the wavefronts of the pairs in
+  // flight (workspaces that a few pairs' wavefronts would fill go in waves)
+  int *d_keep = c.take<int>(0);
+  a.keep = d_keep;
+  a.keep_words = tb && c.used < ctx->ws_bytes ? (ctx->ws_bytes - c.used) / 2 / sizeof(int) / n_slots / 4 * 4 : 0;
+  if (ctx->search_keep > 0) a.keep_words = std::min<uint64_t>(a.keep_words, (uint64_t)ctx->search_keep);
+  uint64_t *h_soff = reinterpret_cast<uint64_t *>(ctx->h_stage);  // (the lengths are copied)
+  if (tb) {
+    uint64_t soff = 0;
+    for (uint32_t p = 0; p < n; ++p) {
+      h_soff[p] = soff;
+      soff += (uint64_t)ql[p] + rl[p] + 1;
+    }
+    ce = cudaMemcpyAsync(d_stage_off, h_soff, (size_t)n * 8, cudaMemcpyHostToDevice, st);
+    if (ce != cudaSuccess) return cuda_fail(ce, "uploading the traceback layout");
+  }
   ce = cudaMemsetAsync(d_counter, 0, 64 * sizeof(uint32_t), st);
   if (ce != cudaSuccess) return cuda_fail(ce, "clearing the queue counters");
 
   // score pass
   a.n = n;
   a.counter = d_counter;
+  a.n_left = d_counter + 63;
   a.need = d_need;
   a.ring = d_ring;
+  a.stage = d_stage;
+  a.stage_off = d_stage_off;
   ctx->span_begin(Ctx::PH_FORWARD, st);
   ce = launch_cfg(k_score, cfg_score, a, ctx->sms, n_slots, st);
   ctx->span_end(st);
   ++launches;
   if (ce != cudaSuccess) return cuda_fail(ce, "search score pass");
+  ctx->last_waves = 1;
 
   if (tb) {
-    // wavefront storage per pair, cut into waves that fit the workspace
+    // CIGARs in pair order, and the total and the pairs left over to the host
+    WalkArgs wa{};
+    wa.stage = d_stage;
+    wa.stage_off = d_stage_off;
+    uint64_t h_total = 0;
+    uint32_t h_left = 0;
+    auto place = [&]() -> filtr_status {
+      ctx->span_begin(Ctx::PH_PLACE, st);
+      ce = launch_scan_offsets(out, n, d_offs, d_total, st);
+      if (ce == cudaSuccess) ce = launch_compact(wa, n, d_offs, cigar, cap, out, st);
+      ctx->span_end(st);
+      launches += 2;
+      if (ce != cudaSuccess) return cuda_fail(ce, "CIGAR placement");
+      uint64_t *h = reinterpret_cast<uint64_t *>(ctx->h_stage);
+      ce = cudaMemcpyAsync(h, d_total, 8, cudaMemcpyDeviceToHost, st);
+      if (ce == cudaSuccess) ce = cudaMemcpyAsync(h + 1, d_counter + 63, 4, cudaMemcpyDeviceToHost, st);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+      if (ce != cudaSuccess) return cuda_fail(ce, "reading the CIGAR total");
+      h_total = h[0];
+      h_left = *reinterpret_cast<uint32_t *>(h + 1);
+      return FILTR_OK;
+    };
+    filtr_status rc = place();
+    if (rc != FILTR_OK) return rc;
+    if (h_left > 0) {
+    // wavefront storage of the pairs left over, cut into waves that fit the workspace
     uint64_t *h_need = reinterpret_cast<uint64_t *>(ctx->h_stage);
     ce = cudaMemcpyAsync(h_need, d_need, (size_t)n * 8, cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
@@ -677,12 +949,13 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
       return FILTR_ERR_NOMEM;
     }
     uint64_t *h_aoff = reinterpret_cast<uint64_t *>(ctx->h_stage);
-    uint64_t *h_soff = h_aoff + n;
-    uint32_t *h_ord = reinterpret_cast<uint32_t *>(h_soff + n);
+    uint32_t *h_ord = reinterpret_cast<uint32_t *>(h_aoff + n);
     std::vector<std::pair<uint32_t, uint32_t>> wave_ranges;
-    uint64_t used = 0, soff = 0;
-    uint32_t begin = 0;
+    uint64_t used = 0;
+    uint32_t begin = 0, at = 0;
     for (uint32_t p = 0; p < n; ++p) {
+      h_aoff[p] = 0;
+      if (need[p] == 0) continue;
       const uint64_t w = (need[p] + 3) / 4 * 4;  // keep each pair's store 16-byte aligned
       if (w > arena_words) {
         set_error("pair %u keeps %llu wavefront words; the workspace holds %llu", p,
@@ -690,33 +963,27 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
         return FILTR_ERR_NOMEM;
       }
       if (used + w > arena_words) {
-        wave_ranges.push_back({begin, p});
-        begin = p;
+        wave_ranges.push_back({begin, at});
+        begin = at;
         used = 0;
       }
       h_aoff[p] = used;
       used += w;
-      h_ord[p] = p;
-      h_soff[p] = soff;
-      soff += (uint64_t)ql[p] + rl[p] + 1;
+      h_ord[at++] = p;
     }
-    wave_ranges.push_back({begin, n});
+    wave_ranges.push_back({begin, at});
     if (wave_ranges.size() > 60) {
       set_error("the traceback would take %zu waves", wave_ranges.size());
       return FILTR_ERR_NOMEM;
     }
     ce = cudaMemcpyAsync(d_arena_off, h_aoff, (size_t)n * 8, cudaMemcpyHostToDevice, st);
     if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(d_stage_off, h_soff, (size_t)n * 8, cudaMemcpyHostToDevice, st);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(d_order, h_ord, (size_t)n * 4, cudaMemcpyHostToDevice, st);
+      ce = cudaMemcpyAsync(d_order, h_ord, (size_t)at * 4, cudaMemcpyHostToDevice, st);
     if (ce != cudaSuccess) return cuda_fail(ce, "uploading the traceback layout");
     a.need = nullptr;
     a.ring = nullptr;
     a.arena = d_arena;
     a.arena_off = d_arena_off;
-    a.stage = d_stage;
-    a.stage_off = d_stage_off;
     ctx->span_begin(Ctx::PH_WALK, st);
     for (size_t w = 0; w < wave_ranges.size(); ++w) {
       a.order = d_order + wave_ranges[w].first;
@@ -730,28 +997,15 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
     if (ce != cudaSuccess) return cuda_fail(ce, "search traceback pass");
     ctx->last_waves = (int)wave_ranges.size();
 
-    // CIGARs in pair order
-    WalkArgs wa{};
-    wa.stage = d_stage;
-    wa.stage_off = d_stage_off;
-    ctx->span_begin(Ctx::PH_PLACE, st);
-    ce = launch_scan_offsets(out, n, d_offs, d_total, st);
-    if (ce == cudaSuccess) ce = launch_compact(wa, n, d_offs, cigar, cap, out, st);
-    ctx->span_end(st);
-    launches += 2;
-    if (ce != cudaSuccess) return cuda_fail(ce, "CIGAR placement");
-    uint64_t *h_total = reinterpret_cast<uint64_t *>(ctx->h_stage);
-    ce = cudaMemcpyAsync(h_total, d_total, 8, cudaMemcpyDeviceToHost, st);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "reading the CIGAR total");
-    if (*h_total > cap) {
-      set_error("CIGARs need %llu ops, cigar_cap is %llu", (unsigned long long)*h_total,
+    rc = place();
+    if (rc != FILTR_OK) return rc;
+    }
+    if (h_total > cap) {
+      set_error("CIGARs need %llu ops, cigar_cap is %llu", (unsigned long long)h_total,
                 (unsigned long long)cap);
       ctx->last_launches = launches;
       return FILTR_ERR_CIGAR_CAP;
     }
-  } else {
-    ctx->last_waves = 1;
   }
   ctx->last_launches = launches;
   ctx->last_cells_estimate = 0;
@@ -772,6 +1026,15 @@ extern "C" filtr_status filtr_test_set_search_ring(filtr_ctx *ctx, int32_t entri
     return FILTR_ERR_INVALID;
   }
   reinterpret_cast<Ctx *>(ctx)->search_ring = entries;
+  return FILTR_OK;
+}
+
+extern "C" filtr_status filtr_test_set_search_keep(filtr_ctx *ctx, int64_t words) {
+  if (!ctx || words < 0 || words % 4 != 0) {
+    set_error("filtr_test_set_search_keep: bad arguments");
+    return FILTR_ERR_INVALID;
+  }
+  reinterpret_cast<Ctx *>(ctx)->search_keep = words;
   return FILTR_OK;
 }
 

@@ -193,3 +193,21 @@ def test_traceback_waves(F):
         small.close()
     ores, oops, ooff = oracle.search_batch(b)
     compare_search(b, res, cig, ores, oops, ooff, True, label="waves")
+
+
+@pytest.mark.parametrize("keep", [0, 4, 16, 64, 2000, 40000])
+@pytest.mark.parametrize("opts", [dict(), dict(band=7), dict(adapt=(10, 5)), dict(alphabet=4)])
+def test_kept_wavefronts(F, ctx, keep, opts):
+    """Wavefronts kept in one pass, or too many for a warp's share of the workspace
+    (for every pair, for some, for none): the same results, whatever the share."""
+    qs, rs = synth.random_pairs(150, 220, 220, 4, seed=70, related=0.7)
+    for n in (9, 10, 11, 12, 21, 31):  # distances around the walk's ten levels
+        q = np.full(n, 2, np.uint8)
+        qs.append(q)
+        rs.append(np.full(60, 1, np.uint8) if n % 2 else np.full(n, 3, np.uint8))
+    b = synth.pack(*with_edges(qs, rs, np.random.default_rng(70), 4), 4, np.zeros((4, 4), np.int8))
+    F.lib().filtr_test_set_search_keep(ctx.handle, keep)
+    try:
+        check(F, ctx, b, label=f"keep {keep} {opts}", **opts)
+    finally:
+        F.lib().filtr_test_set_search_keep(ctx.handle, 0)

@@ -184,7 +184,7 @@ int Ctx::split_blocks_per_sm(bool packed, int R, const ScoreParams &sp) {
                                    sp.use_band, sp.alphabet);
   auto it = occ_cache.find(key);
   if (it != occ_cache.end()) return it->second;
-  const int nb = std::max(1, packed ? split_pack_blocks_per_sm(R, sp) : split_full_blocks_per_sm(sp));
+  const int nb = std::max(1, packed ? split_pack_blocks_per_sm(R, sp) : split_full_blocks_per_sm(R, sp));
   occ_cache[key] = nb;
   return nb;
 }

@@ -53,7 +53,7 @@ FILTR_HD void strip_cols(int64_t row0, int64_t Hs, int64_t M, int64_t N, bool ba
 // plus 31 pipeline steps, R/8 words per lane per step, 32 lanes.
 FILTR_HD int64_t strip_tb_words(int64_t jlo, int64_t jhi, int R) {
   int64_t ncol = jhi >= jlo ? (jhi - jlo + 1) : 0;
-  return ncol > 0 ? (ncol + 31) * (R / 8) * 32 : 0;
+  return ncol > 0 ? (ncol + 31) * ((R + 7) / 8) * 32 : 0;
 }
 
 // Traceback bits.  Each cell contributes four bits, pushed most significant

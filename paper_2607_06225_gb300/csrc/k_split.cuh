@@ -4,7 +4,8 @@
 //
 // A batch whose pairs do not fill the device leaves most warps idle when a warp
 // takes a whole pair, and its time is that of its longest pair.  Here the unit
-// of work is one strip of 32 * R rows (R = 8, or 16 in the packed tile), so a
+// of work is one strip of 32 * R rows (R = 8, or 16 in the packed tile, or 4 for one
+// long banded pair), so a
 // pair of M rows uses M / (32 R) warps and takes about N + lag steps instead of
 // strips x N.  The cells, traceback words and results are those of k_full /
 // k_pack with the same R.
@@ -184,10 +185,10 @@ SplitSpace split_space(uint64_t n, uint64_t ns, uint64_t stride);
 constexpr uint32_t SPLIT_MAX_STRIPS = 12000;
 void split_bind(SplitArgs *a, char *mem, const SplitSpace &sp, uint32_t stride);
 cudaError_t launch_split(const SplitLaunch &l, cudaStream_t st);
-cudaError_t launch_split_full(const SplitArgs &a, int grid, cudaStream_t st);
+cudaError_t launch_split_full(const SplitArgs &a, int R, int grid, cudaStream_t st);  // R = 8; banded: or 4
 cudaError_t launch_split_pack(const SplitArgs &a, int R, int grid, cudaStream_t st);
-int split_full_blocks_per_sm(const ScoreParams &sp);
+int split_full_blocks_per_sm(int R, const ScoreParams &sp);
 int split_pack_blocks_per_sm(int R, const ScoreParams &sp);
-inline int split_rows(bool packed, int R) { return 32 * (packed ? R : 8); }
+inline int split_rows(bool packed, int R) { return 32 * (packed || R == 4 ? R : 8); }
 
 }  // namespace filtr

@@ -6,8 +6,6 @@
 namespace filtr {
 namespace {
 
-constexpr int SPLIT_R = 8;
-
 // H in 30 bits above minus infinity (finite scores stay below 2^28), and H - F in
 // 23: F opens from the row above, so a finite F is at most the largest score plus
 // two opened gaps (below 2^23) short of H; the largest difference stands for an
@@ -29,9 +27,9 @@ struct FullLink : SplitLink {
   }
 };
 
-template <bool LOCAL, bool AFFINE, bool TB, bool BAND>
+template <int R, bool LOCAL, bool AFFINE, bool TB, bool BAND>
 __global__ void __launch_bounds__(FULL_WARPS * 32) k_split_full(const SplitArgs a) {
-  constexpr int R = SPLIT_R, HS = 32 * R;
+  constexpr int HS = 32 * R;
   extern __shared__ __align__(16) int8_t smem[];
   const GraphDesc *gd = a.f.gd;
   if (gd && gd->abort) return;
@@ -97,17 +95,17 @@ __global__ void __launch_bounds__(FULL_WARPS * 32) k_split_full(const SplitArgs 
   }
 }
 
-template <bool LOCAL, bool AFFINE, bool TB, bool BAND>
+template <int R, bool LOCAL, bool AFFINE, bool TB, bool BAND>
 cudaError_t launch_sf(const SplitArgs &a, int grid, cudaStream_t st) {
-  auto k = k_split_full<LOCAL, AFFINE, TB, BAND>;
-  k<<<grid, FULL_WARPS * 32, full_smem_bytes(SPLIT_R, a.f.sp.alphabet), st>>>(a);
+  auto k = k_split_full<R, LOCAL, AFFINE, TB, BAND>;
+  k<<<grid, FULL_WARPS * 32, full_smem_bytes(R, a.f.sp.alphabet), st>>>(a);
   return cudaGetLastError();
 }
-template <bool LOCAL, bool AFFINE, bool TB, bool BAND>
+template <int R, bool LOCAL, bool AFFINE, bool TB, bool BAND>
 int occ_sf(const ScoreParams &sp) {
   int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_split_full<LOCAL, AFFINE, TB, BAND>, FULL_WARPS * 32,
-                                                full_smem_bytes(SPLIT_R, sp.alphabet));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_split_full<R, LOCAL, AFFINE, TB, BAND>, FULL_WARPS * 32,
+                                                full_smem_bytes(R, sp.alphabet));
   return nb;
 }
 
@@ -121,20 +119,26 @@ int occ_sf(const ScoreParams &sp) {
   X(true, true, false, false) X(true, true, false, true) X(true, true, true, false) \
   X(true, true, true, true)
 
-cudaError_t launch_split_full(const SplitArgs &a, int grid, cudaStream_t st) {
+cudaError_t launch_split_full(const SplitArgs &a, int R, int grid, cudaStream_t st) {
   const ScoreParams &sp = a.f.sp;
   const bool L = sp.mode == FILTR_LOCAL, AF = sp.affine != 0, T = sp.traceback != 0, B = sp.use_band != 0;
 #define FILTR_CASE(l, af, t, b) \
-  if (L == l && AF == af && T == t && B == b) return launch_sf<l, af, t, b>(a, grid, st);
+  if (L == l && AF == af && T == t && B == b) { \
+    if (R == 4 && b) return launch_sf<b ? 4 : 8, l, af, t, b>(a, grid, st); \
+    if (R == 8) return launch_sf<8, l, af, t, b>(a, grid, st); \
+  }
   FILTR_SPLIT_CASES(FILTR_CASE)
 #undef FILTR_CASE
   return cudaErrorInvalidValue;
 }
 
-int split_full_blocks_per_sm(const ScoreParams &sp) {
+int split_full_blocks_per_sm(int R, const ScoreParams &sp) {
   const bool L = sp.mode == FILTR_LOCAL, AF = sp.affine != 0, T = sp.traceback != 0, B = sp.use_band != 0;
 #define FILTR_CASE(l, af, t, b) \
-  if (L == l && AF == af && T == t && B == b) return occ_sf<l, af, t, b>(sp);
+  if (L == l && AF == af && T == t && B == b) { \
+    if (R == 4 && b) return occ_sf<b ? 4 : 8, l, af, t, b>(sp); \
+    if (R == 8) return occ_sf<8, l, af, t, b>(sp); \
+  }
   FILTR_SPLIT_CASES(FILTR_CASE)
 #undef FILTR_CASE
   return 0;

@@ -28,7 +28,7 @@
 // Traceback: 4 bits per cell, each the sign of a difference shifted into the
 // lane's word (tb_push4): E > D, F > max(D, E), E took the extension, F took the
 // extension.  Cell k of a word ends in bits [4*(7 - k), 4*(7 - k) + 4).  Per
-// strip: step-major, then word (R/8 per lane), then lane.
+// strip: step-major, then word (R/8 per lane, half of one for R = 4), then lane.
 #pragma once
 
 #include <climits>
@@ -41,6 +41,10 @@ constexpr unsigned STRIP_FULLMASK = 0xffffffffu;
 
 template <int R>
 struct ProfWord;
+template <>
+struct ProfWord<4> {
+  using T = uint32_t;
+};
 template <>
 struct ProfWord<8> {
   using T = uint2;
@@ -140,7 +144,7 @@ __device__ __forceinline__ void strip_pass(const StripPair &P, int s, int jlo, i
                                            int prev_jhi, int64_t tb_base, IO &io, LaneBest &best,
                                            int &endH) {
   constexpr int HS = 32 * R;
-  constexpr int WPS = R / 8;
+  constexpr int WPS = (R + 7) / 8;
   using PW = typename ProfWord<R>::T;
   const int lane = threadIdx.x & 31;
   const int M = P.M, lo = P.lo, hi = P.hi, o = P.o, e = P.e;
@@ -311,6 +315,7 @@ __device__ __forceinline__ void strip_pass(const StripPair &P, int s, int jlo, i
       upF = Fup;
       prevIn = inH;
       if (TB) {
+        if constexpr (R % 8 != 0) tbw[WPS - 1] <<= 4 * (8 - R % 8);  // cell k's nibble stays at its place
 #pragma unroll
         for (int w = 0; w < WPS; ++w) P.tb[tb_base + ((int64_t)t * WPS + w) * 32 + lane] = tbw[w];
       }

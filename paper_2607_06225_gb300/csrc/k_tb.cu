@@ -81,7 +81,7 @@ __device__ __forceinline__ uint32_t full_bits(const uint32_t *tb, FullGeom &g, i
   const int l = rho / g.R, k = rho - l * g.R;
   const int64_t t = (int64_t)j - g.jlo + l;
   if (t < 0 || t >= g.nsteps) return 0;  // never taken on a consistent traceback
-  const int wps = g.R / 8;
+  const int wps = (g.R + 7) / 8;
   const uint32_t w = __ldg(tb + g.base + (t * wps + (k >> 3)) * 32 + l);
   return tb_nibble(w, k);
 }
@@ -366,7 +366,7 @@ struct TileLoader {
       }
       t = j0 - jlo + l;
       at = base + (k >> 3) * 32 + l;
-      stride = 4 * R;
+      stride = (R + 7) / 8 * 32;
       sub = 4 * (7 - (k & 7));
     }
     const uint32_t *w = tb + at + (int64_t)t * stride;

@@ -54,17 +54,27 @@ filtr_status validate_seq(Ctx *c, const uint8_t *q, uint32_t M, const uint8_t *r
 }
 
 // a warp per row strip of the int32 tile (k_split.cuh); withhold != 0 is the timeout test
-filtr_status run_long(Ctx *c, const ScoreParams &sp, const filtr_params *params, const uint8_t *q,
-                      uint32_t M, const uint8_t *r, uint32_t N, filtr_result *out, uint32_t *cigar,
-                      uint64_t cap, cudaStream_t st, int withhold, unsigned long long timeout_ns,
-                      bool sync = true) {
-  (void)params;
-  constexpr int R = 8, HS = 32 * R;
+filtr_status run_long(Ctx *c, const ScoreParams &sp, const uint8_t *q, uint32_t M, const uint8_t *r,
+                      uint32_t N, filtr_result *out, uint32_t *cigar, uint64_t cap, cudaStream_t st,
+                      int withhold, unsigned long long timeout_ns, bool sync = true, int R = 8) {
+  const int HS = 32 * R;
   int64_t widest = N;
   if (sp.use_band) {
     int64_t lo, hi;
     band_limits(M, N, sp.band, sp.band_literal, &lo, &hi);
     widest = std::max<int64_t>(1, std::min<int64_t>(N, hi - lo + HS));
+    // A banded strip starts when the one above is a strip's height further, so the
+    // pair's time is the steps down its rows: strips of 4 rows per lane take 159
+    // cheaper steps (0.27 us) for 128 rows where strips of 8 take 287 of 0.32 us for 256:
+    // forward sweep of an 80 kbp pair with a 7 kbp wide band 31.3 -> 29.1 ms, its walk
+    // over more strips 7.2 -> 7.7.  Not where a wide band keeps more than a warp per
+    // scheduler busy, nor where the traceback (up to twice as much) does not fit.
+    if (R == 8 && widest / 128 + 6 <= 4 * (int64_t)c->sms) {
+      const uint64_t need = split_space(1, ((uint64_t)M + 127) / 128, (uint64_t)widest + 1).bytes +
+                            (sp.traceback ? 4 * (full_tb_words(M, N, 4, sp) + M + N) : 0) + 8192;
+      if (need <= c->ws_bytes)
+        return run_long(c, sp, q, M, r, N, out, cigar, cap, st, withhold, timeout_ns, sync, 4);
+    }
   }
   const uint32_t nstrips = (uint32_t)((M + (uint64_t)HS - 1) / HS);
   const uint64_t tb_words = sp.traceback ? full_tb_words(M, N, R, sp) : 0;
@@ -99,7 +109,7 @@ filtr_status run_long(Ctx *c, const ScoreParams &sp, const filtr_params *params,
   TbLayout L{};
   L.off = 0;
   L.family = FAM_FULL;
-  L.R = R;
+  L.R = (uint8_t)R;
   L.warps = 1;
   L.valid = sp.traceback ? 1 : 0;
   uint64_t misc[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // stage_off, q_off, r_off
@@ -183,7 +193,6 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
                             const uint8_t *q, uint32_t M, const uint8_t *r, uint32_t N,
                             filtr_result *out, uint32_t *cigar, uint64_t cap, cudaStream_t st,
                             int C) {
-  (void)params;
   const int64_t K = (int64_t)M + N;
   const int64_t nseg = (K + C - 1) / C;
   static const int kLadder[] = {1, 2, 4, 8, 16, XD_MAX_WARPS};
@@ -451,7 +460,7 @@ filtr_status long_pair_async(Ctx *c, const ScoreParams &sp, const filtr_params *
   c->ev_used = 0;
   c->spans.clear();
   const filtr_status rc =
-      run_long(c, sp, params, q, M, r, N, out, cigar, cap, st, 0, SPLIT_TIMEOUT_NS, false);
+      run_long(c, sp, q, M, r, N, out, cigar, cap, st, 0, SPLIT_TIMEOUT_NS, false);
   if (!c->done_ev) cudaEventCreateWithFlags(&c->done_ev, cudaEventDisableTiming);
   if (c->done_ev) cudaEventRecord(c->done_ev, st);
   return rc;
@@ -525,7 +534,7 @@ filtr_status filtr_align_long(filtr_ctx *ctx, const filtr_params *params, const 
     c->xdrop_warps0 = w0;
     return rc;
   }
-  rc = run_long(c, sp, params, q, M, r, N, out, cigar, cigar_cap, st, 0, SPLIT_TIMEOUT_NS);
+  rc = run_long(c, sp, q, M, r, N, out, cigar, cigar_cap, st, 0, SPLIT_TIMEOUT_NS);
   if (!c->done_ev) cudaEventCreateWithFlags(&c->done_ev, cudaEventDisableTiming);
   if (c->done_ev) cudaEventRecord(c->done_ev, st);
   return rc;
@@ -601,7 +610,7 @@ filtr_status filtr_test_long_timeout(filtr_ctx *ctx, const filtr_params *params,
   if (c->done_ev) cudaEventSynchronize(c->done_ev);
   sp.traceback = 0;
   filtr_result *d_out = reinterpret_cast<filtr_result *>(c->d_small + 2048);
-  rc = run_long(c, sp, params, q, M, r, N, d_out, nullptr, 0, c->own_stream, 1, timeout_ns);
+  rc = run_long(c, sp, q, M, r, N, d_out, nullptr, 0, c->own_stream, 1, timeout_ns);
   return rc;
 }
 

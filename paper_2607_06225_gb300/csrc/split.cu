@@ -185,7 +185,7 @@ cudaError_t launch_split(const SplitLaunch &l, cudaStream_t st) {
   cudaError_t e = cudaGetLastError();
   const int grid = std::min(l.grid, SPLIT_MAX_WARPS / FULL_WARPS);
   if (e == cudaSuccess)
-    e = l.packed ? launch_split_pack(l.a, l.R, grid, st) : launch_split_full(l.a, grid, st);
+    e = l.packed ? launch_split_pack(l.a, l.R, grid, st) : launch_split_full(l.a, l.R, grid, st);
   if (e != cudaSuccess) return e;
   k_split_finish<<<(unsigned)std::min<int64_t>((l.count + 3) / 4, 1 << 16), 128, 0, st>>>(l.a, pa.rows);
   return cudaGetLastError();

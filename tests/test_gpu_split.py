@@ -162,3 +162,40 @@ def test_tall_pair_in_a_batch(F, ctx):
     got = run(F, ctx, b, sc, 0)
     assert ctx.last_stats()["device_plan"] == 0
     same(got, run(F, ctx, b, sc, 1))
+
+
+@pytest.mark.parametrize("mode,gaps", [("global", dict(affine=True, gap_open=4, gap_extend=2)),
+                                       ("global", dict(affine=False, gap_extend=3)),
+                                       ("local", dict(affine=True, gap_open=11, gap_extend=1))])
+@pytest.mark.parametrize("band,literal", [(0, False), (3, False), (40, True), (300, False)])
+def test_long_banded_low_strips(F, ctx, mode, gaps, band, literal):
+    """One banded pair in strips of 128 rows: heights at the edges of one, two and
+    five strips, bands narrower and wider than a strip."""
+    for m, n in [(1, 1), (4, 60), (127, 127), (128, 140), (129, 100), (257, 257), (640, 650), (641, 641)]:
+        b = pairs(4, 900 + m, [(m, n)])
+        q, r = b.pair(0)
+        sc = dict(mode=mode, traceback=True, band=band, band_literal=literal, **gaps)
+        res, cig, rc = F.align_long(ctx, F.make_params(DNA_S, **sc), q, r)
+        assert rc == 0, F.last_error()
+        o = oracle.align(q, r, DNA_S, **sc)
+        for f in ("score", "q_begin", "r_begin", "q_end", "r_end", "status", "cells"):
+            assert int(res[f]) == int(o[f]), (m, n, f, int(res[f]), int(o[f]))
+        assert np.array_equal(cig, o["cigar"]), (m, n)
+
+
+def test_long_banded_either_height(F):
+    """A workspace that holds the traceback of 256-row strips but not of 128-row ones."""
+    b = pairs(4, 77, [(20000, 20000)])
+    q, r = b.pair(0)
+    prm = F.make_params(DNA_S, mode="global", affine=True, gap_open=4, gap_extend=2, band=64,
+                        traceback=True)
+    out = []
+    for ws in (64 << 20, 5 << 20):  # the two heights need 5.9 and 4.3 MB
+        c = F.Context(0, ws)
+        try:
+            res, cig, rc = F.align_long(c, prm, q, r)
+            assert rc == 0, F.last_error()
+            out.append((res.tobytes(), cig.tobytes()))
+        finally:
+            c.close()
+    assert out[0] == out[1]

@@ -324,7 +324,7 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   int split = SPLIT_NONE;
   const bool may_split = !plain && !sp.use_xdrop && !costs && ctx->split_mode != 1 &&
                          (ctx->split_mode == 2 || n <= (sp.use_band ? SPLIT_MAX_BANDED : SPLIT_MAX_PAIRS));
-  if (may_split && (ctx->split_mode == 2 || sp.use_band || n <= SPLIT_LATENCY_PAIRS))
+  if (may_split && (ctx->split_mode == 2 || n <= SPLIT_LATENCY_PAIRS))
     split = n <= SPLIT_LATENCY_PAIRS ? SPLIT_PACK8 : SPLIT_PACK8_16;
   if (!costs) costs = kDefaultShapeCost;
 
@@ -510,10 +510,13 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     n_main = at;
   }
   const bool dev_split = dev_plan && split != SPLIT_NONE && !one_strip;
-  // unbanded pairs planned a warp each, one of which would outlast the others:
-  // planned again on the host, a warp per strip
-  const bool tall = dev_plan && may_split && split == SPLIT_NONE && max_m > SPLIT_TALL_ROWS &&
-                    (double)max_m * (double)max_n > 2.0 * (double)dsum.cells / (10.0 * ctx->sms);
+  // pairs planned a warp each, one of which would take a large part of the batch's
+  // time: planned again on the host, a warp per strip (the rule: k_split.cuh)
+  const double share = (double)dsum.cells / (10.0 * ctx->sms);  // a warp's cells
+  const double wide = std::min((double)max_n, 2.0 * (double)sp.band + 1.0);
+  const bool tall = dev_plan && may_split && split == SPLIT_NONE &&
+                    (sp.use_band ? max_m > SPLIT_BAND_ROWS && (double)max_m * wide > 0.5 * share
+                                 : max_m > SPLIT_TALL_ROWS && (double)max_m * (double)max_n > 2.0 * share);
   if (tall) split = SPLIT_PACK8_16;
   if (dev_plan && !tall && (!sp.traceback || dsum.tb_words <= tb_budget) &&
       (!dev_split || split_fits(w.groups, sp.traceback ? dsum.tb_words : 0, &split_words))) {

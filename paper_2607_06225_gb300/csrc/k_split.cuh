@@ -47,18 +47,30 @@ constexpr int SPLIT_SLOTS = 2;
 constexpr int SPLIT_TAG = 53;              // the tag's first bit
 constexpr int SPLIT_TURNS = 2047;
 constexpr int SPLIT_MAX_WARPS = 2 * SPLIT_TURNS - 16;
-// Which batches run a warp per strip.  Banded ones of up to SPLIT_MAX_BANDED pairs
-// (reads of 0.1-20 kb, band 256, whole calls: 64 reads 62.5 -> 13.5 ms, 512 reads
-// 36.7 -> 16.4, 4000 reads 70.6 -> 28.2; beyond, the slots' memory decides).
-// Unbanded ones of up to SPLIT_LATENCY_PAIRS (64 protein pairs of 100-1000: 3.74 ->
-// 0.57 ms; from 608 pairs the packed tile's taller strips are as fast or faster,
-// 0.73 against 0.85 ms), or up to SPLIT_MAX_PAIRS when the tallest pair has more
-// than SPLIT_TALL_ROWS rows and would outlast the batch (twice a warp's share).
+// Which batches run a warp per strip (whole calls, plain against split).
+// Up to SPLIT_LATENCY_PAIRS, whose shapes the plain path launches one after the other:
+// 64 protein pairs of 100-1000 3.74 / 0.57 ms, 16 banded pairs of 100-600 0.55 / 0.22.
+// More pairs are planned on the device and their shapes run side by side: unbanded ones
+// split up to SPLIT_MAX_PAIRS when the tallest pair has more than SPLIT_TALL_ROWS rows
+// and would outlast the batch (twice a warp's share; 608 pairs of 100-1000 0.73 / 0.85),
+// banded ones up to SPLIT_MAX_BANDED from SPLIT_BAND_ROWS rows and half a warp's share
+// (256 of 100-1500, band 256, traceback 2.02 / 1.27 ms, 3000 of them 4.26 / 3.14; but
+// 3000 scores of 100-600 0.56 / 0.62 and 20,000 of 100-1500 8.29 / 9.15).
 constexpr unsigned long long SPLIT_TIMEOUT_NS = 20ull * 1000 * 1000 * 1000;  // 20 s without progress
-constexpr uint32_t SPLIT_MAX_BANDED = 65536;
+constexpr uint32_t SPLIT_LATENCY_PAIRS = 255;
 constexpr uint32_t SPLIT_MAX_PAIRS = 4096;
-constexpr uint32_t SPLIT_LATENCY_PAIRS = 256;
 constexpr uint32_t SPLIT_TALL_ROWS = 2048;
+constexpr uint32_t SPLIT_MAX_BANDED = 16384;
+constexpr uint32_t SPLIT_BAND_ROWS = 1408;
+// Captured pipelines run their shapes side by side and know only bounds.  Plain against
+// split, local pairs with traceback: 64 of up to 700 0.39 / 0.36 ms, of up to 2000
+// 1.59 / 0.96; 256 of up to 1000 0.62 / 0.82, of up to 2000 2.03 / 1.57; banded (256):
+// 16 of up to 300 0.26 / 0.25, 256 of up to 600 0.55 / 0.64, of up to 1500 2.09 / 1.67.
+inline bool split_graph(bool band, uint32_t max_pairs, uint32_t max_len) {
+  if (max_pairs <= 64) return band || max_len > 1024;
+  return band ? max_pairs <= SPLIT_MAX_PAIRS && max_len > 1024
+              : max_pairs <= SPLIT_LATENCY_PAIRS && max_len > 1408;
+}
 
 struct SplitArgs {
   FullArgs f;                  // batch, parameters, outputs, traceback (order, counter unused)

@@ -199,3 +199,14 @@ def test_long_banded_either_height(F):
         finally:
             c.close()
     assert out[0] == out[1]
+
+
+@pytest.mark.parametrize("n", [255, 256, 300])
+def test_banded_batch_with_tall_pairs(F, ctx, n):
+    """The default choice around the size where batches are planned on the device:
+    many low banded pairs and a few tall ones, against the warp-per-pair kernels."""
+    rng = np.random.default_rng(n)
+    sizes = [(int(m), int(m) + 5) for m in rng.integers(40, 300, n - 3)] + [(3000, 2990), (2050, 2100), (1409, 1400)]
+    b = pairs(4, 31 + n, sizes)
+    sc = dict(mode="global", affine=True, gap_open=4, gap_extend=2, band=50, traceback=True)
+    same(run(F, ctx, b, sc, 0), run(F, ctx, b, sc, 1))

@@ -88,7 +88,7 @@ enum {
   FILTR_ST_UNREACHABLE = 2, /* literal band excludes (M,N) (global) */
   FILTR_ST_EMPTY = 3,       /* local best score is 0: empty alignment */
   FILTR_ST_TOO_WIDE = 4,    /* X-drop region wider than the kernel window (see filtr_align_batch) */
-  FILTR_ST_TIMEOUT = 5      /* a bounded wait of the intra-pair kernel ran out (no result) */
+  FILTR_ST_TIMEOUT = 5      /* a bounded wait between a pair's row strips ran out (no result) */
 };
 
 /* Table 1's own affine form: M(i,j) = max(M, I, D)(i-1, j-1) + s, I and D open
@@ -251,9 +251,9 @@ filtr_status filtr_align_batch_noalloc(const filtr_params *params, uint32_t n_pa
  *   q, r : DEVICE codes (M, N up to 2^31-1);  out : DEVICE, one filtr_result;
  *   cigar: DEVICE, cigar_cap ops.
  * X-drop pairs run as one antidiagonal sweep with checkpointed traceback: every
- * `C`-th antidiagonal's state is kept, and the backward pass recomputes one
- * segment at a time, so the traceback memory is bounded by the workspace.
- * Band / full-matrix pairs split the query into row strips of 256 rows, one
+ * `C`-th antidiagonal's state is kept, and the segments that the path crosses are
+ * recomputed, side by side where the workspace holds them, else one at a time.
+ * Band / full-matrix pairs split the query into row strips of 256 rows (banded ones also 128), one
  * warp per strip at a time, which hand their bottom rows down through global
  * memory in self-tagged words; every wait is bounded and a timeout returns
  * FILTR_ERR_TIMEOUT.  Pairs with M <= 512 or M * N < 2^22
@@ -331,13 +331,13 @@ typedef struct {
  *           unit-cost global alignment score: match 0, mismatch -1, gap 1 per
  *           residue), q_begin = r_begin = 0, q_end = M, r_end = N, status
  *           FILTR_ST_OK, cells = wavefront entries evaluated (the sum over scores
- *           of the domain's width)
+ *           of the domain's width, whether or not all of them could matter)
  *   cigar : DEVICE, cigar_cap ops (may be NULL without traceback); CIGARs in
  *           pair order, FILTR_ERR_CIGAR_CAP as filtr_align_batch.
  * The call reads the lengths back once (a short synchronisation on `stream`);
- * with traceback it also reads back each pair's wavefront storage (a second
- * synchronisation) and recomputes the pairs with every wavefront kept, in
- * waves that fit the workspace.  FILTR_ERR_INVALID for NULL pointers,
+ * with traceback it also reads back the CIGAR total (a second synchronisation).
+ * Wavefronts are kept in the workspace; pairs whose wavefronts outgrow a warp's
+ * share of it are computed again, in waves that fit.  FILTR_ERR_INVALID for NULL pointers,
  * negative adapt thresholds, an alphabet other than 0 or 4, or (alphabet 4) a
  * code >= 4; FILTR_ERR_UNSUPPORTED when a pair has
  * M + N > FILTR_SEARCH_MAX_LEN (its sequences are staged in shared memory);
@@ -386,8 +386,8 @@ typedef struct {
  *   partner         : DEVICE, int32 per base at the base's own offset (same
  *                     layout as seq): its partner's index within the sequence,
  *                     or -1 (required with traceback, else may be NULL)
- * One synchronisation (codes and lengths); each sequence's triangle
- * (n(n+1)/2 words) lives in the context's workspace, in waves of sequences that
+ * One synchronisation (codes and lengths); each sequence's table
+ * (about 2 n^2 bytes, or n(n+1)/2 words where that does not fit) lives in the workspace, in waves of sequences that
  * fit.  FILTR_ERR_INVALID for NULL pointers, negative parameters or a code >= 4;
  * FILTR_ERR_UNSUPPORTED for a sequence over FILTR_FOLD_MAX_LEN; FILTR_ERR_NOMEM
  * when one triangle does not fit the workspace. */

@@ -837,6 +837,7 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
   const uint32_t ring_cap = ctx->search_ring > 0 ? (uint32_t)ctx->search_ring : 64u;
   a.ring_c = 32;
   while (a.ring_c < a.ring_half && a.ring_c < ring_cap) a.ring_c <<= 1;
+  while (a.ring_c > 32 && (uint64_t)(a.q_words + a.r_words + 2 * a.ring_c) * 4 > 227 * 1024) a.ring_c >>= 1;
   LaunchCfg cfg_score, cfg_tb;
   auto k_score = tb ? (p2 ? k_search_score<true, true> : k_search_score<false, true>)
                     : (p2 ? k_search_score<true, false> : k_search_score<false, false>);

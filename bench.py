@@ -6,13 +6,13 @@ reference, seeded 20x20 substitution matrix, affine gaps (open 11, extend 1),
 local alignment, score + end coordinates + CIGAR.  Metric: GCUPS (cells whose
 recurrence was evaluated / second), inputs resident in HBM.
 
-Also reported on the same JSON line: the same call through the host-buffer
-entry point (e2e), the plain one-launch-per-pair form and the whole-GPU
-per-pair form (filtr_align_long) on samples, the roofline of the forward
-kernels against the measured integer throughput of their cell widths, the CPU
-oracle on a bounded sample (its results compared with the GPU's), SM clocks
-sampled during the timed region, and under "configs" the same record for the
-short-DNA, long-read and megabase-pair workloads.
+Also measured: the same call through the host-buffer entry point (e2e), the plain
+one-launch-per-pair form and the whole-GPU per-pair form (filtr_align_long) on
+samples, the roofline of the forward kernels against the measured integer
+throughput of their cell widths, the CPU oracle on a bounded sample (its results
+compared with the GPU's), SM clocks sampled during the timed region, and under
+"configs" the same record for the short-DNA, long-read and megabase-pair workloads.
+The whole record goes to stderr; stdout gets one JSON line of its main figures.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 """
@@ -826,6 +826,42 @@ def plain_long_per_pair(F, ctx, params, batch, nsample, stream, dev, res):
             "call": "filtr_align_long per pair (intra-pair kernel on every SM)"}
 
 
+def printed_line(rec):
+    """The record's printed form, one line of at most 2,900 characters (what reads it
+    may keep only the last 3,000 of a program's output): the workload's own figures in
+    full, one or two figures of every other measurement.  The whole record goes to
+    stderr."""
+    def rounded(x):
+        if isinstance(x, float):
+            return float(f"{x:.6g}")
+        if isinstance(x, dict):
+            return {k: rounded(v) for k, v in x.items()}
+        return [rounded(v) for v in x] if isinstance(x, list) else x
+
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else d
+
+    out = pick(rec, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+               "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "e2e",
+               "gpu_launches", "clocks")
+    out["phases_ms"] = pick(rec.get("phases_ms"), "forward", "walk")
+    out["roofline"] = pick(rec.get("roofline"), "bound", "kernel", "achieved", "peak", "unit", "frac",
+                           "traffic")
+    for key, keys in (("plain_per_pair", ("pairs", "gcups_plain", "gcups_batched_same_pairs")),
+                      ("plain_long_per_pair", ("pairs", "gcups")), ("graph", ("value", "ms_per_step")),
+                      ("cpu_baseline", ("value", "cores", "kind"))):
+        if rec.get(key):
+            out[key] = pick(rec[key], *keys)
+    if rec.get("serving"):
+        s = rec["serving"]
+        out["serving"] = dict(pick(s, "capacity_gcups", "load_frac_of_capacity", "p50_ms", "p99_ms", "refused"),
+                              fixed_rate=pick(s["fixed_rate"], "offered_rate_hz", "p50_ms", "p99_ms"))
+    if rec.get("configs"):
+        out["configs"] = {w: dict(pick(r, "value", "ms_per_step"), e2e=r["e2e"]["value"])
+                          for w, r in rec["configs"].items()}
+    return json.dumps(rounded(out))
+
+
 def measure_workload(F, ctx, synth, wl, args, steps, warmup, stream, flush, dev, rank, world, dist,
                      probe):
     """One workload: untimed setup and warm-up, `steps` timed steps (CUDA events,
@@ -1059,7 +1095,8 @@ def main():
         if rank == 0:
             line["configs"] = subs
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(printed_line(line), flush=True)
     if dist:
         dist.barrier()
         dist.destroy_process_group()

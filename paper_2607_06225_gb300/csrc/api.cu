@@ -361,6 +361,10 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     pa.n = n;
     pa.sp = sp;
     pa.tab = make_shape_table(costs, sp, split);
+    if (may_split && split == SPLIT_NONE && sp.traceback) {  // what a warp per strip would keep
+      pa.ref_tab = make_shape_table(costs, sp, SPLIT_PACK8_16);
+      pa.use_ref = 1;
+    }
     pa.state = d_ps;
     pa.key = d_pkey;
     pa.words = d_pwords;
@@ -464,15 +468,18 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   // never needs workspace that a plain one did not.
   const uint32_t split_stride = (uint32_t)max_n + 1;
   SplitSpace split_spc[SHAPE_TILED];
+  auto plain_refuses = [&]() -> bool {  // a pair the plain shapes may refuse for its traceback: they decide
+    if (!sp.traceback) return false;
+    ScoreParams full = sp;
+    full.use_band = 0;
+    const ShapeTable plain_tab = make_shape_table(costs, sp);
+    for (int i = 0; i < plain_tab.n_elig; ++i)
+      if (shape_tb_words(plain_tab, plain_tab.elig[i], (uint32_t)max_m, (uint32_t)max_n, full) > tb_budget)
+        return true;
+    return false;
+  };
   auto split_fits = [&](const std::vector<Group> &groups, uint64_t tb_words, uint64_t *words) -> bool {
-    if (sp.traceback) {  // a pair the plain shapes may refuse for its traceback: they decide
-      ScoreParams full = sp;
-      full.use_band = 0;
-      const ShapeTable plain_tab = make_shape_table(costs, sp);
-      for (int i = 0; i < plain_tab.n_elig; ++i)
-        if (shape_tb_words(plain_tab, plain_tab.elig[i], (uint32_t)max_m, (uint32_t)max_n, full) > tb_budget)
-          return false;
-    }
+    if (plain_refuses()) return false;
     size_t bytes = 0;
     for (size_t g = 0; g < groups.size(); ++g) {
       const uint64_t rows = split_rows(groups[g].family == FAM_PACK, groups[g].R);
@@ -483,6 +490,17 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     }
     *words = (bytes + 3) / 4;
     return bytes <= ctx->ws_bytes / 4 && tb_words + *words + 64 <= tb_budget;
+  };
+  // The same from the device plan's totals, before that plan is given up: the pairs
+  // in one launch of the lowest strips take no less room than spread over the shapes
+  // (but for the parts' rounding, one shape's worth each).
+  auto split_would_fit = [&]() -> bool {
+    const uint64_t ns = (max_m + split_rows(false, 8) - 1) / split_rows(false, 8);
+    if (plain_refuses() || ns > SPLIT_MAX_STRIPS) return false;
+    const size_t bytes =
+        split_space(n, ns, split_stride).bytes + (SHAPE_TILED - 1) * split_space(1, ns, 0).bytes;
+    const uint64_t tb_words = sp.traceback ? dsum.tb_words_ref : 0;
+    return bytes <= ctx->ws_bytes / 4 && tb_words + (bytes + 3) / 4 + 64 <= tb_budget;
   };
   uint64_t split_words = 0;
   // one strip each: nothing to split (and 8 rows per lane is the shape of such pairs anyway)
@@ -511,12 +529,15 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   }
   const bool dev_split = dev_plan && split != SPLIT_NONE && !one_strip;
   // pairs planned a warp each, one of which would take a large part of the batch's
-  // time: planned again on the host, a warp per strip (the rule: k_split.cuh)
+  // time: planned again on the host, a warp per strip (the rule: k_split.cuh), unless
+  // the workspace would not hold that: the device's plan, whose shapes run side by
+  // side, is the faster one then
   const double share = (double)dsum.cells / (10.0 * ctx->sms);  // a warp's cells
   const double wide = std::min((double)max_n, 2.0 * (double)sp.band + 1.0);
   const bool tall = dev_plan && may_split && split == SPLIT_NONE &&
                     (sp.use_band ? max_m > SPLIT_BAND_ROWS && (double)max_m * wide > 0.5 * share
-                                 : max_m > SPLIT_TALL_ROWS && (double)max_m * (double)max_n > 2.0 * share);
+                                 : max_m > SPLIT_TALL_ROWS && (double)max_m * (double)max_n > 2.0 * share) &&
+                    split_would_fit();
   if (tall) split = SPLIT_PACK8_16;
   if (dev_plan && !tall && (!sp.traceback || dsum.tb_words <= tb_budget) &&
       (!dev_split || split_fits(w.groups, sp.traceback ? dsum.tb_words : 0, &split_words))) {

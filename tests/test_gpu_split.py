@@ -210,3 +210,25 @@ def test_banded_batch_with_tall_pairs(F, ctx, n):
     b = pairs(4, 31 + n, sizes)
     sc = dict(mode="global", affine=True, gap_open=4, gap_extend=2, band=50, traceback=True)
     same(run(F, ctx, b, sc, 0), run(F, ctx, b, sc, 1))
+
+
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("kind", ["local", "band"])
+def test_tall_pair_without_room_for_strips(F, kind, tb):
+    """A tall pair in a batch whose hand-over slots (301 pairs x 2 slots of 4001 words,
+    19.3 MB) exceed a quarter of the workspace: the device's plan, whose shapes run
+    side by side, is kept, and with room for the slots it is given up."""
+    rng = np.random.default_rng(13)
+    sizes = [(5000, 4000)] + [(int(rng.integers(100, 400)), int(rng.integers(100, 400))) for _ in range(300)]
+    sc = dict(dict(affine=True, gap_open=11, gap_extend=1, traceback=tb), **KINDS[kind])
+    b = pairs(20, 14, sizes)
+    out = []
+    for ws, planned_on_device in ((64 << 20, 1), (256 << 20, 0)):
+        c = F.Context(0, ws)
+        try:
+            out.append(run(F, c, b, sc, 0))
+            assert c.last_stats()["device_plan"] == planned_on_device
+            same(out[-1], run(F, c, b, sc, 1))
+        finally:
+            c.close()
+    same(out[0], out[1])

@@ -252,7 +252,7 @@ filtr_status filtr_align_batch_noalloc(const filtr_params *params, uint32_t n_pa
  *   cigar: DEVICE, cigar_cap ops.
  * X-drop pairs run as one antidiagonal sweep with checkpointed traceback: every
  * `C`-th antidiagonal's state is kept, and the segments that the path crosses are
- * recomputed, side by side where the workspace holds them, else one at a time.
+ * recomputed side by side, in as many groups as the workspace asks for.
  * Band / full-matrix pairs split the query into row strips of 256 rows (banded ones also 128), one
  * warp per strip at a time, which hand their bottom rows down through global
  * memory in self-tagged words; every wait is bounded and a timeout returns

@@ -45,7 +45,7 @@ struct Ctx {
   uint32_t last_launches = 0;
   int xdrop_warps0 = 0;       // first window width (warps) of X-drop pairs, 0: estimated
   int ckpt_interval = 0;      // > 0: filtr_align_long always checkpoints X-drop tracebacks
-  bool ckpt_recompute = false;  // checkpointed traceback: recompute segments, no single pass
+  bool ckpt_recompute = false;  // checkpointed traceback: one segment at a time (test hook)
   // ordering of successive calls: the next call waits for this event, so the
   // workspace and the pinned staging are never reused while still in flight
   cudaEvent_t done_ev = nullptr;

@@ -271,13 +271,13 @@ cudaError_t launch_xdrop(const FullArgs &a, int W, int grid, uint32_t *overflow,
                          uint32_t *n_overflow, cudaStream_t s);
 int xd_pairs_per_cta(int W, const ScoreParams &sp);
 struct WalkState;
-cudaError_t launch_walk_segment(const WalkArgs &a, const uint32_t *seg_tb, const int32_t *seg_ck,
-                                int k_start, int wpk, WalkState *st, cudaStream_t s);
+// recomputed segments of one long pair (k_tb.cu): their descriptors and group widths
+// by segment, the window origins from antidiagonal k0 + 1 on
+cudaError_t launch_walk_segments(const WalkArgs &a, const struct XdCkpt *seg, const int32_t *width,
+                                 const int32_t *ck, int C, int k0, WalkState *st, cudaStream_t s);
 int xd_max_blocks_per_sm(int W, const ScoreParams &sp);
 cudaError_t launch_walk(const WalkArgs &a, cudaStream_t s);
 cudaError_t launch_walk_xd(const WalkArgs &a, cudaStream_t s);  // X-drop pairs, a warp each
-cudaError_t launch_walk_pool(const WalkArgs &a, const uint32_t *pool, const int32_t *seg_ck_all,
-                             const uint64_t *seg_off, const int32_t *seg_w, int C, cudaStream_t s);
 // In a captured pipeline (gd set) the n given here is the graph's capacity,
 // which sizes the grid; the kernels take the launch's n from gd.
 cudaError_t launch_scan_offsets(const filtr_result *out, uint32_t n, uint64_t *offs,

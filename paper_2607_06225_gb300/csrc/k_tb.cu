@@ -400,28 +400,27 @@ struct TileLoader {
 // Where antidiagonal k's window origin and traceback row live (antidiagonals stay
 // below 2^31).  run(k): row k's words, with those of the rows around it in the
 // range (lo, hi] at multiples of wpk.
-struct XdRows {  // one pair's own layout or a recomputed segment: row = k - row_off
+struct XdRows {  // one pair's own layout
   const int32_t *ck;
   const uint32_t *tb;
-  int wpk, row_off;
+  int wpk;
   int lo, hi;
-  __device__ __forceinline__ int origin(int k) const { return __ldg(ck + (k - row_off)); }
-  __device__ __forceinline__ const uint32_t *run(int k) { return tb + (int64_t)(k - row_off) * wpk; }
+  __device__ __forceinline__ int origin(int k) const { return __ldg(ck + k); }
+  __device__ __forceinline__ const uint32_t *run(int k) { return tb + (int64_t)k * wpk; }
 };
-struct XdPoolRows {  // single-pass segmented sweep: segment s = (k - 1) / C
-  const uint32_t *pool;
-  const int32_t *seg_ck_all;
-  const uint64_t *seg_off;
-  const int32_t *seg_w;
-  int C;
-  int wpk, lo, hi;  // the segment looked up last
+struct XdSegRows {  // recomputed segments, segment s = (k - 1) / C, from antidiagonal k0 + 1 on
+  const XdCkpt *seg;     // by segment: where its rows are
+  const int32_t *width;  // by segment: group width it was computed at
+  const int32_t *ck;     // origins of k0 + 1, k0 + 2, ...
+  int C, k0;
+  int wpk, lo, hi;       // the segment looked up last
   const uint32_t *base;
-  __device__ __forceinline__ int origin(int k) const { return __ldg(seg_ck_all + (k - 1)); }
+  __device__ __forceinline__ int origin(int k) const { return __ldg(ck + (k - 1 - k0)); }
   __device__ __forceinline__ const uint32_t *run(int k) {
     if (k <= lo || k > hi) {
       const int s = (k - 1) / C;
-      wpk = xd_words_per_k(__ldg(seg_w + s), 8);
-      base = pool + __ldg(seg_off + s);
+      wpk = xd_words_per_k(__ldg(width + s), 8);
+      base = seg[s].seg_tb;
       lo = s * C;
       hi = lo + C;
     }
@@ -678,7 +677,7 @@ __global__ void __launch_bounds__(128) k_walk_xdw(const WalkArgs a) {
   w.v = f.score;
   XdLoader<XdRows> ld;
   ld.rows = XdRows{reinterpret_cast<const int32_t *>(base), base + xd_origin_words(M, N),
-                   xd_words_per_k(L.warps, L.R), 0, INT_MIN, INT_MAX};
+                   xd_words_per_k(L.warps, L.R), INT_MIN, INT_MAX};
   ld.k_min = 0;
   ld.k_max = w.i + w.j;
   walk_band(w, ld, band[wib], -1);
@@ -728,12 +727,11 @@ __global__ void __launch_bounds__(128) k_walk_tw(const WalkArgs a) {
   w.store(out + p);
 }
 
-// Resumable walk over one recomputed segment (antidiagonals (k_start, k_end])
-// of a checkpointed X-drop traceback; one warp.  Stops when the walk leaves
-// the segment (the next, earlier segment continues from the saved state) or
-// when the alignment's start is reached.
-__global__ void k_walk_segw(const WalkArgs a, const uint32_t *seg_tb, const int32_t *seg_ck,
-                            int k_start, int wpk, WalkState *ws) {
+// Resumable walk over recomputed segments (antidiagonals above k0) of a
+// checkpointed X-drop traceback; one warp.  Stops when the walk reaches k0 (earlier
+// segments, recomputed next, go on from the saved state) or when the alignment's
+// start is reached.
+__global__ void k_walk_segments(const WalkArgs a, const XdSegRows rows, WalkState *ws) {
   __shared__ WalkBand band;
   __shared__ int8_t s_sub[MAX_ALPHA * MAX_ALPHA];
   load_subst(s_sub, a.sp);
@@ -749,12 +747,12 @@ __global__ void k_walk_segw(const WalkArgs a, const uint32_t *seg_tb, const int3
   w.n = st.n;
   w.cur = st.cur;
   w.run = st.run;
-  XdLoader<XdRows> ld;
-  ld.rows = XdRows{seg_ck, seg_tb, wpk, k_start + 1, INT_MIN, INT_MAX};
-  ld.k_min = k_start;
+  XdLoader<XdSegRows> ld;
+  ld.rows = rows;
+  ld.k_min = rows.k0;
   ld.k_max = w.i + w.j;
-  // (a walk in a gap stops on k_start as well; 0 is the start itself)
-  const bool done = walk_band(w, ld, band, k_start > 0 ? k_start : -1);
+  // (a walk in a gap stops on k0 as well; 0 is the start itself)
+  const bool done = walk_band(w, ld, band, rows.k0 > 0 ? rows.k0 : -1);
   __syncwarp();
   if (done) w.store(a.out + p);
   if (threadIdx.x == 0) {
@@ -769,30 +767,6 @@ __global__ void k_walk_segw(const WalkArgs a, const uint32_t *seg_tb, const int3
     o.run = w.run;
     *ws = o;
   }
-}
-
-// The whole traceback of a single-pass segmented sweep; one warp.
-__global__ void k_walk_poolw(const WalkArgs a, const XdPoolRows rows) {
-  __shared__ WalkBand band;
-  __shared__ int8_t s_sub[MAX_ALPHA * MAX_ALPHA];
-  load_subst(s_sub, a.sp);
-  if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-  const uint32_t p = a.order[0];
-  const FwdOut f = a.fwd[p];
-  if (f.status != FILTR_ST_OK && f.status != FILTR_ST_DROPPED) {
-    if (threadIdx.x == 0) a.out[p].cigar_len = 0;
-    return;
-  }
-  WalkCore w = walk_core(a, a.b, p, s_sub);
-  w.i = f.end_i;
-  w.j = f.end_j;
-  w.v = f.score;
-  XdLoader<XdPoolRows> ld;
-  ld.rows = rows;
-  ld.k_min = 0;
-  ld.k_max = w.i + w.j;
-  walk_band(w, ld, band, -1);
-  w.store(a.out + p);
 }
 
 // Exclusive scan of cigar_len (pair order) into offs; *total = sum.  One CTA.
@@ -887,15 +861,9 @@ cudaError_t launch_walk_xd(const WalkArgs &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_walk_pool(const WalkArgs &a, const uint32_t *pool, const int32_t *seg_ck_all,
-                             const uint64_t *seg_off, const int32_t *seg_w, int C, cudaStream_t s) {
-  k_walk_poolw<<<1, 32, 0, s>>>(a, XdPoolRows{pool, seg_ck_all, seg_off, seg_w, C, 0, 0, 0, nullptr});
-  return cudaGetLastError();
-}
-
-cudaError_t launch_walk_segment(const WalkArgs &a, const uint32_t *seg_tb, const int32_t *seg_ck,
-                                int k_start, int wpk, WalkState *st, cudaStream_t s) {
-  k_walk_segw<<<1, 32, 0, s>>>(a, seg_tb, seg_ck, k_start, wpk, st);
+cudaError_t launch_walk_segments(const WalkArgs &a, const XdCkpt *seg, const int32_t *width, const int32_t *ck,
+                                 int C, int k0, WalkState *st, cudaStream_t s) {
+  k_walk_segments<<<1, 32, 0, s>>>(a, XdSegRows{seg, width, ck, C, k0, 0, 0, 0, nullptr}, st);
   return cudaGetLastError();
 }
 

@@ -198,14 +198,6 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   static const int kLadder[] = {1, 2, 4, 8, 16, XD_MAX_WARPS};
   Carve cv{c->ws, c->ws_bytes};
   int32_t *ck_buf = cv.take<int32_t>((size_t)(nseg + 1) * xd_ckpt_stride());
-  // single pass: every segment of the path is recomputed with traceback at once,
-  // into a pool (the rest of the workspace), and walked once; when the pool does
-  // not hold them, one segment at a time is recomputed and walked
-  const bool single = sp.traceback && !c->ckpt_recompute;
-  uint32_t *seg_tb = (sp.traceback && !single)
-                         ? cv.take<uint32_t>((size_t)C * xd_words_per_k(XD_MAX_WARPS, 8))
-                         : nullptr;
-  int32_t *seg_ck = (sp.traceback && !single) ? cv.take<int32_t>(C) : nullptr;
   XdCkpt *d_ck = cv.take<XdCkpt>(2 * nseg + 1);
   int32_t *d_flags = cv.take<int32_t>(nseg + 1);
   WalkState *d_ws = cv.take<WalkState>(1);
@@ -214,27 +206,21 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   TbLayout *d_tbl = cv.take<TbLayout>(1);
   uint64_t *d_misc = cv.take<uint64_t>(8);   // stage_off, offsets, CIGAR offset
   uint32_t *d_ovf = cv.take<uint32_t>(4);
-  uint32_t *d_stage = sp.traceback ? cv.take<uint32_t>((size_t)M + N + 1) : nullptr;
-  int32_t *seg_ck_all = single ? cv.take<int32_t>((size_t)nseg * C) : nullptr;
-  uint64_t *seg_off = single ? cv.take<uint64_t>(nseg) : nullptr;
-  int32_t *seg_wd = single ? cv.take<int32_t>(nseg) : nullptr;
-  if (cv.used > c->ws_bytes) {
-    set_error("checkpointed traceback needs %zu workspace bytes; the context has %zu", cv.used,
-              c->ws_bytes);
+  // the CIGAR staging at the workspace's end, and what lies between: the pool that
+  // the segments are recomputed into
+  uint32_t *pool = cv.take<uint32_t>(0);
+  const uint64_t stage_words = sp.traceback ? (uint64_t)M + N + 1 : 0;
+  if (cv.used + stage_words * 4 > c->ws_bytes) {
+    set_error("checkpointed traceback needs %llu workspace bytes; the context has %zu",
+              (unsigned long long)(cv.used + stage_words * 4), c->ws_bytes);
     return FILTR_ERR_NOMEM;
   }
-  uint32_t *pool = nullptr;
-  uint64_t pool_words = 0;
-  if (single) {
-    pool = cv.take<uint32_t>(0);
-    pool_words = cv.used < c->ws_bytes ? (c->ws_bytes - cv.used) / 4 : 0;
-  }
-  // host staging: the one-pair batch, the segment descriptors, the flags, and the
-  // segments' places in the pool
+  const uint64_t pool_words = (c->ws_bytes - cv.used) / 4 - stage_words;
+  uint32_t *d_stage = pool + pool_words;
+  // host staging: the one-pair batch, the segment descriptors, the flags
   const size_t desc_off = 4096;
   const size_t flags_off = desc_off + (size_t)(2 * nseg + 1) * sizeof(XdCkpt);
-  const size_t off_off = (flags_off + (size_t)(nseg + 1) * 4 + 63) / 64 * 64;
-  if (!c->ensure_host(off_off + (size_t)nseg * 12 + 64)) return FILTR_ERR_NOMEM;
+  if (!c->ensure_host(flags_off + (size_t)(nseg + 1) * 4 + 64)) return FILTR_ERR_NOMEM;
   char *h = reinterpret_cast<char *>(c->h_stage);
   uint32_t one[16] = {0, M, N};  // order, q_len, r_len
   TbLayout L{};
@@ -305,111 +291,59 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   c->last_xd16 = sp.xd16 ? 1u : 0u;
   c->last_xd16_rerun = 0;
   if (!sp.traceback || (f.status != FILTR_ST_OK && f.status != FILTR_ST_DROPPED)) return FILTR_OK;
-  WalkArgs wp;
-  wp.b = b;
-  wp.sp = sp;
-  wp.order = d_one;
-  wp.n_order = 1;
-  wp.out = out;
-  wp.fwd = d_fwd;
-  wp.tb = nullptr;
-  wp.tbl = d_tbl;
-  wp.stage = d_stage;
-  wp.stage_off = d_misc;
-  const int64_t ke = (int64_t)f.end_i + f.end_j;
-  if (single) {
-    // The forward sweep is one chain, each antidiagonal waiting for the last; the
-    // segments of the path, given their checkpoints, are not.  So the forward goes
-    // without traceback (a megabase pair: 475 ms instead of 579), and all segments
-    // are recomputed with it side by side, a launch per width.
-    const int64_t n_path = (ke + C - 1) / C;
-    uint64_t *h_off = reinterpret_cast<uint64_t *>(h + off_off);
-    int32_t *h_wd = reinterpret_cast<int32_t *>(h_off + nseg);
-    uint64_t words = 0;
-    for (int64_t sgi = 0; sgi < n_path; ++sgi) {
-      h_wd[sgi] = hflags[1 + sgi];
-      if (h_wd[sgi] <= 0) {
-        set_error("checkpointed sweep: segment %lld has no width", (long long)sgi);
+  // The forward sweep is one chain, each antidiagonal waiting for the last; the
+  // segments of the path, given their checkpoints, are not.  So the forward goes
+  // without traceback (a megabase pair: 475 ms instead of 579), and the segments are
+  // recomputed with it side by side, a launch per width, and walked: all at once
+  // where the pool holds them, else in groups, from the path's end backwards.
+  const int64_t ke = (int64_t)f.end_i + f.end_j, n_path = (ke + C - 1) / C;
+  XdCkpt *by_width = hk + nseg;
+  struct SegGroup {  // segments [s0, s1)
+    int64_t s0, s1;
+    int64_t first[7];       // its descriptors of each width
+    const int32_t *ck;      // origins of its antidiagonals
+  };
+  std::vector<SegGroup> groups;
+  int64_t nb = 0;
+  for (int64_t s1 = n_path; s1 > 0;) {
+    int64_t s0 = s1;
+    uint64_t words = 0;  // rows
+    for (; s0 > 0 && !(c->ckpt_recompute && s0 < s1); --s0) {
+      const int W = hflags[s0];  // of segment s0 - 1
+      if (W <= 0) {
+        set_error("checkpointed sweep: segment %lld has no width", (long long)s0 - 1);
         return FILTR_ERR_CUDA;
       }
-      h_off[sgi] = words;
-      words += (uint64_t)C * xd_words_per_k(h_wd[sgi], 8);
+      const uint64_t w = (uint64_t)C * xd_words_per_k(W, 8);
+      if (words + w + (uint64_t)(s1 - s0 + 1) * C > pool_words) break;
+      words += w;
     }
-    if (words > pool_words) {  // one segment at a time instead
-      const bool saved = c->ckpt_recompute;
-      c->ckpt_recompute = true;
-      const filtr_status rc = run_xdrop_ckpt(c, sp, params, q, M, r, N, out, cigar, cap, st, C);
-      c->ckpt_recompute = saved;
-      return rc;
+    if (s0 == s1) {
+      set_error("checkpointed traceback: the workspace of %zu bytes does not hold one segment", c->ws_bytes);
+      return FILTR_ERR_NOMEM;
     }
-    FullArgs ra = fa;
-    ra.sp = sp;  // traceback on
-    ra.out = reinterpret_cast<filtr_result *>(c->d_small + 3072);  // mode 2 writes no result
-    e = cudaMemcpyAsync(seg_off, h_off, n_path * 8, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(seg_wd, h_wd, n_path * 4, cudaMemcpyHostToDevice, st);
-    XdCkpt *hb = hk + nseg;
-    int64_t nb = 0, first[7];
+    SegGroup g{s0, s1, {}, reinterpret_cast<int32_t *>(pool + words)};
+    uint64_t at = 0;
+    for (int64_t s = s0; s < s1; ++s) {
+      hk[s] = XdCkpt{2, C, ck_buf, (int)(s * C), (int)std::min<int64_t>((s + 1) * C, ke), pool + at,
+                     reinterpret_cast<int32_t *>(pool + words) + (s - s0) * C, d_flags};
+      at += (uint64_t)C * xd_words_per_k(hflags[1 + s], 8);
+    }
     for (int wi = 0; wi < 6; ++wi) {
-      first[wi] = nb;
-      for (int64_t sgi = 0; sgi < n_path; ++sgi)
-        if (h_wd[sgi] == kLadder[wi])
-          hb[nb++] = XdCkpt{2, C, ck_buf, (int)(sgi * C), (int)std::min<int64_t>((sgi + 1) * C, ke),
-                            pool + h_off[sgi], seg_ck_all + sgi * C, d_flags};
+      g.first[wi] = nb;
+      for (int64_t s = s0; s < s1; ++s)
+        if (hflags[1 + s] == kLadder[wi]) by_width[nb++] = hk[s];
     }
-    first[6] = nb;
-    if (e == cudaSuccess && nb)
-      e = cudaMemcpyAsync(d_ck + nseg, hb, nb * sizeof(XdCkpt), cudaMemcpyHostToDevice, st);
-    c->span_begin(Ctx::PH_FORWARD, st);
-    for (int wi = 5; wi >= 0 && e == cudaSuccess; --wi) {
-      if (first[wi + 1] == first[wi]) continue;
-      ra.ck = d_ck + nseg + first[wi];
-      ra.n_ck = (uint32_t)(first[wi + 1] - first[wi]);
-      const int per = xd_pairs_per_cta(kLadder[wi], ra.sp);
-      e = launch_xdrop(ra, kLadder[wi], (int)((ra.n_ck + per - 1) / per), d_ovf, d_ovf + 1, st);
-      ++launches;
-    }
-    c->span_end(st);
-    c->span_begin(Ctx::PH_WALK, st);
-    if (e == cudaSuccess) e = launch_walk_pool(wp, pool, seg_ck_all, seg_off, seg_wd, C, st);
-    c->span_end(st);
-    uint64_t *d_offs = d_misc + 4;
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_offs, 0, 8, st);
-    if (e == cudaSuccess) e = launch_compact(wp, 1, d_offs, cigar, cap, out, st);
-    filtr_result *hr = reinterpret_cast<filtr_result *>(h + 1024);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hr, out, sizeof(filtr_result), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "single-pass traceback");
-    c->last_launches = launches + 2;
-    c->last_waves = 1;
-    if (hr->cigar_len > cap) {
-      set_error("the CIGAR needs %u ops, cigar_cap is %llu", hr->cigar_len, (unsigned long long)cap);
-      return FILTR_ERR_CIGAR_CAP;
-    }
-    return FILTR_OK;
+    g.first[6] = nb;
+    groups.push_back(g);
+    s1 = s0;
   }
-  // backward: one segment at a time, from the end cell's antidiagonal down to
-  // 0, each recomputed at the width that completed it going forward
-  WalkState w0{f.end_i, f.end_j, f.score, 0, 0, -1, 0, 0};
+  if (groups.empty()) groups.push_back(SegGroup{0, 0, {}, nullptr});  // the path is the origin alone
   WalkState *hw = reinterpret_cast<WalkState *>(h + 512);
-  *hw = w0;
-  XdCkpt *hb = hk + nseg;
-  std::vector<int> seg_w;
-  int64_t nb = 0;
-  for (int64_t khi = ke; khi > 0;) {
-    const int64_t klo = ((khi - 1) / C) * C;
-    const int W = hflags[1 + klo / C];
-    if (W <= 0) {
-      set_error("checkpointed sweep: segment at antidiagonal %lld has no width", (long long)klo);
-      return FILTR_ERR_CUDA;
-    }
-    hb[nb++] = XdCkpt{2, C, ck_buf, (int)klo, (int)khi, seg_tb, seg_ck, d_flags};
-    seg_w.push_back(W);
-    khi = klo;
-  }
+  *hw = WalkState{f.end_i, f.end_j, f.score, 0, 0, -1, 0, 0};
   e = cudaMemcpyAsync(d_ws, hw, sizeof(WalkState), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && nb)
-    e = cudaMemcpyAsync(d_ck + nseg, hb, nb * sizeof(XdCkpt), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_fail(e, "segment setup");
+    e = cudaMemcpyAsync(d_ck, hk, (nseg + nb) * sizeof(XdCkpt), cudaMemcpyHostToDevice, st);
   FullArgs ra = fa;
   ra.sp = sp;  // traceback on
   ra.out = reinterpret_cast<filtr_result *>(c->d_small + 3072);  // mode 2 writes no result
@@ -424,14 +358,22 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   wa.tbl = d_tbl;
   wa.stage = d_stage;
   wa.stage_off = d_misc;
-  for (int64_t sgi = 0; sgi < nb; ++sgi) {
-    ra.ck = d_ck + nseg + sgi;
-    e = launch_xdrop(ra, seg_w[sgi], 1, d_ovf, d_ovf + 1, st);
-    if (e == cudaSuccess)
-      e = launch_walk_segment(wa, seg_tb, seg_ck, hb[sgi].k_start, xd_words_per_k(seg_w[sgi], 8),
-                              d_ws, st);
-    launches += 2;
-    if (e != cudaSuccess) return cuda_fail(e, "segment recompute");
+  for (const SegGroup &g : groups) {
+    c->span_begin(Ctx::PH_FORWARD, st);
+    for (int wi = 5; wi >= 0 && e == cudaSuccess; --wi) {
+      if (g.first[wi + 1] == g.first[wi]) continue;
+      ra.ck = d_ck + nseg + g.first[wi];
+      ra.n_ck = (uint32_t)(g.first[wi + 1] - g.first[wi]);
+      const int per = xd_pairs_per_cta(kLadder[wi], ra.sp);
+      e = launch_xdrop(ra, kLadder[wi], (int)((ra.n_ck + per - 1) / per), d_ovf, d_ovf + 1, st);
+      ++launches;
+    }
+    c->span_end(st);
+    c->span_begin(Ctx::PH_WALK, st);
+    if (e == cudaSuccess) e = launch_walk_segments(wa, d_ck, d_flags + 1, g.ck, C, (int)(g.s0 * C), d_ws, st);
+    ++launches;
+    c->span_end(st);
+    if (e != cudaSuccess) return cuda_fail(e, "recomputing and walking segments");
   }
   uint64_t *d_offs = d_misc + 4;
   e = cudaMemsetAsync(d_offs, 0, 8, st);
@@ -441,7 +383,7 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "checkpointed traceback");
   c->last_launches = launches + 1;
-  c->last_waves = (int)nb;
+  c->last_waves = (int)groups.size();
   if (hr->cigar_len > cap) {
     set_error("the CIGAR needs %u ops, cigar_cap is %llu", hr->cigar_len, (unsigned long long)cap);
     return FILTR_ERR_CIGAR_CAP;

@@ -175,3 +175,32 @@ def test_traceback_pool_exhausted_falls_back(F, ctx):
     assert np.array_equal(res, big)
     assert np.array_equal(cig, cig_big)
     assert int(res["status"]) in (0, 1)
+
+
+@pytest.mark.parametrize("zdrop", [False, True])
+def test_segments_in_groups(F, ctx, zdrop):
+    """The same pair in workspaces that hold all, some and about one of its segments'
+    tracebacks: the segments go in groups, from the path's end backwards, each group
+    from the checkpoints of the one forward sweep.  (A 400 k antidiagonal sweep has 98
+    segments of 4096, half a megabyte or more each; checkpoints and staging take 15 MB.)"""
+    b = synth.long_pair(length=200_000, seg=100, seed=17, xdrop=400)
+    q, r = b.pair(0)
+    sc = dict(b.scoring)
+    if zdrop:
+        sc.update(xdrop=None, zdrop=1100)
+    params = F.make_params(b.subst, **sc)
+    out, waves = [], []
+    for ws in (1 << 30, 40 << 20, 24 << 20, 17 << 20):
+        c = F.Context(0, ws)
+        try:
+            res, cig, rc = F.align_long(c, params, q, r)
+            if rc == F._lib.ERR_NOMEM and ws == 17 << 20:
+                continue  # not one segment of the width that this sweep needs
+            assert rc == 0, F.last_error()
+            out.append((res.tobytes(), cig.tobytes()))
+            waves.append(c.last_stats()["waves"])
+        finally:
+            c.close()
+    assert all(o == out[0] for o in out[1:])
+    assert int(res["status"]) == 0
+    assert waves[0] == 1 and 1 < waves[1] < 40 and waves[1] < waves[2] < 98, waves

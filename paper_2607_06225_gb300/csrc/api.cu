@@ -123,11 +123,11 @@ filtr_status to_score_params(const filtr_params *p, ScoreParams *sp) {
     sp->smin = std::min(sp->smin, (int32_t)p->subst[t]);
     sp->smax = std::max(sp->smax, (int32_t)p->subst[t]);
   }
-  // one match score and one mismatch score (DNA +2 / -4): the packed sweep
-  // then scores two cells by comparing codes instead of looking them up
-  sp->uni = 1;
+  // DNA with one match score and one mismatch score (+2 / -4): the packed sweep
+  // then scores cells by comparing codes of two bits instead of looking them up
+  sp->uni = p->alphabet == FILTR_ALPHA_DNA ? 1 : 0;
   sp->uni_match = p->subst[0];
-  sp->uni_mismatch = p->alphabet > 1 ? p->subst[1] : 0;
+  sp->uni_mismatch = p->subst[1];
   for (int a = 0; a < p->alphabet; ++a)
     for (int b = 0; b < p->alphabet; ++b)
       if (p->subst[a * p->alphabet + b] != (a == b ? sp->uni_match : sp->uni_mismatch)) sp->uni = 0;

@@ -117,7 +117,7 @@ struct ScoreParams {
   int32_t traceback;
   int32_t precision;           // FILTR_PREC_*
   int32_t smin, smax;          // smallest / largest substitution score
-  int32_t uni, uni_match, uni_mismatch;  // 1: one score on the diagonal, one off it
+  int32_t uni, uni_match, uni_mismatch;  // uni 1: DNA with one score on the diagonal, one off it
   int32_t xd16;                // 1: the antidiagonal sweep runs two cells per register
   int8_t subst[MAX_ALPHA * MAX_ALPHA];
 };

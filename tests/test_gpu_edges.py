@@ -133,3 +133,30 @@ def test_walk_across_long_gaps(F, ctx, kw, alphabet):
     assert rc == 0, F.last_error()
     osc = {k: v for k, v in sc.items() if k != "precision"}
     compare(b, osc, res, cig, *oracle_batch(b, osc), label=str(kw))
+
+
+@pytest.mark.parametrize("mode", ["global", "local"])
+@pytest.mark.parametrize("drop", [dict(xdrop=60), dict(zdrop=60), dict(xdrop=60, band=80)])
+@pytest.mark.parametrize("W", [1, 2, 4])
+def test_one_match_score_over_twenty_letters(F, ctx, W, drop, mode):
+    """A protein matrix with one match and one mismatch score, which the sweep may not
+    treat as DNA: its codes do not fit two bits.  Mutations move codes by four, eight,
+    twelve and sixteen, so that any comparison of low bits alone takes them for matches."""
+    rng = np.random.default_rng(400 + W)
+    subst = np.full((20, 20), -3, np.int8)
+    np.fill_diagonal(subst, 4)
+    qs, rs = [], []
+    for n in (1, 17, 90, 300, 700, 1500):
+        r = rng.integers(0, 20, n).astype(np.uint8)
+        q = np.where(rng.random(n) < 0.15, (r + 4 * rng.integers(1, 5, n)) % 20, r).astype(np.uint8)
+        qs.append(np.concatenate([q[:n // 2], rng.integers(0, 20, n // 60).astype(np.uint8), q[n // 2:]]))
+        rs.append(r)
+    b = synth.pack(qs, rs, 20, subst)
+    sc = dict(mode=mode, affine=True, gap_open=5, gap_extend=2, traceback=True, **drop)
+    assert F.lib().filtr_test_set_first_width(ctx.handle, W) == F.OK
+    try:
+        res, cig, rc = F.align_batch(ctx, F.make_params(b.subst, **sc), b)
+        assert rc == 0, F.last_error()
+        compare(b, sc, res, cig, *oracle_batch(b, sc), label=f"W={W}")
+    finally:
+        F.lib().filtr_test_set_first_width(ctx.handle, 0)

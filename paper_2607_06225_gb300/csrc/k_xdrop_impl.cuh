@@ -157,12 +157,17 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
       __syncthreads();
   };
 
+  // The M/I/D form runs in batches only: its instances carry no checkpoint code.
+  // (With it, the descriptors' bookkeeping took the one-warp score-only ones to 127
+  // registers, four blocks per SM: 1000 reads of 4-8 kbp, score only, 11.9 ms; without it
+  // 96 registers, five blocks, 10.9 ms; with traceback 135 -> 100 registers.)
+  constexpr bool CKPT = VAR != 2;
   const uint32_t ck_i = blockIdx.x * (W == 1 ? 4 : 1) + grp;
   bool first_item = true;
   for (;;) {
     // ---- next pair --------------------------------------------------------------
     uint32_t t0 = 0;
-    if (a.ck) {  // checkpointed sweep of one pair: a descriptor per group
+    if (CKPT && a.ck) {  // checkpointed sweep of one pair: a descriptor per group
       t0 = (first_item && ck_i < a.n_ck) ? 0u : a.n_order;
       first_item = false;
     } else if (W == 1) {
@@ -183,7 +188,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32) k_xdrop(const FullArgs 
     if (a.sp.use_band) band_limits(M, N, a.sp.band, a.sp.band_literal, &blo, &bhi);
     const int band_lo = (int)max(blo, -(int64_t)M), band_hi = (int)min(bhi, (int64_t)N);
 
-    const XdCkpt *ck = a.ck ? a.ck + ck_i : nullptr;
+    const XdCkpt *ck = CKPT && a.ck ? a.ck + ck_i : nullptr;
     const int ckmode = ck ? ck->mode : 0;
     const int seg = ck ? ck->k_start / ck->C : 0;
     if (ckmode == 3) {

@@ -59,6 +59,11 @@ filtr_status filtr_test_set_search_keep(filtr_ctx *ctx, int64_t words);
  * strips and the workspace allows.  Results do not depend on it. */
 filtr_status filtr_test_set_split(filtr_ctx *ctx, int32_t mode);
 
+/* Rows per strip of the lowest strips that the last filtr_align_batch or
+ * filtr_align_long ran a warp each, or that the last filtr_graph_create captured so;
+ * 0: a warp per pair. */
+filtr_status filtr_test_last_strip_rows(filtr_ctx *ctx, int32_t *rows);
+
 /* Cell width of the antidiagonal (X-drop / Z-drop) sweep: 0 the default (two
  * cells per register for affine pairs whose threshold leaves room, int32
  * otherwise), 1 int32 always, 2 two cells per register with the base score

@@ -282,6 +282,7 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   }
   ctx->ev_used = 0;
   ctx->spans.clear();
+  ctx->last_strip_rows = 0;
   uint32_t launches = 0;
 
   // 1. workspace parts whose size depends on n only
@@ -712,6 +713,7 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     sl.R = g.R;
     sl.count = g.end - g.begin;
     const uint64_t rows = split_rows(sl.packed, g.R);
+    ctx->last_strip_rows = ctx->last_strip_rows ? std::min(ctx->last_strip_rows, (int)rows) : (int)rows;
     sl.max_strips = (uint32_t)((max_m + rows - 1) / rows);
     const int64_t items = sl.count * (int64_t)sl.max_strips;
     sl.grid = (int)std::min<int64_t>((int64_t)ctx->sms * ctx->split_blocks_per_sm(sl.packed, g.R, sp),

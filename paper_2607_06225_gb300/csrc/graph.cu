@@ -459,6 +459,11 @@ filtr_status filtr_graph_create(filtr_ctx *ctx, const filtr_params *params, uint
     }
   }
   const uint64_t tb_words = sp.traceback ? (workspace_bytes - fixed) / 4 : 0;
+  c->last_strip_rows = 0;
+  for (int i = 0; i < ss.n && ss.split != SPLIT_NONE; ++i) {
+    const int rows = split_rows(costs[ss.k[i]].packed, costs[ss.k[i]].R);
+    c->last_strip_rows = i ? std::min(c->last_strip_rows, rows) : rows;
+  }
 
   Graph *g = new Graph;
   g->ctx = c;

@@ -129,6 +129,7 @@ filtr_status run_long(Ctx *c, const ScoreParams &sp, const uint8_t *q, uint32_t 
   sl.count = 1;
   sl.max_strips = nstrips;
   sl.grid = grid;
+  c->last_strip_rows = HS;
   sl.a.f.b = b;
   sl.a.f.sp = sp;
   sl.a.f.order = d_one;
@@ -280,6 +281,7 @@ filtr_status run_xdrop_ckpt(Ctx *c, const ScoreParams &sp, const filtr_params *p
   if (e != cudaSuccess) return cuda_fail(e, "checkpointed forward sweep");
   const FwdOut f = *hf;
   c->last_launches = launches;
+  c->last_strip_rows = 0;
   if (hflags[0] == 3) {  // the packed sweep left its 16-bit range: the whole pair in int32
     ScoreParams s32 = sp;
     s32.xd16 = 0;
@@ -516,6 +518,15 @@ filtr_status filtr_test_set_split(filtr_ctx *ctx, int32_t mode) {
     return FILTR_ERR_INVALID;
   }
   reinterpret_cast<Ctx *>(ctx)->split_mode = mode;
+  return FILTR_OK;
+}
+
+filtr_status filtr_test_last_strip_rows(filtr_ctx *ctx, int32_t *rows) {
+  if (!ctx || !rows) {
+    set_error("filtr_test_last_strip_rows: NULL argument");
+    return FILTR_ERR_INVALID;
+  }
+  *rows = reinterpret_cast<Ctx *>(ctx)->last_strip_rows;
   return FILTR_OK;
 }
 

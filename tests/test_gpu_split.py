@@ -232,3 +232,36 @@ def test_tall_pair_without_room_for_strips(F, kind, tb):
         finally:
             c.close()
     same(out[0], out[1])
+
+
+def strip_rows(F, ctx):
+    import ctypes as C
+
+    rows = C.c_int32(-1)
+    assert F.lib().filtr_test_last_strip_rows(ctx.handle, C.byref(rows)) == F.OK
+    return rows.value
+
+
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("mode,gaps", [("global", dict(affine=True, gap_open=4, gap_extend=2)),
+                                       ("global", dict(affine=False, gap_extend=3)),
+                                       ("local", dict(affine=True, gap_open=11, gap_extend=1)),
+                                       ("local", dict(affine=False, gap_extend=5))])
+@pytest.mark.parametrize("band,literal", [(0, False), (3, False), (40, True), (300, False)])
+def test_long_pair_in_strips_of_128_rows(F, ctx, mode, gaps, band, literal, tb):
+    """Long banded pairs (over 512 rows and 2^22 cells of the full matrix) in the lowest
+    strips: heights at and around their edges, bands narrower and wider than a strip, a
+    band whose strips start past the first column or hold no cell."""
+    for m, n in [(2047, 2060), (2048, 2048), (2049, 2100), (2176, 2150), (2177, 2177), (4097, 1040), (1025, 4200)]:
+        b = pairs(4, 900 + m, [(m, n)])
+        q, r = b.pair(0)
+        sc = dict(mode=mode, traceback=tb, band=band, band_literal=literal, **gaps)
+        res, cig, rc = F.align_long(ctx, F.make_params(DNA_S, **sc), q, r)
+        assert rc == 0, F.last_error()
+        assert strip_rows(F, ctx) == 128
+        o = oracle.align(q, r, DNA_S, **sc)
+        fields = ("score", "q_end", "r_end", "status", "cells") + (("q_begin", "r_begin") if tb else ())
+        for f in fields:
+            assert int(res[f]) == int(o[f]), (m, n, f, int(res[f]), int(o[f]))
+        if tb:
+            assert np.array_equal(cig, o["cigar"]), (m, n)

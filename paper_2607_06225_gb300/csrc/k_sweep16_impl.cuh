@@ -474,7 +474,9 @@ struct Sweep16 {
       if (jA > jB) return X16_END;
       low = jA - cn;
       high = jB - cn;
-      if (low < 0 || high >= WIN) return X16_WIDE;
+      // (a range that would fit, were the window not held to diagonals and whole
+      // threads, goes to a wider group, and past the widest to the int32 sweep)
+      if (low < 0 || high >= WIN) return W == XD_MAX_WARPS && high - low < WIN ? X16_OVF : X16_WIDE;
       const int bp = (int)(b2 & 0xffffu), rp = xrun ? (int)(brun2 & 0xffffu) : bp;
       int tmin = rp - X;
       if (ZD) tmin -= max(abs(2 * jA - kk - dbest), abs(2 * jB - kk - dbest));

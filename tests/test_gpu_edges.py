@@ -160,3 +160,42 @@ def test_one_match_score_over_twenty_letters(F, ctx, W, drop, mode):
         compare(b, sc, res, cig, *oracle_batch(b, sc), label=f"W={W}")
     finally:
         F.lib().filtr_test_set_first_width(ctx.handle, 0)
+
+
+@pytest.mark.parametrize("mode", ["local", "global"])
+@pytest.mark.parametrize("long", [False, True])
+def test_regions_as_wide_as_the_widest_window(F, ctx, mode, long):
+    """Antidiagonals of up to 8192 live cells, the documented limit, where nothing is
+    pruned; 8193 are too many.  The longer side makes the range move off the window's
+    middle.  Batches and the checkpointed sweep, both cell widths."""
+    rng = np.random.default_rng(500)
+    qs, rs = [], []
+    for m, n in [(8140, 8500), (8170, 8600), (8900, 8180), (8187, 8400), (8300, 8191), (8191, 8191), (8192, 8192)]:
+        r = rng.integers(0, 4, n).astype(np.uint8)
+        q = np.where(rng.random(n) < 0.1, rng.integers(0, 4, n), r).astype(np.uint8)
+        qs.append(np.concatenate([q, rng.integers(0, 4, m).astype(np.uint8)])[:m])
+        rs.append(r)
+    # (a global corner-to-corner band of free gaps keeps all cells: no gap costs anything)
+    sc = dict(mode=mode, affine=True, gap_open=4 if mode == "local" else 0, gap_extend=2 if mode == "local" else 0,
+              xdrop=7999, traceback=True)
+    b = synth.pack(qs, rs, 4, synth.dna_subst(0 if mode == "global" else 1, -1))
+    params = F.make_params(b.subst, **sc)
+    out = []
+    for packed in (0, 1):
+        assert F.lib().filtr_test_set_packed_sweep(ctx.handle, packed) == F.OK
+        if long:
+            F.lib().filtr_test_set_checkpoint(ctx.handle, 4096)
+        try:
+            if long:
+                got = [F.align_long(ctx, params, q, r) for q, r in zip(qs, rs)]
+                res, cig = np.array([g[0] for g in got]), np.concatenate([g[1] for g in got])
+            else:
+                res, cig, rc = F.align_batch(ctx, params, b)
+                assert rc == 0, F.last_error()
+                cig = cig[:int(res["cigar_len"].sum())]
+        finally:
+            F.lib().filtr_test_set_packed_sweep(ctx.handle, 0)
+            F.lib().filtr_test_set_checkpoint(ctx.handle, 0)
+        assert list(res["status"]) == [0] * 6 + [4]
+        out.append((res[:-1].tobytes(), cig.tobytes()))
+    assert out[0] == out[1]

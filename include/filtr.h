@@ -173,7 +173,11 @@ filtr_status filtr_pack(const uint8_t *codes, uint64_t n, int32_t alphabet, uint
  * out in pair order; if the total exceeds cigar_cap the call returns
  * FILTR_ERR_CIGAR_CAP after the stream completes and each result carries its
  * length.  Band and X-drop pairs whose live region outgrows the widest kernel
- * window (8192 cells on one antidiagonal) get FILTR_ST_TOO_WIDE.  Returns FILTR_ERR_INVALID
+ * window (8192 cells on one antidiagonal) get FILTR_ST_TOO_WIDE.  Small batches and tall
+ * pairs run a warp per row strip, with bounded waits between strips; when one runs out
+ * (20 s without progress, as on a device that other work holds), the pairs of that
+ * launch get FILTR_ST_TIMEOUT and no result, and a call that waits for its CIGAR total
+ * (cigar_cap below the sum of all lengths) returns FILTR_ERR_TIMEOUT.  Returns FILTR_ERR_INVALID
  * before any launch for bad params or codes, FILTR_ERR_UNSUPPORTED when scores
  * could reach 2^28 in magnitude (largest |substitution score| x shorter side +
  * 3 x open + extend x (longest query + longest reference)) or, for local
@@ -427,7 +431,9 @@ filtr_status filtr_fold_batch(filtr_ctx *ctx, const filtr_fold_params *params, u
  *   was aligned), FILTR_ERR_CIGAR_CAP (results complete, CIGARs that do not
  *   fit cigar_cap not written), FILTR_ERR_UNSUPPORTED (the plan chose a tile
  *   shape that the graph, which launches only the shapes some pair within its
- *   bounds can take, does not hold: nothing was aligned; not expected).
+ *   bounds can take, does not hold: nothing was aligned; not expected),
+ *   FILTR_ERR_TIMEOUT (a bounded wait between a pair's strips ran out: the pairs of
+ *   that launch have FILTR_ST_TIMEOUT and no result).
  * filtr_graph_destroy: waits for the device, frees the graph; NULL is a no-op. */
 typedef struct filtr_graph filtr_graph;
 filtr_status filtr_graph_create(filtr_ctx *ctx, const filtr_params *params, uint32_t max_pairs,

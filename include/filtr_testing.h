@@ -59,6 +59,11 @@ filtr_status filtr_test_set_search_keep(filtr_ctx *ctx, int64_t words);
  * strips and the workspace allows.  Results do not depend on it. */
 filtr_status filtr_test_set_split(filtr_ctx *ctx, int32_t mode);
 
+/* Waits between a pair's strips in batches and in pipelines captured from now on: with
+ * withhold != 0 the first strip of every pair never publishes, so that the waits run
+ * out; after timeout_ns (0: the default) without progress. */
+filtr_status filtr_test_set_strip_wait(filtr_ctx *ctx, int32_t withhold, uint64_t timeout_ns);
+
 /* Rows per strip of the lowest strips that the last filtr_align_batch or
  * filtr_align_long ran a warp each, or that the last filtr_graph_create captured so;
  * 0: a warp per pair. */

@@ -180,6 +180,8 @@ def lib():
         L.filtr_test_set_device_plan.argtypes = [C.c_void_p, C.c_int32]
         L.filtr_test_set_split.restype = i32
         L.filtr_test_set_split.argtypes = [C.c_void_p, C.c_int32]
+        L.filtr_test_set_strip_wait.restype = i32
+        L.filtr_test_set_strip_wait.argtypes = [C.c_void_p, C.c_int32, C.c_uint64]
         L.filtr_test_last_strip_rows.restype = i32
         L.filtr_test_last_strip_rows.argtypes = [C.c_void_p, C.POINTER(C.c_int32)]
         L.filtr_test_set_search_ring.restype = i32

@@ -296,7 +296,9 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   FwdOut *d_fwd = c.take<FwdOut>(n);
   uint64_t *d_offs = c.take<uint64_t>(n);
   const size_t n_counters = (size_t)n + 4096;
-  uint32_t *d_counters = c.take<uint32_t>(n_counters);
+  uint32_t *d_counters = c.take<uint32_t>(n_counters);  // zeroed with the plan
+  // (a split batch takes no counters but, for a wait that ran out, the last)
+  int *d_timed_out = reinterpret_cast<int *>(d_counters + n_counters - 1);
   uint64_t *d_total = c.take<uint64_t>(4);
   uint32_t *d_ovf = c.take<uint32_t>(n);
   uint32_t *d_novf = c.take<uint32_t>(8);  // [0] window overflows, [4] packed-range overflows
@@ -720,7 +722,9 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
                                      (items + FULL_WARPS - 1) / FULL_WARPS);
     sl.a.f = fa;
     sl.a.f.order = d_order + g.begin;
-    sl.a.timeout_ns = SPLIT_TIMEOUT_NS;
+    sl.a.timed_out = d_timed_out;
+    sl.a.timeout_ns = ctx->strip_timeout_ns ? ctx->strip_timeout_ns : SPLIT_TIMEOUT_NS;
+    sl.a.withhold = ctx->strip_withhold;
     size_t at = 0;
     for (int x = 0; x < gi; ++x) at += split_spc[x].bytes;
     split_bind(&sl.a, d_split + at, split_spc[gi], split_stride);
@@ -894,8 +898,15 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     if (cap < P.cigar_upper) {
       uint64_t *h_total = reinterpret_cast<uint64_t *>(ctx->h_stage);
       ce = cudaMemcpyAsync(h_total, d_total, 8, cudaMemcpyDeviceToHost, st);
+      if (ce == cudaSuccess && split != SPLIT_NONE)
+        ce = cudaMemcpyAsync(h_total + 1, d_timed_out, 4, cudaMemcpyDeviceToHost, st);
       if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
       if (ce != cudaSuccess) return cuda_fail(ce, "reading the CIGAR total");
+      if (split != SPLIT_NONE && static_cast<uint32_t>(h_total[1]) != 0) {  // (4 bytes were copied)
+        set_error("a wait between a pair's strips ran out");
+        ctx->last_launches = launches;
+        return FILTR_ERR_TIMEOUT;
+      }
       if (*h_total > cap) {
         set_error("CIGARs need %llu ops, cigar_cap is %llu", (unsigned long long)*h_total,
                   (unsigned long long)cap);

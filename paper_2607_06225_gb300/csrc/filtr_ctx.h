@@ -37,6 +37,8 @@ struct Ctx {
   Plan plan;                       // the last call's plan; its buffers are reused
   int dev_plan_mode = 0;           // 0: device planner by batch size, 1: never, 2: always
   int split_mode = 0;              // a warp per strip: 0 by batch size, 1 never, 2 whenever possible
+  int strip_withhold = 0;          // test hook: strip 0 of every pair never publishes
+  uint64_t strip_timeout_ns = 0;   // test hook: limit of a wait between strips, 0 default
   int last_strip_rows = 0;         // lowest strips the last call or graph gave a warp each, 0 none
   int64_t search_keep = 0;         // search with traceback: most words a warp keeps (test hook), 0 default
   int search_ring = 0;             // search score pass: shared-memory ring entries, 0 default

@@ -202,6 +202,7 @@ struct GraphDesc {
   uint64_t cap;
   uint32_t n;
   int32_t abort;   // 0, or the filtr_status that stopped this launch
+  int32_t timed_out;  // a wait between a pair's strips ran out
 };
 struct DevPlanSummary;
 

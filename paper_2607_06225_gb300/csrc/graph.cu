@@ -26,10 +26,10 @@ namespace {
 
 __global__ void k_graph_desc(GraphDesc d, GraphDesc *dst) {
   d.abort = 0;
+  d.timed_out = 0;
   *dst = d;
 }
 
-// One thread: the checks filtr_align_batch makes on the host.
 // One thread: the checks filtr_align_batch makes on the host, and that every
 // pair's shape is one the graph launches (shapes_in: bit k for shape k).
 __global__ void k_graph_check(const DevPlanState *ps, GraphDesc *gd, uint32_t max_len,
@@ -61,6 +61,7 @@ __global__ void k_graph_setcond(const CondArgs c, const DevPlanSummary *sum, con
 __global__ void k_graph_finish(const GraphDesc *gd, const uint64_t *cigar_total, int traceback,
                                int32_t *status) {
   int32_t code = gd->abort;
+  if (code == 0 && gd->timed_out) code = FILTR_ERR_TIMEOUT;
   if (code == 0 && traceback && *cigar_total > gd->cap) code = FILTR_ERR_CIGAR_CAP;
   *status = code;
 }
@@ -323,7 +324,9 @@ cudaError_t capture(Graph *g, const ShapeCost *costs, const ShapeSet &ss, uint64
       sl.max_strips = ss.strips[i];
       sl.grid = ss.grid[i];
       sl.a.f = fa;
-      sl.a.timeout_ns = SPLIT_TIMEOUT_NS;
+      sl.a.timed_out = &g->d_gd->timed_out;
+      sl.a.timeout_ns = g->ctx->strip_timeout_ns ? g->ctx->strip_timeout_ns : SPLIT_TIMEOUT_NS;
+      sl.a.withhold = g->ctx->strip_withhold;
       split_bind(&sl.a, d_strip[i], ss.space[i], g->max_len + 1);
       e = launch_split(sl, st2);
     } else {

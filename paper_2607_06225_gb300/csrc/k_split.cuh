@@ -34,7 +34,7 @@
 // warps.
 //
 // Every wait is bounded by a time limit on %globaltimer; a wait that runs out sets
-// the error word, after which no wait waits, and the pairs report
+// the error word, after which no wait waits, and the launch's pairs report
 // FILTR_ST_TIMEOUT.
 #pragma once
 
@@ -81,6 +81,7 @@ struct SplitArgs {
   uint32_t ring_stride;
   int4 *res;                   // per item: best cell (v, i, j) and H at the corner
   int *err;
+  int *timed_out;              // set to 1 with the results when err was set (nullptr: nobody asks)
   unsigned long long timeout_ns;
   int withhold;                // test hook: strip 0 never publishes (forces the timeout)
 };

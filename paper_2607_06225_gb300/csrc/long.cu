@@ -521,6 +521,16 @@ filtr_status filtr_test_set_split(filtr_ctx *ctx, int32_t mode) {
   return FILTR_OK;
 }
 
+filtr_status filtr_test_set_strip_wait(filtr_ctx *ctx, int32_t withhold, uint64_t timeout_ns) {
+  if (!ctx) {
+    set_error("filtr_test_set_strip_wait: ctx is NULL");
+    return FILTR_ERR_INVALID;
+  }
+  reinterpret_cast<Ctx *>(ctx)->strip_withhold = withhold != 0;
+  reinterpret_cast<Ctx *>(ctx)->strip_timeout_ns = timeout_ns;
+  return FILTR_OK;
+}
+
 filtr_status filtr_test_last_strip_rows(filtr_ctx *ctx, int32_t *rows) {
   if (!ctx || !rows) {
     set_error("filtr_test_last_strip_rows: NULL argument");

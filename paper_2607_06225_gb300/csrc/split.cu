@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(128) k_split_finish(const SplitArgs a, int row
     filtr_result res{};
     res.cells = band_cells((uint32_t)M, (uint32_t)N, a.f.sp);
     if (*(volatile int *)a.err) {
+      if (a.timed_out) *a.timed_out = 1;
       res.status = FILTR_ST_TIMEOUT;
       res.cells = 0;
     } else if (a.f.sp.mode == FILTR_LOCAL) {

@@ -265,3 +265,49 @@ def test_long_pair_in_strips_of_128_rows(F, ctx, mode, gaps, band, literal, tb):
             assert int(res[f]) == int(o[f]), (m, n, f, int(res[f]), int(o[f]))
         if tb:
             assert np.array_equal(cig, o["cigar"]), (m, n)
+
+
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("kind", ["local", "int32", "band"])
+def test_waits_that_run_out(F, ctx, kind, tb):
+    """Batches and captured pipelines whose pairs' first strips publish nothing, with a
+    wait limit of 20 ms: every pair of the launch reports FILTR_ST_TIMEOUT, the calls
+    that wait for the device report it too, and the context works on."""
+    b = pairs(20, 15, [(600, 500), (200, 300), (1100, 900), (513, 64), (2000, 1500)])
+    sc = dict(dict(affine=True, gap_open=11, gap_extend=1, traceback=tb), **KINDS[kind])
+    params = F.make_params(b.subst, **sc)
+    want = run(F, ctx, b, sc, 1)
+
+    def timed_out(res):
+        assert (res["status"] == 5).all()
+        for f in ("score", "cells", "cigar_len"):
+            assert (res[f] == 0).all(), f
+
+    assert F.lib().filtr_test_set_strip_wait(ctx.handle, 1, 20_000_000) == F.OK
+    F.lib().filtr_test_set_split(ctx.handle, 2)
+    try:
+        res, _, rc = F.align_batch(ctx, params, b)
+        assert rc == F.OK
+        timed_out(res)
+        if tb:
+            res, _, rc = F.align_batch(ctx, params, b, cigar_cap=10, raise_on_error=False)
+            assert rc == F._lib.ERR_TIMEOUT
+            timed_out(res)
+        g = F.Graph(ctx, params, b.n, 2000, 1 << 30)
+        try:
+            res, _, status = F.graph_align(g, b)
+            assert status == F._lib.ERR_TIMEOUT
+            timed_out(res)
+        finally:
+            g.close()
+    finally:
+        F.lib().filtr_test_set_strip_wait(ctx.handle, 0, 0)
+    same(run(F, ctx, b, sc, 2), want)
+    g = F.Graph(ctx, params, b.n, 2000, 1 << 30)
+    try:
+        for _ in range(2):
+            res, cig, status = F.graph_align(g, b)
+            assert status == F.OK
+            same((res, cig[:int(res["cigar_len"].sum())] if tb else want[1]), want)
+    finally:
+        g.close()

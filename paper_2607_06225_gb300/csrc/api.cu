@@ -322,10 +322,10 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
     return FILTR_ERR_NOMEM;
   }
   const ShapeCost *costs = ctx->tuned_costs(sp);
-  // Few pairs: a warp per strip instead of per pair (k_split.cuh), unless a tune
-  // table says which warp-per-pair shapes to use
+  // Few pairs: a warp per strip instead of per pair (k_split.cuh)
   int split = SPLIT_NONE;
-  const bool may_split = !plain && !sp.use_xdrop && !costs && ctx->split_mode != 1 &&
+  const bool may_split = !plain && !sp.use_xdrop && ctx->split_mode != 1 &&
+                         (!costs || split_priced(costs, sp, SPLIT_PACK8)) &&
                          (ctx->split_mode == 2 || n <= (sp.use_band ? SPLIT_MAX_BANDED : SPLIT_MAX_PAIRS));
   if (may_split && (ctx->split_mode == 2 || n <= SPLIT_LATENCY_PAIRS))
     split = n <= SPLIT_LATENCY_PAIRS ? SPLIT_PACK8 : SPLIT_PACK8_16;

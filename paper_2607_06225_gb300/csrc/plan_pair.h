@@ -121,6 +121,26 @@ FILTR_HD bool split_shape_ok(int split, bool packed, int R) {
   return (R == 8 && split != SPLIT_PACK16) || (R == 16 && split != SPLIT_PACK8);
 }
 
+// Whether installed shape costs leave a warp per strip a choice.  A table of warp-per-pair
+// step times says nothing about which form is faster, so the size rules hold with one as
+// without, and its costs pick among the strip shapes.  But a caller who prices a strip
+// shape out (over four times the cheapest shape's price of a row; measured ones differ
+// by up to a half) has chosen other shapes.
+inline bool split_priced(const ShapeCost *costs, const ScoreParams &sp, int split) {
+  const bool pack_ok = !sp.use_band && sp.precision != FILTR_PREC_I32;
+  for (int packed = 0; packed <= (pack_ok ? 1 : 0); ++packed) {
+    double all = 1e300, strip = 1e300;
+    for (int k = 0; k < SHAPE_TILED; ++k) {
+      if ((costs[k].packed ? 1 : 0) != packed) continue;
+      const double row = costs[k].per_row + (double)costs[k].per_step / costs[k].R;
+      if (row < all) all = row;
+      if (row < strip && split_shape_ok(split, costs[k].packed, costs[k].R)) strip = row;
+    }
+    if (strip > 4.0 * all) return false;
+  }
+  return true;
+}
+
 inline ShapeTable make_shape_table(const ShapeCost *costs, const ScoreParams &sp, int split = SPLIT_NONE) {
   ShapeTable t{};
   const bool pack_ok = !sp.use_band && !sp.use_xdrop && sp.precision != FILTR_PREC_I32;

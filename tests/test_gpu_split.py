@@ -311,3 +311,35 @@ def test_waits_that_run_out(F, ctx, kind, tb):
             same((res, cig[:int(res["cigar_len"].sum())] if tb else want[1]), want)
     finally:
         g.close()
+
+
+def test_tuned_contexts_keep_strips(F):
+    """filtr_autotune, and its table applied elsewhere, leave the choice of a warp per
+    strip to the batch's size; a table that prices the strips' shapes out does not."""
+    b = pairs(20, 16, [(600, 500), (200, 300), (1100, 900), (513, 64), (2000, 1500)] * 6)
+    sc = dict(mode="local", affine=True, gap_open=11, gap_extend=1, traceback=True)
+    params = F.make_params(b.subst, **sc)
+    c1, c2, c3 = F.Context(0, 4 << 30), F.Context(0, 1 << 30), F.Context(0, 1 << 30)
+    try:
+        table = c1.autotune(params)
+        c2.tune_apply(params, table)
+        forced = {f"{kind} R={r}": 1000.0 for kind, r in F.TUNE_SHAPES}
+        forced["i16x2 R=24"] = 0.001
+        c3.tune_apply(params, forced)
+        want = None
+        for c, strips in ((c1, True), (c2, True), (c3, False)):
+            got = run(F, c, b, sc, 0)
+            assert (strip_rows(F, c) > 0) == strips
+            same(got, run(F, c, b, sc, 1))
+            F.lib().filtr_test_set_split(c.handle, 0)
+            g = F.Graph(c, params, b.n, 2000, 512 << 20)
+            assert (strip_rows(F, c) > 0) == strips
+            res, cig, status = F.graph_align(g, b)
+            assert status == F.OK
+            same((res, cig[:int(res["cigar_len"].sum())]), got)
+            g.close()
+            want = want or got
+            same(got, want)
+    finally:
+        for c in (c1, c2, c3):
+            c.close()

@@ -227,7 +227,9 @@ __global__ void __launch_bounds__(FOLD_THREADS) k_fold(const FoldArgs a) {
 // tables no longer fit shared memory beside the staging and live in the
 // sequence's area.
 // Measured against the plain kernel, whole calls: 1024 folds of 300 bases 8.92 ->
-// 1.35 ms, 1024 of 500 bases with X = 2 34.0 -> 4.6 ms.  What bounds it now: the
+// 1.35 ms, 1024 of 500 bases with X = 2 34.0 -> 4.6 ms, 512 of 640 bases 51.4 -> 6.9,
+// 300 of 800 75.4 -> 5.9, 160 of 1200 218 -> 14.5, 100 of 1500 395 -> 13.3, 500 of 40 to 1300
+// (every class, one launch after the other) 239 -> 18.8.  What bounds it now: the
 // bulk phase waits for its chunks and barriers (one block alone on an SM takes
 // 0.94 ms for 500 bases, three share it in 1.46 ms).
 constexpr int FOLD_PLAIN = 5;  // not a tiled class: the plain kernel

@@ -50,6 +50,7 @@ constexpr int FOLD_MC = 16;                      // staged split points per chun
 constexpr int FOLD_RS = FOLD_MC + 8;             // staged row stride (48 bytes: conflict free)
 constexpr int16_t FOLD_NEG = -16384;             // two of them still fit 16 bits
 constexpr uint32_t FOLD_NEG2 = 0xC000C000u;
+static_assert(FILTR_FOLD_MAX_LEN / 2 + 1 < -FOLD_NEG, "F <= n / 2: a sum with a missing cell stays negative");
 
 // halfwords of a row of Q
 FILTR_HD int fold_row_stride(int n) { return (n + 8) & ~7; }
@@ -249,8 +250,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_fold_tiled(const FoldTiledArg
       for (int i = 2 * tid; i <= n - L; i += 2 * NT) {
         uint32_t f2 = FOLD_NEG2;
         if (i + 1 >= dl && i <= dh) {
-          // (i, i+x) + (i+x, e) and (i, e-x) + (e-x, e), two x at a time; x = t + 1
-          // (odd t never reaches it, even t may) is a split of the bulk again
+          // (i, i+x) + (i+x, e) and (i, e-x) + (e-x, e), two x at a time; x = t + 1, reached
+          // when t is odd, is a split of the bulk again (W row 1, the span before the group)
           const uint32_t *wt = W32 + (1 + t) * W2 + (i >> 1);  // W of span t - 1 at i
           f2 = wt[W2];
           const uint32_t *wd = wt;                             // ... at i + x - 1

@@ -60,7 +60,7 @@
 //
 // Measured against the sweep with a sliding origin (one delta per antidiagonal,
 // four code paths, and every bound, range and code handled per antidiagonal: 362
-// warp instructions each): see the figures at x16_launch_any.
+// warp instructions each): see the figures at x16_launch.
 #include <algorithm>
 #include <climits>
 
@@ -1080,7 +1080,13 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
 // reductions every antidiagonal costs more: the megabase pair's forward took
 // 670 ms that way, 601 ms on one warp.)  The traceback rows and the checkpoint
 // records are those of 8-slot threads: thread t of the one-warp group writes
-// words 2t and 2t + 1.  W >= 4 runs W warps of 8-slot threads.
+// words 2t and 2t + 1.  W >= 4 runs W warps of 8-slot threads; those instances take
+// 168 to 193 registers (half the blocks per SM of the sweep with a sliding origin; at
+// W = 32, held to 64, they spill 284 to 516 bytes) and gain for their fewer instructions.
+// Whole calls, the sliding origin and this: W = 1, 10,000 long reads 244 -> 134 ms; W = 2,
+// 1,500 Z-drop reads 17.7 -> 10.9; W = 4, 1,000 reads of 4-8 kbp with X = 1500 26.1 -> 18.6;
+// W = 8, X = 3500 48.1 -> 35.8; W = 16, 400 reads, X = 7000 44.6 -> 29.3; W = 32, 200 protein
+// pairs of 6-9 thousand, X = 7500 70.7 -> 41.4.
 template <int KW, int G, bool LOCAL, bool TB, bool ZD>
 cudaError_t x16_launch(const FullArgs &a, int grid, uint32_t *ovf, uint32_t *novf, X16Knobs kn,
                        cudaStream_t s) {

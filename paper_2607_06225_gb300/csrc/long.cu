@@ -34,7 +34,6 @@ struct Carve {
   }
 };
 
-
 filtr_status validate_seq(Ctx *c, const uint8_t *q, uint32_t M, const uint8_t *r, uint32_t N,
                           int alphabet, cudaStream_t st) {
   uint32_t *d_bad = reinterpret_cast<uint32_t *>(c->d_small);

@@ -934,72 +934,72 @@ static filtr_status search_impl(Ctx *ctx, const filtr_search_params *prm, uint32
     filtr_status rc = place();
     if (rc != FILTR_OK) return rc;
     if (h_left > 0) {
-    // wavefront storage of the pairs left over, cut into waves that fit the workspace
-    uint64_t *h_need = reinterpret_cast<uint64_t *>(ctx->h_stage);
-    ce = cudaMemcpyAsync(h_need, d_need, (size_t)n * 8, cudaMemcpyDeviceToHost, st);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "reading the wavefront sizes");
-    std::vector<uint64_t> need(h_need, h_need + n);
-    c.used = ring_mark;  // the ring is free again: the arena takes the rest
-    const size_t arena_base = (c.used + 255) / 256 * 256;
-    const uint64_t arena_words =
-        ctx->ws_bytes > arena_base ? (ctx->ws_bytes - arena_base) / sizeof(int) : 0;
-    int *d_arena = reinterpret_cast<int *>(ctx->ws + arena_base);
-    if (!ctx->ensure_host((size_t)n * 8 * 2 + (size_t)n * 4 + 256)) {
-      set_error("pinned host allocation failed");
-      return FILTR_ERR_NOMEM;
-    }
-    uint64_t *h_aoff = reinterpret_cast<uint64_t *>(ctx->h_stage);
-    uint32_t *h_ord = reinterpret_cast<uint32_t *>(h_aoff + n);
-    std::vector<std::pair<uint32_t, uint32_t>> wave_ranges;
-    uint64_t used = 0;
-    uint32_t begin = 0, at = 0;
-    for (uint32_t p = 0; p < n; ++p) {
-      h_aoff[p] = 0;
-      if (need[p] == 0) continue;
-      const uint64_t w = (need[p] + 3) / 4 * 4;  // keep each pair's store 16-byte aligned
-      if (w > arena_words) {
-        set_error("pair %u keeps %llu wavefront words; the workspace holds %llu", p,
-                  (unsigned long long)w, (unsigned long long)arena_words);
+      // wavefront storage of the pairs left over, cut into waves that fit the workspace
+      uint64_t *h_need = reinterpret_cast<uint64_t *>(ctx->h_stage);
+      ce = cudaMemcpyAsync(h_need, d_need, (size_t)n * 8, cudaMemcpyDeviceToHost, st);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+      if (ce != cudaSuccess) return cuda_fail(ce, "reading the wavefront sizes");
+      std::vector<uint64_t> need(h_need, h_need + n);
+      c.used = ring_mark;  // the ring is free again: the arena takes the rest
+      const size_t arena_base = (c.used + 255) / 256 * 256;
+      const uint64_t arena_words =
+          ctx->ws_bytes > arena_base ? (ctx->ws_bytes - arena_base) / sizeof(int) : 0;
+      int *d_arena = reinterpret_cast<int *>(ctx->ws + arena_base);
+      if (!ctx->ensure_host((size_t)n * 8 * 2 + (size_t)n * 4 + 256)) {
+        set_error("pinned host allocation failed");
         return FILTR_ERR_NOMEM;
       }
-      if (used + w > arena_words) {
-        wave_ranges.push_back({begin, at});
-        begin = at;
-        used = 0;
+      uint64_t *h_aoff = reinterpret_cast<uint64_t *>(ctx->h_stage);
+      uint32_t *h_ord = reinterpret_cast<uint32_t *>(h_aoff + n);
+      std::vector<std::pair<uint32_t, uint32_t>> wave_ranges;
+      uint64_t used = 0;
+      uint32_t begin = 0, at = 0;
+      for (uint32_t p = 0; p < n; ++p) {
+        h_aoff[p] = 0;
+        if (need[p] == 0) continue;
+        const uint64_t w = (need[p] + 3) / 4 * 4;  // keep each pair's store 16-byte aligned
+        if (w > arena_words) {
+          set_error("pair %u keeps %llu wavefront words; the workspace holds %llu", p,
+                    (unsigned long long)w, (unsigned long long)arena_words);
+          return FILTR_ERR_NOMEM;
+        }
+        if (used + w > arena_words) {
+          wave_ranges.push_back({begin, at});
+          begin = at;
+          used = 0;
+        }
+        h_aoff[p] = used;
+        used += w;
+        h_ord[at++] = p;
       }
-      h_aoff[p] = used;
-      used += w;
-      h_ord[at++] = p;
-    }
-    wave_ranges.push_back({begin, at});
-    if (wave_ranges.size() > 60) {
-      set_error("the traceback would take %zu waves", wave_ranges.size());
-      return FILTR_ERR_NOMEM;
-    }
-    ce = cudaMemcpyAsync(d_arena_off, h_aoff, (size_t)n * 8, cudaMemcpyHostToDevice, st);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(d_order, h_ord, (size_t)at * 4, cudaMemcpyHostToDevice, st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "uploading the traceback layout");
-    a.need = nullptr;
-    a.ring = nullptr;
-    a.arena = d_arena;
-    a.arena_off = d_arena_off;
-    ctx->span_begin(Ctx::PH_WALK, st);
-    for (size_t w = 0; w < wave_ranges.size(); ++w) {
-      a.order = d_order + wave_ranges[w].first;
-      a.n = wave_ranges[w].second - wave_ranges[w].first;
-      a.counter = d_counter + 1 + w;
-      ce = launch_cfg(k_tb, cfg_tb, a, ctx->sms, UINT64_MAX, st);
-      ++launches;
-      if (ce != cudaSuccess) break;
-    }
-    ctx->span_end(st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "search traceback pass");
-    ctx->last_waves = (int)wave_ranges.size();
+      wave_ranges.push_back({begin, at});
+      if (wave_ranges.size() > 60) {
+        set_error("the traceback would take %zu waves", wave_ranges.size());
+        return FILTR_ERR_NOMEM;
+      }
+      ce = cudaMemcpyAsync(d_arena_off, h_aoff, (size_t)n * 8, cudaMemcpyHostToDevice, st);
+      if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(d_order, h_ord, (size_t)at * 4, cudaMemcpyHostToDevice, st);
+      if (ce != cudaSuccess) return cuda_fail(ce, "uploading the traceback layout");
+      a.need = nullptr;
+      a.ring = nullptr;
+      a.arena = d_arena;
+      a.arena_off = d_arena_off;
+      ctx->span_begin(Ctx::PH_WALK, st);
+      for (size_t w = 0; w < wave_ranges.size(); ++w) {
+        a.order = d_order + wave_ranges[w].first;
+        a.n = wave_ranges[w].second - wave_ranges[w].first;
+        a.counter = d_counter + 1 + w;
+        ce = launch_cfg(k_tb, cfg_tb, a, ctx->sms, UINT64_MAX, st);
+        ++launches;
+        if (ce != cudaSuccess) break;
+      }
+      ctx->span_end(st);
+      if (ce != cudaSuccess) return cuda_fail(ce, "search traceback pass");
+      ctx->last_waves = (int)wave_ranges.size();
 
-    rc = place();
-    if (rc != FILTR_OK) return rc;
+      rc = place();
+      if (rc != FILTR_OK) return rc;
     }
     if (h_total > cap) {
       set_error("CIGARs need %llu ops, cigar_cap is %llu", (unsigned long long)h_total,

@@ -868,12 +868,18 @@ filtr_status align_batch_impl(Ctx *ctx, const filtr_params *params, uint32_t n,
   };
   if (!ladder(P.xdrop_w0)) return cuda_fail(ce, "rerun");
   if (!pending16.empty()) {  // pairs that left the packed range: the int32 sweep
-    std::vector<uint32_t> todo;
-    todo.swap(pending16);
-    n_xd16_rerun = (uint32_t)todo.size();
+    std::vector<uint32_t> left;
+    left.swap(pending16);
+    pending.clear();  // (what outgrew the widest group keeps its status)
+    n_xd16_rerun = (uint32_t)left.size();
     fa.sp.xd16 = 0;
-    const int w0 = std::max(1, (int)P.xdrop_w0);
-    if (!rerun(todo, w0) || !ladder(w0)) return cuda_fail(ce, "int32 rerun");
+    for (int W : {1, 2, 4, 8, 16, 32}) {  // each pair from the width that it had come to
+      std::vector<uint32_t> todo;
+      todo.swap(pending);
+      for (uint32_t p : left)
+        if (P.tbl[p].warps == W) todo.push_back(p);
+      if (!todo.empty() && !rerun(todo, W)) return cuda_fail(ce, "int32 rerun");
+    }
   }
   if (n_trivial) {
     ce = launch_trivial(b, sp, d_order + n_main, n_trivial, out, d_fwd, st);

@@ -156,6 +156,8 @@ struct Sweep16 {
   static constexpr int S = 8 * G, P = 4 * G, WIN = W * 32 * S, ROW = WIN / 8;
   // a fast step needs k and c itself (else a fast block counts them as a whole)
   static constexpr bool STEP_K = LOCAL || ZD || W > 1 || !UNI;
+  // the widest group's window moves by single slots: no wider one takes its pairs over
+  static constexpr bool ANY_SLOT = W == XD_MAX_WARPS;
   // parameters of the pair and the thread
   X16Shared<W> &sh;
   const int8_t *s_sub;
@@ -474,9 +476,14 @@ struct Sweep16 {
       if (jA > jB) return X16_END;
       low = jA - cn;
       high = jB - cn;
-      // (a range that would fit, were the window not held to diagonals and whole
-      // threads, goes to a wider group, and past the widest to the int32 sweep)
-      if (low < 0 || high >= WIN) return W == XD_MAX_WARPS && high - low < WIN ? X16_OVF : X16_WIDE;
+      // (A window moved by whole threads may be left by a range some 20 cells narrower,
+      // the widest group's, held to diagonals, by one of two cells less.  Such a pair none
+      // of whose antidiagonals has more cells than the window goes on in the int32 sweep,
+      // whose window follows the range; others would outgrow that one too)
+      if (low < 0 || high >= WIN) {
+        const int most = min(min(M, N) + 1, (band_hi - band_lo) / 2 + 1);
+        return W == XD_MAX_WARPS && most <= WIN ? X16_OVF : X16_WIDE;
+      }
       const int bp = (int)(b2 & 0xffffu), rp = xrun ? (int)(brun2 & 0xffffu) : bp;
       int tmin = rp - X;
       if (ZD) tmin -= max(abs(2 * jA - kk - dbest), abs(2 * jB - kk - dbest));
@@ -570,10 +577,27 @@ struct Sweep16 {
     }
   }
 
-  // the window moves up by t threads: thread x takes the state of thread x + t
-  __device__ __forceinline__ void move_array(uint32_t (&v)[P], int t) {
+  // the window moves up by s slots, whole threads but in the widest group: thread x
+  // takes the state of thread x + s / S
+  __device__ __forceinline__ void move_array(uint32_t (&v)[P], int s) {
+    const int t = s / S;
     const bool in = tid + t >= 0 && tid + t < W * 32;
-    if constexpr (W == 1) {
+    if constexpr (ANY_SLOT) {
+      __syncthreads();
+      sh.move[tid] = make_uint4(v[0], v[1], v[2], v[3]);
+      __syncthreads();
+      const uint16_t *half = reinterpret_cast<const uint16_t *>(sh.move);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        uint32_t x = 0;
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const int q = base_slot + r + 4 * hh + s;
+          if (q >= 0 && q < WIN) x |= (uint32_t)half[(q & ~7) + 2 * (q & 3) + (q >> 2 & 1)] << (16 * hh);
+        }
+        v[r] = x;
+      }
+    } else if constexpr (W == 1) {
 #pragma unroll
       for (int r = 0; r < P; ++r) {
         const uint32_t x = __shfl_sync(X16_FULL, v[r], (lane + t) & 31);
@@ -590,19 +614,19 @@ struct Sweep16 {
       v[3] = x.w;
     }
   }
-  __device__ __forceinline__ void move_window(int t) {
-    move_array(Ha, t);
-    move_array(Hb, t);
-    move_array(En, t);
-    move_array(Fn, t);
-    move_array(Ho, t);
-    c += t * S;
-    pl -= t * S;
-    ph -= t * S;
-    if (pbs >= 0) pbs -= t * S;
+  __device__ __forceinline__ void move_window(int s) {
+    move_array(Ha, s);
+    move_array(Hb, s);
+    move_array(En, s);
+    move_array(Fn, s);
+    move_array(Ho, s);
+    c += s;
+    pl -= s;
+    ph -= s;
+    if (pbs >= 0) pbs -= s;
     if (ol <= oh) {
-      ol -= t * S;
-      oh -= t * S;
+      ol -= s;
+      oh -= s;
     }
     if constexpr (W > 1) {
       // the next step reads its neighbours' edges and the warps' reductions (the
@@ -820,21 +844,34 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
         }
       }
       if (LOCAL) w.Z2 = x16_splat(min(max(X16_C0 - w.base, 0), 0x7fff));
+      const bool phase_b = resumed && first_b;
       // room on each side (a block moves an end by 8 slots), and the new codes
       // (in one-warp groups the first and last thread stay dead besides: a fast
       // step does not clear the edge values that wrap around to them)
       constexpr int ROOM = X16_BLOCK / 2 + 1 + (W == 1 ? S : 1);
+      int block = X16_BLOCK;
       if (w.pl < ROOM || w.ph > WIN - 1 - ROOM) {
         const int mid = (w.pl + w.ph) >> 1;
-        const int t = (mid - WIN / 2) / S;
-        if (t != 0) {
-          w.move_window(t);
+        int s = SW::ANY_SLOT ? mid - WIN / 2 : (mid - WIN / 2) / S * S;
+        if (SW::ANY_SLOT && w.ph - w.pl >= WIN - 2 * ROOM) {
+          // less room than a block takes: two antidiagonals at a time (columns [a1, b1] and
+          // up to b2 at most), in a window that holds them and the live range, if one does
+          block = 2;
+          const int l = w.c + w.pl, h = w.c + w.ph, k1 = w.k + 1, k2 = k1 + 1, d = phase_b ? 0 : 1;
+          const int a1 = max(max(max(0, k1 - M), (k1 + w.band_lo + 1) >> 1), l);
+          const int b1 = min(min(min(N, k1), (k1 + w.band_hi) >> 1), h + 1);
+          const int b2 = phase_b ? b1 : min(min(min(N, k2), (k2 + w.band_hi) >> 1), b1 + 1);
+          const int most = min(l, a1 - d);  // the origin
+          const int least = max(h + 1, b2 + 1 - d) - WIN;
+          s = max(min(w.c, most), min(least, most)) - w.c;
+        }
+        if (s != 0) {
+          w.move_window(s);
           w.load_codes(w.k, w.c);
           ahead = false;
         }
       }
       const int kb = w.k + 1;
-      const bool phase_b = resumed && first_b;
       if (UNI) {
         if (ahead) {
           w.qn = qx;
@@ -843,7 +880,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
           w.load_next(w.qn, w.rn, 0);
           if (phase_b) w.rn = 0;  // a lone phase B step takes a query code only
         }
-        ahead = !phase_b;
+        ahead = !phase_b && block == X16_BLOCK;
         if (ahead) w.load_next(qx, rx, X16_BLOCK / 2);
       } else if (phase_b) {
         const int i = kb - w.c - base_slot;
@@ -855,7 +892,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
       }
       if (TB) {  // the block's window origins
         const int x = phase_b ? 0 : lane;
-        if (w.warp == 0 && lane < (phase_b ? 1 : X16_BLOCK) && kb + x <= k_last)
+        if (w.warp == 0 && lane < (phase_b ? 1 : block) && kb + x <= k_last)
           ckp[kb - row0 + x] = phase_b ? w.c : w.c + 1 + (x >> 1);
       }
       const int bp = (int)(w.b2 & 0xffffu), rp = w.xrun ? max((int)(w.brun2 & 0xffffu), bp) : bp;
@@ -886,7 +923,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W == 1 ? (G == 2 ? 3 : 
         }
       } else {
         int x = phase_b ? 1 : 0;
-        const int xe = phase_b ? 2 : X16_BLOCK;
+        const int xe = phase_b ? 2 : block;
 #pragma unroll 1
         for (; x < xe && w.k < k_last; ++x) {
           if (resumed) w.track = false;

@@ -193,6 +193,8 @@ def test_regions_as_wide_as_the_widest_window(F, ctx, mode, long):
                 res, cig, rc = F.align_batch(ctx, params, b)
                 assert rc == 0, F.last_error()
                 cig = cig[:int(res["cigar_len"].sum())]
+                # (ranges of 8191 and 8192 cells that move may need the int32 sweep's window)
+                assert ctx.last_stats()["pairs_xd16_rerun"] <= 2
         finally:
             F.lib().filtr_test_set_packed_sweep(ctx.handle, 0)
             F.lib().filtr_test_set_checkpoint(ctx.handle, 0)

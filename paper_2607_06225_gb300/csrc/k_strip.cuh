@@ -131,6 +131,7 @@ struct LaneBest {
 //   FETCH                     -- constexpr bool: lane 0's input row is
 //                                fetched ahead with fetch() instead of in()
 //   int2 in(int j)            -- (not FETCH) lane 0 only: (H, F) of the strip above
+//   bool wait(int j)          -- (not FETCH) before in(j); false ends the pass
 //   int fetch(int j, int jmax, int2 &v) -- (FETCH) lane x loads (H, F) of column
 //                                j + x of the strip above for the n columns
 //                                (1 <= n <= 32, up to jmax) known to be ready,
@@ -138,9 +139,9 @@ struct LaneBest {
 //   void out(int j, int H, int F) -- lane 31 only: this strip's bottom row
 // prev_jlo / prev_jhi: the strip above's columns (empty for s == 0).
 // endH receives H(M, jhi) for the lane holding row M when this is the last
-// strip.
+// strip.  False if wait() ended the pass.
 template <int R, bool LOCAL, bool AFFINE, bool TB, bool BAND, class IO>
-__device__ __forceinline__ void strip_pass(const StripPair &P, int s, int jlo, int jhi, int prev_jlo,
+__device__ __forceinline__ bool strip_pass(const StripPair &P, int s, int jlo, int jhi, int prev_jlo,
                                            int prev_jhi, int64_t tb_base, IO &io, LaneBest &best,
                                            int &endH) {
   constexpr int HS = 32 * R;
@@ -240,6 +241,12 @@ __device__ __forceinline__ void strip_pass(const StripPair &P, int s, int jlo, i
         vin.x = __shfl_sync(STRIP_FULLMASK, pv.x, j0 - pbase);
         vin.y = AFFINE ? __shfl_sync(STRIP_FULLMASK, pv.y, j0 - pbase) : NEG;
       }
+    } else if constexpr (!TB) {
+      // A per-warp buffer never ends the pass, but with this exit the compiler lays the
+      // step out better: local scores of 300 pairs of 128 31.4 us, 35.5 without; of 8000
+      // protein pairs 1.44 and 1.48 ms.  (With traceback it is the other way round: 20,000
+      // local pairs of 100-300 1.85 and 1.78 ms.)
+      if (need && !io.wait(j0)) return false;
     }
     int inH = __shfl_up_sync(STRIP_FULLMASK, upH, 1);
     int inF = AFFINE ? __shfl_up_sync(STRIP_FULLMASK, upF, 1) : NEG;
@@ -336,6 +343,7 @@ __device__ __forceinline__ void strip_pass(const StripPair &P, int s, int jlo, i
       if (top + k == M) endH = Hc[k];
   }
   __syncwarp();
+  return true;
 }
 
 // warp-wide reduction of LaneBest with the tie-break (all lanes get the result)

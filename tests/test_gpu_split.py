@@ -332,7 +332,8 @@ def test_tuned_contexts_keep_strips(F):
             assert (strip_rows(F, c) > 0) == strips
             same(got, run(F, c, b, sc, 1))
             F.lib().filtr_test_set_split(c.handle, 0)
-            g = F.Graph(c, params, b.n, 2000, 512 << 20)
+            # (every shape that a table may choose has strip buffers of up to 80 MB)
+            g = F.Graph(c, params, b.n, 2000, 4 << 30)
             assert (strip_rows(F, c) > 0) == strips
             res, cig, status = F.graph_align(g, b)
             assert status == F.OK

@@ -447,7 +447,7 @@ filtr_status filtr_graph_create(filtr_ctx *ctx, const filtr_params *params, uint
   // what those need (the check node compares ref_words).
   const uint64_t ref_words = sp.traceback ? (workspace_bytes - fixed) / 4 : 0;
   if (max_len > 256 && split_priced(costs, sp, SPLIT_PACK8) && c->split_mode != 1 &&
-      (c->split_mode == 2 || split_graph(sp.use_band != 0, max_pairs, max_len))) {
+      (c->split_mode == 2 || split_graph(sp.use_band != 0, sp.traceback != 0, max_pairs, max_len))) {
     const int order[2] = {max_pairs <= SPLIT_LATENCY_PAIRS ? SPLIT_PACK8 : SPLIT_PACK8_16, SPLIT_PACK16};
     for (int mode : order) {
       const ShapeSet s = graph_shapes(c, sp, costs, max_len, max_pairs, mode);

@@ -66,8 +66,10 @@ constexpr uint32_t SPLIT_BAND_ROWS = 1408;
 // split, local pairs with traceback: 64 of up to 700 0.39 / 0.36 ms, of up to 2000
 // 1.59 / 0.96; 256 of up to 1000 0.62 / 0.82, of up to 2000 2.03 / 1.57; banded (256):
 // 16 of up to 300 0.26 / 0.25, 256 of up to 600 0.55 / 0.64, of up to 1500 2.09 / 1.67.
-inline bool split_graph(bool band, uint32_t max_pairs, uint32_t max_len) {
-  if (max_pairs <= 64) return band || max_len > 1024;
+// Scores only: 40 local pairs of up to 1100 0.260 / 0.271, of up to 1220 0.311 / 0.302, of
+// up to 1500 0.60 / 0.37; 64 banded (60) of up to 380 0.138 / 0.149, of up to 620 0.201 / 0.187.
+inline bool split_graph(bool band, bool traceback, uint32_t max_pairs, uint32_t max_len) {
+  if (max_pairs <= 64) return band ? traceback || max_len > 512 : max_len > (traceback ? 1024u : 1152u);
   return band ? max_pairs <= SPLIT_MAX_PAIRS && max_len > 1024
               : max_pairs <= SPLIT_LATENCY_PAIRS && max_len > 1408;
 }

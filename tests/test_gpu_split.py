@@ -344,3 +344,17 @@ def test_tuned_contexts_keep_strips(F):
     finally:
         for c in (c1, c2, c3):
             c.close()
+
+
+@pytest.mark.parametrize("kind,tb,n,length,strips", [
+    ("local", True, 40, 1024, False), ("local", True, 40, 1025, True), ("local", False, 40, 1152, False),
+    ("local", False, 40, 1153, True), ("band", True, 64, 300, True), ("band", False, 64, 512, False),
+    ("band", False, 64, 513, True), ("local", False, 65, 1408, False), ("local", False, 255, 1409, True)])
+def test_which_pipelines_take_strips(F, ctx, kind, tb, n, length, strips):
+    F.lib().filtr_test_set_split(ctx.handle, 0)
+    sc = dict(dict(affine=True, gap_open=11, gap_extend=1, traceback=tb), **KINDS[kind])
+    g = F.Graph(ctx, F.make_params(PROT_S, **sc), n, length, 3 << 30)
+    try:
+        assert (strip_rows(F, ctx) > 0) == strips
+    finally:
+        g.close()
